@@ -1,0 +1,340 @@
+// Binary64 exponential, logarithm, quotient, reciprocal and roots on 64-bit integers.
+//
+// GB300 has one binary64 unit per SM: a warp-wide DFMA, DADD or DMUL holds it for 19 cycles
+// (measured; 64 cycles from issue to result), while a 64 x 64 -> high 64 bit integer product
+// takes 4 to 5 cycles of the SM's integer pipes, a 64-bit sum under 1 and a 32-bit product 0.5 to
+// 1. The functions below therefore run entirely on integers, with 58 to 62 significant bits
+// where binary64 carries 53, and round once when they return a binary64 value: they are cheaper
+// and closer to the exact result than any binary64 sequence. The binary64 unit then runs the
+// sums and products around them, at the same time.
+//
+// Everything here is plain integer arithmetic, the same on the host as on the device (the
+// starting values of the reciprocal and root differ: the device takes the hardware's
+// approximations, the host rounds exact ones to the same 23 bits).
+#pragma once
+
+#include <stdint.h>
+#include <string.h>
+#ifndef __CUDA_ARCH__
+#include <math.h>
+#endif
+
+#include "fix_table.h"
+
+#ifdef __CUDACC__
+#define FX __host__ __device__ __forceinline__
+#else
+#define FX static inline
+#endif
+
+namespace hyp {
+
+typedef unsigned long long u64;
+typedef long long i64;
+typedef uint32_t u32;
+
+#ifdef __CUDACC__
+__device__ const u64 FIX_EXP_DEV[256] = {FIX_EXP_BODY};
+__device__ const u64 FIX_LOG_DEV[128][2] = {FIX_LOG_BODY};
+#endif
+static const u64 FIX_EXP_HOST[256] = {FIX_EXP_BODY};
+static const u64 FIX_LOG_HOST[128][2] = {FIX_LOG_BODY};
+
+FX u64 fix_exp_entry(int j) {
+#ifdef __CUDA_ARCH__
+    return FIX_EXP_DEV[j];
+#else
+    return FIX_EXP_HOST[j];
+#endif
+}
+
+FX const u64* fix_log_row(int j) {
+#ifdef __CUDA_ARCH__
+    return FIX_LOG_DEV[j];
+#else
+    return FIX_LOG_HOST[j];
+#endif
+}
+
+FX u64 bits_of(double x) {
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(x);
+#else
+    u64 u;
+    memcpy(&u, &x, 8);
+    return u;
+#endif
+}
+
+FX double double_of(u64 u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((i64)u);
+#else
+    double x;
+    memcpy(&x, &u, 8);
+    return x;
+#endif
+}
+
+FX int clz64(u64 x) {       // x != 0
+#ifdef __CUDA_ARCH__
+    return __clzll((i64)x);
+#else
+    return __builtin_clzll(x);
+#endif
+}
+
+FX u32 mulhi32(u32 a, u32 b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (u32)(((u64)a * b) >> 32);
+#endif
+}
+
+FX int mulhi32s(int a, int b) {
+#ifdef __CUDA_ARCH__
+    return __mulhi(a, b);
+#else
+    return (int)(((i64)a * b) >> 32);
+#endif
+}
+
+// The high 64 bits of a b, at most two units low: the carry out of the low words is not formed
+// (three 32-bit products instead of four and their carries).
+FX u64 mulhi64(u64 a, u64 b) {
+    const u32 ah = (u32)(a >> 32), al = (u32)a, bh = (u32)(b >> 32), bl = (u32)b;
+    return (u64)ah * bh + mulhi32(ah, bl) + mulhi32(al, bh);
+}
+
+// The high 64 bits of a signed by an unsigned factor (a few units off).
+FX i64 mulhi64su(i64 a, u64 b) {
+    const u64 p = mulhi64((u64)a, b);
+    return (i64)(a < 0 ? p - b : p);
+}
+
+// A positive number (m / 2^63) 2^e, m in [2^63, 2^64), or zero (m = 0).
+struct xf {
+    u64 m;
+    int e;
+};
+
+FX xf xf_mul(xf a, xf b) {
+    const u64 p = mulhi64(a.m, b.m);            // [2^62, 2^64)
+    const int up = (int)(p >> 63);
+    return xf{up ? p : p + p, a.e + b.e + up};
+}
+
+// The xf of a positive normal binary64 value.
+FX xf xf_of(double x) {
+    const u64 u = bits_of(x);
+    return xf{(u << 11) | 0x8000000000000000ull, (int)((u >> 52) & 0x7ff) - 1023};
+}
+
+// v 2^-q (v any 64-bit value) normalised.
+FX xf xf_fixed(u64 v, int q) {
+    if (v == 0) return xf{0, 0};
+    const int z = clz64(v);
+    return xf{v << z, 63 - z - q};
+}
+
+// The binary64 nearest to x, for exponents inside binary64's normal range.
+FX double f64_of_xf(xf x) {
+    if (x.m == 0) return 0.0;
+    const u64 v = (x.m >> 11) + ((x.m >> 10) & 1);      // leading one at bit 52, or 2^53 if carried
+    return double_of(v + ((u64)(u32)(x.e + 1022) << 52));
+}
+
+// The same for any exponent: zero below the normal range, infinity above it.
+FX double f64_of_xf_any(xf x) {
+    if (x.m == 0 || x.e < -1022) return 0.0;
+    if (x.e > 1022) return double_of(0x7ff0000000000000ull);
+    return f64_of_xf(x);
+}
+
+FX double f64_of_fixed(u64 v, int q) { return f64_of_xf(xf_fixed(v, q)); }
+
+FX float rcp_start(float x) {      // 1 / x within 2^-22, x in [1, 2)
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+FX float rsqrt_start(float x) {    // 1 / sqrt(x) within 2^-22, x in [1, 4)
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / sqrtf(x);
+#endif
+}
+
+FX float float_of_bits(u32 u) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(u);
+#else
+    float x;
+    memcpy(&x, &u, 4);
+    return x;
+#endif
+}
+
+FX u32 bits_of_float(float x) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    u32 u;
+    memcpy(&u, &x, 4);
+    return u;
+#endif
+}
+
+// 2^127 / m for m in [2^63, 2^64): the reciprocal of a mantissa as a mantissa of the same form
+// (2 ulp of 2^-62; just below 2^64 for m = 2^63). A start y of 23 bits and one third-order step
+// y (1 + d + d^2) with the residual d = 1 - m y exact to 2^-63: the error d^3 is below 2^-62.
+FX u64 rcp64(u64 m) {
+    const float f = float_of_bits(0x3f800000u | (u32)((m >> 40) & 0x7fffffu));    // [1, 2)
+    // the start in (1/2, 1], lowered by 2^-22 so that it stays below 1, as y 2^-32
+    const float y0 = rcp_start(f);
+    const u32 b = bits_of_float(y0);                     // exponent 126 (or 127 for y0 = 1)
+    const u32 y = b >= 0x3f800000u ? 0xfffffc00u : (((b & 0x7fffffu) | 0x800000u) << 8) - 0x400u;
+    // m y with m = f 2^63: f y = 1 - d, in units of 2^-63
+    const u64 p = (u64)(u32)(m >> 32) * y + mulhi32((u32)m, y);
+    // (p is up to one low; one less keeps the result below 2^64 at m = 2^63)
+    const i64 d = (i64)(0x7fffffffffffffffull - p);      // |d| < 2^42
+    const int dh = (int)(d >> 12);                       // units of 2^-51
+    const u64 c = (u64)(d + (i64)(((i64)dh * dh) >> 39)); // d + d^2, units of 2^-63
+    // y (1 + c) in units of 2^-64, then the mantissa in [2^63, 2^64)
+    const i64 yc = (i64)((i64)(int)(c >> 31) * (i64)y) + (i64)(((u64)(u32)(c & 0x7fffffffu) * y) >> 31);
+    return ((u64)y << 32) + (u64)yc;
+}
+
+FX xf xf_rcp(xf a) { return xf{rcp64(a.m), -a.e - 1}; }
+
+// 2^64 / sqrt(f) for f = m 2^-62 in [1, 4), m in [2^62, 2^64): the mantissa of the reciprocal root,
+// value r 2^-64. A 23-bit start and one third-order step y (1 + d/2 + 3/8 d^2), d = 1 - f y^2.
+FX u64 rsqrt64(u64 m) {
+    const int up = (int)(m >> 63);                       // f >= 2
+    const float f = float_of_bits((up ? 0x40000000u : 0x3f800000u) |
+                                  ((u32)(m >> (up ? 40 : 39)) & 0x7fffffu));
+    const u32 b = bits_of_float(rsqrt_start(f));
+    const u32 y = b >= 0x3f800000u ? 0xfffffc00u : (((b & 0x7fffffu) | 0x800000u) << 8) - 0x400u;
+    const u64 p = mulhi64(m, (u64)y * y);                // f y^2 in units of 2^-62, up to 2 low
+    const i64 d = (i64)(0x3fffffffffffffffull - p);      // |d| < 2^43
+    const int dh = (int)(d >> 12);                       // units of 2^-50
+    const u64 c = (u64)(d + ((3 * ((i64)dh * dh)) >> 40));   // d/2 + 3/8 d^2, units of 2^-63
+    const i64 yc = (i64)((i64)(int)(c >> 31) * (i64)y) + (i64)(((u64)(u32)(c & 0x7fffffffu) * y) >> 31);
+    return ((u64)y << 32) + (u64)yc;
+}
+
+// e^a for a reduction already split off: a = kk ln2/256 + r, r72 = r in units of 2^-72
+// (0 <= r < 1.02 ln2/256). 2^(kk / 256) from the table times 1 + r + r^2/2 + r^3 (1/6 + r/24 +
+// r^2/120), the terms from the third on in 32-bit words; about 2^-58 of the value.
+FX xf exp_reduced(int kk, u64 r72) {
+    const u64 t = fix_exp_entry(kk & 255);               // 2^-62
+    const u64 r2 = mulhi64(r72, r72);                    // r^2, 2^-80
+    const u32 rh = (u32)(r72 >> 32);                     // 2^-40
+    const u32 r3 = mulhi32((u32)(r2 >> 32), rh);         // r^3, 2^-56
+    // 1/6 + r/24 + r^2/120 in units of 2^-34
+    const u32 c = 2863311531u + mulhi32(rh, 2796203u + mulhi32(rh, 2185u));
+    const u64 p = r72 + (r2 >> 9) + (((u64)r3 * c) >> 18);   // e^r - 1, 2^-72
+    const u64 v = t + (mulhi64(t, p) >> 8);              // [1, 2.0001) in units of 2^-62
+    const int up = (int)(v >> 63);
+    return xf{up ? v : v + v, (kk >> 8) + up};
+}
+
+// e^a, a in units of 2^-Q (Q 53: |a| < 1023; Q 58: |a| < 32).
+template <int Q>
+FX xf exp_fixed(i64 a) {
+    // floor(a 256/ln2), at most 0.01 low: the residue stays nonnegative
+    const int kk = (mulhi32s((int)(a >> 32), FIX_EXP_K19 >> (Q - 53)) - 1) >> 8;
+    const u64 r72 = ((u64)a << (72 - Q)) - (u64)(i64)kk * FIX_EXP_C72;
+    return exp_reduced(kk, r72);
+}
+
+// e^x for a finite binary64 |x| < 512 (the caller checks): the reduction takes every bit of x.
+FX double fix_exp(double x) {
+    const u64 u = bits_of(x);
+    const int ex = (int)((u >> 52) & 0x7ff) - 1023;      // < 9
+    const u64 m = (u << 11) | 0x8000000000000000ull;     // |x| 2^(63 - ex)
+    const bool neg = (i64)u < 0;
+    // |x| in units of 2^-72 mod 2^64 and its leading part in units of 2^-21
+    const int s = 9 + ex;
+    u64 a72 = s >= 0 ? m << s : (s > -64 ? m >> -s : 0);
+    const int sh = 10 - ex;
+    int ah = sh < 32 ? (int)((u32)(m >> 32) >> sh) : 0;
+    if (neg) {
+        a72 = 0 - a72;
+        ah = -ah - 1;
+    }
+    const int kk = (mulhi32s(ah, FIX_EXP_K19) - 1) >> 8;
+    return f64_of_xf(exp_reduced(kk, a72 - (u64)(i64)kk * FIX_EXP_C72));
+}
+
+// ln x in units of 2^-58 for a normal x in [2^-45, 2^45]: x = 2^k y, y in [1, 2), j the top 7
+// fraction bits of y, r = y inv_j - 1 (|r| < 2^-8), ln x = k ln2 - ln inv_j + log1p(r); within
+// 2^-54.
+FX i64 log58(double x) {
+    const u64 u = bits_of(x);
+    const int k = (int)((u >> 52) & 0x7ff) - 1023;
+    const u64 m = (u << 11) | 0x8000000000000000ull;
+    const u64* row = fix_log_row((int)(m >> 56) & 127);
+    const i64 r = (i64)(mulhi64(m, row[0]) - 0x8000000000000000ull);   // 2^-63, |r| < 2^55
+    const i64 rs = r << 7;                               // 2^-70
+    const int rh = (int)(rs >> 32);                      // 2^-38
+    const u64 ra = (u64)(rs < 0 ? -rs : rs);
+    const u64 r2 = mulhi64(ra, ra);                      // 2^-76
+    // 1/3 - r/4 + r^2/5 - r^3/6 + r^4/7 in units of 2^-32 (r/4 and on from 32-bit words)
+    const int c3 = 715827883 - (int)mulhi32s(rh, 9586981);   // 1/6 - r/7, units of 2^-32
+    const int c2 = 858993459 - (mulhi32s(rh, c3) >> 6);      // 1/5 - r (...)
+    const int c1 = 1073741824 - (mulhi32s(rh, c2) >> 6);     // 1/4 - r (...)
+    const int c0 = 1431655765 - (mulhi32s(rh, c1) >> 6);     // 1/3 - r (...)
+    const int r3 = (int)(((i64)(int)(r2 >> 29) * rh) >> 31);   // r^3, 2^-54
+    const i64 l = (r >> 5) - (i64)(r2 >> 19) + (((i64)r3 * c0) >> 28);   // log1p(r), 2^-58
+    return (i64)k * (i64)FIX_LN2_58 + (i64)row[1] + l;
+}
+
+// The binary64 nearest to v 2^-q for a signed v.
+FX double f64_of_signed(i64 v, int q) {
+    const double x = f64_of_fixed((u64)(v < 0 ? -v : v), q);
+    return v < 0 ? -x : x;
+}
+
+// 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of
+// the same range (positive under the roots): one rounding, within 0.51 ulp.
+FX bool fix_in_range(double b) {
+    const int eb = (int)((bits_of(b) >> 52) & 0x7ff);
+    return eb > 1023 - 500 && eb < 1023 + 500;
+}
+
+FX double fix_rcp(double b) {
+    const u64 u = bits_of(b);
+    const double r = f64_of_xf(xf_rcp(xf_of(b)));
+    return double_of(bits_of(r) | (u & 0x8000000000000000ull));
+}
+
+FX double fix_div(double a, double b) {
+    const u64 s = (bits_of(a) ^ bits_of(b)) & 0x8000000000000000ull;
+    const double q = f64_of_xf(xf_mul(xf_of(a), xf_rcp(xf_of(b))));
+    return double_of(bits_of(q) | s);
+}
+
+FX xf xf_rsqrt(xf a) {
+    const int odd = a.e & 1;                             // f = (m / 2^63) 2^odd in [1, 4)
+    const u64 r = rsqrt64(odd ? a.m : a.m >> 1);
+    return xf{r, -((a.e - odd) >> 1) - 1};
+}
+
+FX double fix_rsqrt(double a) { return f64_of_xf(xf_rsqrt(xf_of(a))); }
+
+FX double fix_sqrt(double a) {
+    const xf x = xf_of(a);
+    return f64_of_xf(xf_mul(x, xf_rsqrt(x)));
+}
+
+}  // namespace hyp

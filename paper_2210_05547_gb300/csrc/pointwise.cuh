@@ -243,7 +243,7 @@ __device__ __forceinline__ void ad_prep_body(const Scratch& s, long long lo, lon
         const int i = (int)li;
         const double ux = s.dudx[i], vy = s.dvdy[i], uy = s.dudy_c[i], vx = s.dvdx_c[i];
         const double sxy = uy + vx;
-        s.S[i] = sqrt(ux * ux + vy * vy + 0.5 * sxy * sxy);
+        s.S[i] = cl_sqrt(ux * ux + vy * vy + 0.5 * sxy * sxy);
         const double dv = ux + vy;
         const double om = vx - uy;
         s.div[i] = dv;

@@ -1324,10 +1324,10 @@ __global__ void k_fp64_fast(int fn, int64_t n, const double* __restrict__ a,
                             const double* __restrict__ b, double* __restrict__ out) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        if (fn == 0) out[i] = tang_exp(a[i]);
+        if (fn == 0) out[i] = fast_exp(a[i]);
         else if (fn == 1) out[i] = fast_div(a[i], b[i]);
         else if (fn == 2) out[i] = fast_rcp(b[i]);
-        else out[i] = table_log(a[i]);
+        else out[i] = fast_log(a[i]);
     }
 }
 

@@ -387,7 +387,7 @@ __global__ void k_adprep3(Grid3 g) {
         const double uy = g.dudy_c[q], vx = g.dvdx_c[q], uz = g.dudz_c[q], wx = g.dwdx_c[q];
         const double vz = g.dvdz_c[q], wy = g.dwdy_c[q];
         const double sxy = uy + vx, sxz = uz + wx, syz = vz + wy;
-        g.S[q] = sqrt(ux * ux + vy * vy + wz * wz + 0.5 * sxy * sxy + 0.5 * sxz * sxz + 0.5 * syz * syz);
+        g.S[q] = cl_sqrt(ux * ux + vy * vy + wz * wz + 0.5 * sxy * sxy + 0.5 * sxz * sxz + 0.5 * syz * syz);
         const double dv = ux + vy + wz;
         const double o1 = vx - uy, o2 = uz - wx, o3 = wy - vz;
         const double om2 = o1 * o1 + o2 * o2 + o3 * o3;

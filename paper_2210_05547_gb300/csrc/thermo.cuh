@@ -36,12 +36,11 @@ constexpr double OMEGA_CUT = 40.0;     // skip collision-integral exponentials b
 constexpr double NJA_A = 1.06036, NJA_B = 0.15610, NJA_C = 0.19300, NJA_D = 0.47635;
 constexpr double NJA_E = 1.03587, NJA_F = 1.52996, NJA_G = 1.76474, NJA_H = 3.89411;
 
-// Binary64 exponential, quotient and reciprocal of the closure: on the device the forms of
-// fp64_fast.cuh (Tang's table-driven exp, Newton-refined binary32 reciprocals; within 2 ulp, on
-// about half the FP64-pipe instructions of CUDA's), on the host the C library.
+// Binary64 exponential, quotient, reciprocal, logarithm and roots of the closure: on the device
+// the integer forms of fp64_fast.cuh, on the host the C library.
 __host__ __device__ __forceinline__ double cl_exp(double x) {
 #ifdef __CUDA_ARCH__
-    return tang_exp(x);
+    return fast_exp(x);
 #else
     return exp(x);
 #endif
@@ -63,13 +62,27 @@ __host__ __device__ __forceinline__ double cl_rcp(double b) {
 #endif
 }
 
-// Natural logarithm: on the device Tang's table-driven form for x >= 2 (fp64_fast.cuh; within
-// 1 ulp, 11 FP64 instructions against CUDA's ~28), CUDA's log below; on the host the C library.
 __host__ __device__ __forceinline__ double cl_log(double x) {
 #ifdef __CUDA_ARCH__
-    return table_log(x);
+    return fast_log(x);
 #else
     return log(x);
+#endif
+}
+
+__host__ __device__ __forceinline__ double cl_sqrt(double x) {
+#ifdef __CUDA_ARCH__
+    return fast_sqrt(x);
+#else
+    return sqrt(x);
+#endif
+}
+
+__host__ __device__ __forceinline__ double cl_rsqrt(double x) {
+#ifdef __CUDA_ARCH__
+    return fast_rsqrt(x);
+#else
+    return 1.0 / sqrt(x);
 #endif
 }
 
@@ -478,7 +491,7 @@ __host__ __device__ __forceinline__ void transport_f64(const GasDev& g, double T
 #pragma unroll
     for (int i = 0; i < NSP; ++i) {
         mu_s[i] = 0.1 * cl_exp((g.blA[i] * lnT + g.blB[i]) * lnT + g.blC[i]);
-        const double rs = rsqrt(mu_s[i]);           // 1 / sqrt(mu_i): one FP64 sequence for both
+        const double rs = cl_rsqrt(mu_s[i]);           // 1 / sqrt(mu_i): one FP64 sequence for both
         a[i] = mu_s[i] * rs * g.iMq[i];
         b[i] = g.Mq[i] * rs;
         const double cv_tr = 1.5 * g.Rs[i];
@@ -514,7 +527,7 @@ __host__ __device__ __forceinline__ void transport_f64(const GasDev& g, double T
 #pragma unroll
         for (int i = 0; i < NSP; ++i) den[i] = 0.0;
         const double TmB = cl_exp(-NJA_B * lnT);            // T^-B, shared by every well depth
-        const double rT = rsqrt(T);
+        const double rT = cl_rsqrt(T);
         const double c = p * (rT * (rT * rT));              // 1/D_sr = c Omega dinv_sr
         for (int q = 0; q < g.neps; ++q) {
             const double ts = T * g.eps_inv[q];
@@ -566,7 +579,7 @@ __host__ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rh
     o.p = p;
     o.cv = cv;
     o.Rmix = Rmix;
-    o.a = sqrt(cl_div((cv + Rmix) * p, cv * rho));
+    o.a = cl_sqrt(cl_div((cv + Rmix) * p, cv * rho));
 #pragma unroll
     for (int i = 0; i < NSP; ++i) {
         o.h[i] = s.e[i] + g.Rs[i] * T;
@@ -585,7 +598,7 @@ __host__ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rh
 #pragma unroll
     for (int i = 0; i < NSP; ++i) o.wdot[i] = 0.0;
     if (reactions) {
-        const double T15 = T * T * rsqrt(T);
+        const double T15 = T * T * cl_rsqrt(T);
         double r[NSP];
 #pragma unroll
         for (int i = 0; i < NSP; ++i) {

@@ -113,6 +113,18 @@ FX i64 mulhi64su(i64 a, u64 b) {
     return (i64)(a < 0 ? p - b : p);
 }
 
+// a b 2^-64 rounded to the nearest integer, a signed.
+FX i64 mulhi64su_rn(i64 a, u64 b) {
+    const u64 m = (u64)(a < 0 ? -a : a);
+#ifdef __CUDA_ARCH__
+    const u64 p = __umul64hi(m, b) + ((m * b) >> 63);
+#else
+    const unsigned __int128 w = (unsigned __int128)m * b;
+    const u64 p = (u64)(w >> 64) + (u64)((w >> 63) & 1);
+#endif
+    return a < 0 ? -(i64)p : (i64)p;
+}
+
 // A positive number (m / 2^63) 2^e, m in [2^63, 2^64), or zero (m = 0).
 struct xf {
     u64 m;

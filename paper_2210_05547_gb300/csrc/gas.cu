@@ -113,6 +113,89 @@ double h_sens_over_r(const SpeciesRow& r, double T) {
     return h;
 }
 
+// The integer constants of the closure, and whether the table fits their ranges.
+void fix_constants(GasDev& d) {
+    FixGas& f = d.fix;
+    memset(&f, 0, sizeof(f));
+    bool ok = true;
+    auto put = [&](double x, unsigned long long& m, int& e) {
+        const bool normal = x > 1e-250 && x < 1e250;
+        ok = ok && normal;
+        const xf v = xf_of(normal ? x : 1.0);
+        m = v.m;
+        e = v.e;
+    };
+    auto fixed = [&](double x, int q, double lim) {
+        ok = ok && fabs(x) < lim;
+        return fabs(x) < lim ? (long long)nearbyint(ldexp(x, q)) : 0;
+    };
+    const double lmax = log(T_HI);
+    for (int i = 0; i < NSP; ++i) {
+        double sum = 0.0;
+        ok = ok && d.lev_th[i][0] == 0.0;
+        for (int l = 0; l < d.nlev[i]; ++l) {
+            const double gl = d.lev_g[i][l];
+            ok = ok && gl >= 1.0 && gl <= 60.0 && gl == floor(gl);
+            f.lev_g[i][l] = ok ? (int)gl : 1;
+            sum += gl;
+            if (l > 0) put(d.lev_th[i][l], f.lev_m[i][l], f.lev_e[i][l]);
+        }
+        ok = ok && sum <= 60.0;
+        // theta_v >= 100 K: 1 - e^(-theta_v / T) keeps 54 bits up to 1e5 K
+        if (d.linear[i]) {
+            put(d.theta_v[i], f.tv_m[i], f.tv_e[i]);
+            ok = ok && d.theta_v[i] >= 100.0;
+        }
+        put(d.linear[i] ? d.A_tr[i] * d.inv_sr[i] : d.A_tr[i], f.r_m[i], f.r_e[i]);
+        put(d.iMq[i], f.iMq_m[i], f.iMq_e[i]);
+        if (!d.heavy[i]) continue;
+        f.bA63[i] = fixed(d.blA[i], 63, 0.99);
+        f.bB61[i] = fixed(d.blB[i], 61, 3.9);
+        f.bC57[i] = fixed(d.blC[i], 57, 30.0);
+        const double v = fabs(d.blA[i]) * lmax + fabs(d.blB[i]);
+        ok = ok && v < 3.9 && v * lmax + fabs(d.blC[i]) < 60.0;
+        for (int r = 0; r < NSP; ++r) f.wd64[i][r] = (unsigned long long)ldexp(d.wilke_d[i][r], 64);
+    }
+    // Wilke's a_s = sqrt(mu_s) M_s^(-1/4): all within a factor of 3.9 of each other
+    for (int k = 0; k <= 400; ++k) {
+        const double L = log(T_LO) + (lmax - log(T_LO)) * k / 400;
+        double lo = 1e300, hi = -1e300;
+        for (int i = 0; i < NSP; ++i) {
+            if (!d.heavy[i]) continue;
+            const double a = 0.5 * ((d.blA[i] * L + d.blB[i]) * L + d.blC[i]) + log(d.iMq[i]);
+            lo = fmin(lo, a);
+            hi = fmax(hi, a);
+        }
+        ok = ok && hi - lo < log(3.85);
+    }
+    const double expo[3] = {NJA_D, NJA_F, NJA_H}, coef[3] = {NJA_C, NJA_E, NJA_G};
+    f.njaB64 = (unsigned long long)ldexp(NJA_B, 64);
+    for (int k = 0; k < 3; ++k) f.oc62[k] = (unsigned long long)ldexp(coef[k], 62);
+    double top = 0.0;
+    for (int q = 0; q < d.neps; ++q) {
+        put(NJA_A * d.eps_powB[q], f.om_m[q], f.om_e[q]);
+        double om = NJA_A * d.eps_powB[q] * pow(T_LO, -NJA_B);
+        for (int k = 0; k < 3; ++k) {
+            put(expo[k] * d.eps_inv[q], f.oe_m[q][k], f.oe_e[q][k]);
+            om += coef[k] * exp(-expo[k] * d.eps_inv[q] * T_LO);
+        }
+        ok = ok && om < 3.9;                       // the integral falls with T
+    }
+    for (int k = 0; k < d.npair; ++k) top = fmax(top, d.pair_dinv[k]);
+    put(top, f.dscale_m, f.dscale_e);
+    for (int k = 0; k < d.npair; ++k) f.dinv63[k] = (unsigned long long)ldexp(d.pair_dinv[k] / top, 63);
+    for (int k = 0; k < d.ngroup; ++k) {
+        const double ta = d.g_Ta[k], tb = d.g_Ta[k] - d.g_theta_d[k];
+        f.n59[k] = fixed(d.g_n[k], 59, 8.0);
+        // |n ln T| < 93 and negative temperatures above -400 T_LO keep the exponent below 1000
+        ok = ok && ta > -400.0 * T_LO && tb > -400.0 * T_LO;
+        f.sgn[k] = (ta < 0.0 ? 1 : 0) | (tb < 0.0 ? 2 : 0);
+        if (ta != 0.0) put(fabs(ta), f.ta_m[k], f.ta_e[k]);
+        if (tb != 0.0) put(fabs(tb), f.tb_m[k], f.tb_e[k]);
+    }
+    f.ok = ok;
+}
+
 }  // namespace table
 }  // namespace hyp
 
@@ -400,6 +483,7 @@ extern "C" int hyp_gas_model_load(const char* path, int kind, const hyp_freestre
         d.f_eps_inv[q] = (float)d.eps_inv[q];
         d.f_eps_powB[q] = (float)d.eps_powB[q];
     }
+    fix_constants(d);
     d.etab_lnT0 = log(T_LO);
     d.etab_dlnT = (log(T_HI) - log(T_LO)) / (ETAB_N - 1);
     g->etab_host.assign(2 * NSP * ETAB_N, 0.0);
@@ -447,7 +531,7 @@ namespace gaskern {
 
 template <bool MIXED>
 __global__ void __launch_bounds__(128) k_thermo_eval(
-    GasDev g, int64_t n, const double* __restrict__ rho, const double* __restrict__ e,
+    const __grid_constant__ GasDev g, int64_t n, const double* __restrict__ rho, const double* __restrict__ e,
     const double* __restrict__ Y, double* __restrict__ T, double* __restrict__ p,
     double* __restrict__ wdot, double* __restrict__ mu, double* __restrict__ kk,
     double* __restrict__ D, uint8_t* __restrict__ status) {
@@ -459,8 +543,7 @@ __global__ void __launch_bounds__(128) k_thermo_eval(
 #pragma unroll
         for (int s = 0; s < NSP; ++s) y[s] = Y[s * n + i];
         ClosureOut o;
-        // binary64 modal sums in both precisions: independent states (closure_si_p, MODES32)
-        closure_si_p<MIXED, false>(g, rho[i], e[i], y, temperature_guess(g, e[i], y), reactions && wdot,
+        closure_si_p<MIXED>(g, rho[i], e[i], y, temperature_guess(g, e[i], y), reactions && wdot,
                             diffusion && D, o);
         if (T) T[i] = o.T;
         if (p) p[i] = o.p;

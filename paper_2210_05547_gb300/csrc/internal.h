@@ -40,6 +40,28 @@ int cuda_fail(cudaError_t err, const char* what);
         if (_e != cudaSuccess) return ::hyp::cuda_fail(_e, #call); \
     } while (0)
 
+// Integer constants of the closure (closure_fix.cuh): a name ending in a number n is in units of
+// 2^-n, a pair (_m, _e) is the number (m / 2^63) 2^e, m in [2^63, 2^64).
+struct FixGas {
+    int ok;                                      // the table fits the fixed-point ranges
+    int lev_g[NSP][MAXLEV];                      // degeneracies
+    int lev_e[NSP][MAXLEV], tv_e[NSP], r_e[NSP], iMq_e[NSP];
+    int ta_e[MAXG], tb_e[MAXG], sgn[MAXG];       // sgn: bit 0 T_a < 0, bit 1 T_a - theta_d < 0
+    int om_e[MAXEPS], oe_e[MAXEPS][3], dscale_e;
+    unsigned long long lev_m[NSP][MAXLEV];       // theta_el
+    unsigned long long tv_m[NSP];                // theta_v
+    unsigned long long r_m[NSP];                 // A_tr (atoms), A_tr / (sigma theta_r) (molecules)
+    unsigned long long iMq_m[NSP];               // M^(-1/4)
+    long long bA63[NSP], bB61[NSP], bC57[NSP];   // Blottner
+    unsigned long long wd64[NSP][NSP];           // wilke_d
+    long long n59[MAXG];
+    unsigned long long ta_m[MAXG], tb_m[MAXG];   // |T_a|, |T_a - theta_d|
+    unsigned long long om_m[MAXEPS];             // A eps^B of the collision integral
+    unsigned long long oe_m[MAXEPS][3];          // D / eps, F / eps, H / eps
+    unsigned long long oc62[3], njaB64;          // C, E, G; B
+    unsigned long long dinv63[NSP * (NSP - 1) / 2], dscale_m;   // pair_dinv / dscale
+};
+
 // Gas model as seen by the kernels: a plain struct passed by value as a kernel parameter.
 struct GasDev {
     int kind;                    // hyp_gas_kind
@@ -106,6 +128,7 @@ struct GasDev {
     double ln_isr[NSP];          // ln(1 / (sigma theta_r)) for linear molecules
     double theta0[NSP];          // E0_s / R_u (K): ground-state energy incl. formation
     double e_lo[NSP], e_hi[NSP]; // species energies at the ends of the inversion's range
+    FixGas fix;
 };
 
 }  // namespace hyp

@@ -27,7 +27,6 @@ constexpr int NEWTON_MAXIT = 60;
 // Stop after a Newton step of at most 1e-8 T: the error left after that step is of order
 // (dT/T)^2 ~ 1e-16 relative.
 constexpr double NEWTON_RTOL = 1.0e-8;
-constexpr double NEWTON_RTOL_MIXED = 1.0e-6;   // binary32 modal sums (temperature_from_energy)
 constexpr double SUTH_C1 = 1.458e-6;   // Eq. (24)
 constexpr double SUTH_TS = 110.4;      // Eq. (24)
 constexpr double LEVEL_CUT = 45.0;     // skip electronic levels with theta / T above this
@@ -168,93 +167,6 @@ __host__ __device__ __forceinline__ void species_shift(const GasDev& g, double T
     }
 }
 
-#ifdef __CUDACC__
-// The species modal sums of species_state for the mixed-precision closure (HYP_MIXED), split by
-// what each term contributes to the energy. In binary64: the vibrational factor
-// r = 1 / (e^x - 1) (theta_v r reaches ~T at high temperature) and the Boltzmann factors of the
-// populated electronic levels (theta / T < LEVEL_HOT_F64: the fine-structure levels of O and NO
-// at any temperature, the excited levels once they hold more than ~1e-4 of the population), with
-// the partition function q_el and the mean level energy m1 summed over them in binary64. In
-// binary32: the weakly populated levels (a level's energy share is at most (g_l / g_0) 9 e^-9 <=
-// 6.7e-3 of T, so its binary32 rounding, ~1e-6 relative with that of theta / T, moves e_s by
-// < 1e-8 R_s T), the second and third level moments and the heat capacities with their
-// temperature derivative. A fully binary32 electronic sum was measured to move the inverted
-// temperature by up to 5e-8 relative, which the exponents T_a / T ~ 50 of the dissociation rates
-// carry into the species source terms at ~1e-6 of their scale. The energy is assembled in
-// binary64 from its formation, translational-rotational (exact multiples of T), vibrational and
-// electronic parts. Every binary32 multiply and add is explicit, as in transport_f32.
-constexpr float LEVEL_HOT_F64 = 9.0f;
-
-__device__ __forceinline__ void species_state_f32(const GasDev& g, double T, SpeciesState& s) {
-    const double invT = cl_rcp(T);
-    const float iT = f32_of(invT);
-    const float iT2 = __fmul_rn(iT, iT);
-#pragma unroll
-    for (int i = 0; i < NSP; ++i) {
-        double qd = 0.0, s1d = 0.0;                     // binary64 sums: populated levels
-        float qc = 0.0f, s1c = 0.0f, s2 = 0.0f, s3 = 0.0f;
-        for (int l = 0; l < g.nlev[i]; ++l) {
-            const float th = f32_of(g.lev_th[i][l]);
-            const float x = __fmul_rn(th, iT);
-            if (x > (float)LEVEL_CUT) break;
-            float w;
-            if (x < LEVEL_HOT_F64) {
-                const double wd = th == 0.0f ? g.lev_g[i][l]
-                                             : g.lev_g[i][l] * cl_exp(-(g.lev_th[i][l] * invT));
-                qd += wd;
-                s1d = fma(wd, g.lev_th[i][l], s1d);
-                w = f32_of(wd);
-            } else {
-                w = __fmul_rn(f32_of(g.lev_g[i][l]), expf(-x));
-                qc = __fadd_rn(qc, w);
-                s1c = fmaf(w, th, s1c);
-            }
-            const float wt2 = __fmul_rn(__fmul_rn(w, th), th);
-            s2 = __fadd_rn(s2, wt2);
-            s3 = fmaf(wt2, th, s3);
-        }
-        qd += f64_of(qc);
-        // with no populated excited level (N2, and N and O2 below a few thousand K) the mean level
-        // energy is the weak levels' alone, below 3e-3 T: binary32 suffices
-        const double m1d = s1d == 0.0 ? f64_of(__fdiv_rn(s1c, f32_of(qd)))
-                                      : cl_div(s1d + f64_of(s1c), qd);
-        const float iq = __frcp_rn(f32_of(qd));
-        const float m1 = f32_of(m1d);
-        const float m2 = __fmul_rn(s2, iq);
-        const float m3 = __fmul_rn(s3, iq);
-        const float var = fmaf(-m1, m1, m2);
-        double ev = m1d;                                 // electronic + vibrational energy, K
-        float cvo = fmaf(var, iT2, 1.5f);
-        float cvpo = __fmul_rn(__fmul_rn(fmaf(-2.0f * m1, var, fmaf(-m1, m2, m3)), iT2), iT2);
-        cvpo = fmaf(__fmul_rn(-2.0f * var, iT2), iT, cvpo);
-        if (g.linear[i]) {
-            const double xd = g.theta_v[i] * invT;
-            const double rd = cl_inv_expm1(xd);
-            ev = fma(g.theta_v[i], rd, ev);
-            const float xv = f32_of(xd);
-            const float r = f32_of(rd);
-            const float b = __fmul_rn(__fadd_rn(1.0f, r), r);
-            const float xb = __fmul_rn(__fmul_rn(xv, xv), b);
-            cvo = __fadd_rn(cvo, __fadd_rn(1.0f, xb));
-            // d/dT [x^2 e^x / (e^x - 1)^2] = -(x / T) x b (2 - x - 2 x r)
-            const float t = __fsub_rn(__fsub_rn(2.0f, xv), __fmul_rn(2.0f * xv, r));
-            cvpo = fmaf(-__fmul_rn(xb, iT), t, cvpo);
-            s.iem1[i] = rd;
-            s.xv[i] = xd;
-        } else {
-            s.iem1[i] = 0.0;
-            s.xv[i] = 0.0;
-        }
-        const double ctr = g.linear[i] ? 2.5 : 1.5;     // translation (+ rotation), per R_s
-        s.e[i] = fma(g.Rs[i], fma(ctr, T, ev), g.e0[i]);
-        s.cv[i] = f64_of(__fmul_rn(g.f_Rs[i], cvo));
-        s.cvp[i] = f64_of(__fmul_rn(g.f_Rs[i], cvpo));
-        s.qel[i] = qd;
-        s.m1[i] = m1d;
-    }
-}
-#endif
-
 __host__ __device__ __forceinline__ double mixture_energy(const GasDev& g, double T, const double* Y) {
     SpeciesState s;
     species_state(g, T, s);
@@ -307,47 +219,38 @@ __host__ __device__ __forceinline__ double temperature_guess(const GasDev& g, do
     return Ta + t * h;
 }
 
-#ifdef __CUDACC__
-// The first-order shift of species_shift for the mixed-precision closure. The step is below
-// 1e-6 T (NEWTON_RTOL_MIXED), so the corrections of the partition function and vibrational
-// factor are at most 45 x 1e-6 of the value. They are formed in binary32, whose rounding stays
-// below 1e-11 of the value, and added in binary64. The energies and heat capacities take their
-// binary64 FMA. theta_v / T is not carried on, since nothing reads it after the shift.
-__device__ __forceinline__ void species_shift_f32(const GasDev& g, double T, double dT,
-                                                  SpeciesState& s) {
-    const float iT = __frcp_rn(f32_of(T));
-    const float dTf = f32_of(dT);
-    const float idT = __fmul_rn(iT, dTf);
+// The end of an inversion that did not converge: the energy lies outside the temperature range (T
+// clamped to its end) or the iteration failed; the mixture energies at the ends come from the
+// species energies there, which the gas model holds.
+__host__ __device__ __forceinline__ double temperature_not_found(const GasDev& g, double e,
+                                                        const double* Y, double T,
+                                                        unsigned& status) {
+    double elo = 0.0, ehi = 0.0;
 #pragma unroll
     for (int i = 0; i < NSP; ++i) {
-        s.e[i] = fma(s.cv[i], dT, s.e[i]);
-        s.cv[i] = fma(s.cvp[i], dT, s.cv[i]);
-        s.qel[i] += f64_of(__fmul_rn(__fmul_rn(f32_of(s.qel[i]), f32_of(s.m1[i])), __fmul_rn(iT, idT)));
-        if (g.linear[i]) {
-            const float r = f32_of(s.iem1[i]);
-            s.iem1[i] += f64_of(__fmul_rn(__fmul_rn(f32_of(s.xv[i]), idT), __fmul_rn(__fadd_rn(1.0f, r), r)));
-        }
+        elo += Y[i] * g.e_lo[i];
+        ehi += Y[i] * g.e_hi[i];
     }
+    if (e <= elo) {
+        status |= HYP_STATUS_T_CLAMPED;
+        return T_LO;
+    }
+    if (e >= ehi) {
+        status |= HYP_STATUS_T_CLAMPED;
+        return T_HI;
+    }
+    status |= HYP_STATUS_NOT_CONVERGED;
+    return T;
 }
-#endif
 
 // Safeguarded Newton for sum_s Y_s e_s(T) = e; s holds the species state at the returned T.
-// MIXED (device only): the electronic modal sums in binary32 (species_state_f32). Their rounding
-// moves sum_s Y_s e_s(T) by up to ~1e-8 c_v T, so successive Newton steps need not fall below
-// 1e-8 T; the iteration stops at 1e-6 T instead, where the step's own error, (dT/T)^2 relative,
-// and that of the first-order shift are ~1e-12, far below the binary32 part.
-template <bool MIXED = false>
 __host__ __device__ __forceinline__ double temperature_from_energy(const GasDev& g, double e,
                                                           const double* Y, double T0,
                                                           unsigned& status, SpeciesState& s) {
     double T = fmin(fmax(T0, T_LO), T_HI);
     double lo = T_LO, hi = T_HI;
     for (int it = 0; it < NEWTON_MAXIT; ++it) {
-#ifdef __CUDA_ARCH__
-        if constexpr (MIXED) species_state_f32(g, T, s);
-        else
-#endif
-            species_state(g, T, s);
+        species_state(g, T, s);
         double f = -e, cv = 0.0;
 #pragma unroll
         for (int i = 0; i < NSP; ++i) {
@@ -356,37 +259,14 @@ __host__ __device__ __forceinline__ double temperature_from_energy(const GasDev&
         }
         if (f > 0.0) hi = T; else lo = T;
         double Tn = T - cl_div(f, cv);
-        if (fabs(Tn - T) <= (MIXED ? NEWTON_RTOL_MIXED : NEWTON_RTOL) * T) {
-#ifdef __CUDA_ARCH__
-            if constexpr (MIXED) species_shift_f32(g, T, Tn - T, s);
-            else
-#endif
-                species_shift(g, T, Tn - T, s);
+        if (fabs(Tn - T) <= NEWTON_RTOL * T) {
+            species_shift(g, T, Tn - T, s);
             return Tn;
         }
         if (!(Tn > lo && Tn < hi)) Tn = 0.5 * (lo + hi);
         T = Tn;
     }
-    {
-        // the energy lies outside the temperature range (T clamped to its end) or the iteration
-        // failed; the mixture energies at the ends come from the species energies there, which
-        // the gas model holds (full species evaluations inlined here would only add code)
-        double elo = 0.0, ehi = 0.0;
-#pragma unroll
-        for (int i = 0; i < NSP; ++i) {
-            elo += Y[i] * g.e_lo[i];
-            ehi += Y[i] * g.e_hi[i];
-        }
-        if (e <= elo) {
-            T = T_LO;
-            status |= HYP_STATUS_T_CLAMPED;
-        } else if (e >= ehi) {
-            T = T_HI;
-            status |= HYP_STATUS_T_CLAMPED;
-        } else {
-            status |= HYP_STATUS_NOT_CONVERGED;
-        }
-    }
+    T = temperature_not_found(g, e, Y, T, status);
     species_state(g, T, s);
     return T;
 }
@@ -409,7 +289,7 @@ struct ClosureOut {
 // Blottner, Eucken, Wilke and Chapman-Enskog formulas as the FP64 code in closure_si, on binary32
 // copies of the constants. Inputs and outputs cross with the integer conversions of fp32.cuh.
 __device__ __forceinline__ void transport_f32(const GasDev& g, double T, double lnT, double p,
-                                     const SpeciesState& s, bool diffusion, ClosureOut& o) {
+                                     const double* cv, bool diffusion, ClosureOut& o) {
     // every binary32 multiply and add is explicit (fmaf where a fused operation is meant,
     // __fmul_rn / __fadd_rn / __fdiv_rn elsewhere): no contraction is left to the compiler, so
     // the result does not depend on the kernel this body is compiled into
@@ -423,7 +303,7 @@ __device__ __forceinline__ void transport_f32(const GasDev& g, double T, double 
         a[i] = __fmul_rn(__fmul_rn(mu_s[i], ir), g.f_iMq[i]);
         b[i] = __fmul_rn(g.f_Mq[i], ir);
         const float cv_tr = __fmul_rn(1.5f, g.f_Rs[i]);
-        k_s[i] = __fmul_rn(mu_s[i], fmaf(2.5f, cv_tr, __fsub_rn(f32_of(s.cv[i]), cv_tr)));
+        k_s[i] = __fmul_rn(mu_s[i], fmaf(2.5f, cv_tr, __fsub_rn(f32_of(cv[i]), cv_tr)));
     }
     float mu = 0.0f, kk = 0.0f;
 #pragma unroll
@@ -551,21 +431,13 @@ __host__ __device__ __forceinline__ void transport_f64(const GasDev& g, double T
     }
 }
 
-// Full closure (SI). reactions: evaluate w_s; diffusion: evaluate D_s. MIXED (device only): the
-// species modal sums (electronic and vibrational parts of e_s, c_v,s, the partition-function
-// factors), the forward rate exponentials, transport and diffusion in binary32; the Newton
-// iteration for T, the assembly of e_s, the equilibrium constants and backward rates stay FP64.
-// MODES32 (with MIXED): the split modal sums of species_state_f32. Its binary64-or-binary32
-// choice per electronic level follows T, so it stays uniform across a warp where neighbouring
-// cells have similar temperatures (the right-hand side); the sweep of independent states
-// (hyp_thermo_eval), whose temperatures differ from lane to lane, keeps the binary64 sums.
-template <bool MIXED, bool MODES32 = MIXED>
-__host__ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rho, double e,
-                                             const double* Y, double T0, bool reactions,
-                                             bool diffusion, ClosureOut& o) {
+// Full closure (SI) in binary64. reactions: evaluate w_s; diffusion: evaluate D_s.
+__host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho, double e, const double* Y,
+                                           double T0, bool reactions, bool diffusion,
+                                           ClosureOut& o) {
     SpeciesState s;
     o.status = rho > 0.0 ? 0u : HYP_STATUS_NONPHYSICAL;
-    const double T = temperature_from_energy<MIXED && MODES32>(g, e, Y, T0, o.status, s);
+    const double T = temperature_from_energy(g, e, Y, T0, o.status, s);
     double ym = 0.0, cv = 0.0;
 #pragma unroll
     for (int i = 0; i < NSP; ++i) {
@@ -628,12 +500,7 @@ __host__ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rh
             for (int rx = g.gstart[k]; rx < g.gstart[k + 1]; ++rx)
                 w += g.C[rx] * (g.spec[rx] >= 0 ? conc[g.spec[rx]] : 1.0);
             const double base = g.g_n[k] * lnT;
-            double Ef;
-#ifdef __CUDA_ARCH__
-            if (MIXED) Ef = f64_of(expf(f32_of(base - g.g_Ta[k] * invT)));
-            else
-#endif
-                Ef = cl_exp(base - g.g_Ta[k] * invT);
+            const double Ef = cl_exp(base - g.g_Ta[k] * invT);
             const double Eb = cl_exp(base - (g.g_Ta[k] - g.g_theta_d[k]) * invT) * cl_div(den, num);
             const double Rg = w * (Ef * fwd - Eb * bwd);
 #pragma unroll
@@ -644,20 +511,100 @@ __host__ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rh
         for (int i = 0; i < NSP; ++i) o.wdot[i] = g.M[i] * molar[i];
     }
 
-    if constexpr (MIXED) {
-#ifdef __CUDA_ARCH__
-        transport_f32(g, T, lnT, p, s, diffusion, o);
-#endif
-    } else {
-        transport_f64(g, T, lnT, p, s, diffusion, o);
-    }
+    transport_f64(g, T, lnT, p, s, diffusion, o);
 }
 
-__host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho, double e, const double* Y,
-                                           double T0, bool reactions, bool diffusion,
-                                           ClosureOut& o) {
-    closure_si_p<false>(g, rho, e, Y, T0, reactions, diffusion, o);
+}  // namespace hyp
+
+#include "closure_fix.cuh"
+
+namespace hyp {
+
+#ifdef __CUDACC__
+// The binary64 closure out of line: the states and gases that closure_fix.cuh does not take.
+static __device__ __noinline__ void closure_general(const GasDev& g, double rho, double e, const double* Y,
+                                             double T0, bool reactions, bool diffusion,
+                                             ClosureOut* o) {
+    closure_si(g, rho, e, Y, T0, reactions, diffusion, *o);
 }
+
+// The closure on integers; false (o unspecified) for states outside its range. MIXED: transport
+// and diffusion coefficients in binary32.
+template <bool MIXED>
+__device__ __forceinline__ bool closure_fix(const GasDev& g, double rho, double e, const double* Y,
+                                            double T0, bool reactions, bool diffusion,
+                                            ClosureOut& o) {
+    constexpr int LIM = 300;
+    const u64 ur = bits_of(rho);
+    if ((unsigned)((int)(ur >> 52) - 1023 + LIM) > 2u * LIM) return false;   // sign bit included
+    FixState s;
+    o.status = 0u;
+    const double T = temperature_from_energy_fix(g, e, Y, T0, o.status, s);
+    double ym = 0.0, cv = 0.0, ymol[NSP];
+#pragma unroll
+    for (int i = 0; i < NSP; ++i) {
+        ymol[i] = Y[i] * g.invM[i];
+        ym += ymol[i];
+        cv += Y[i] * s.cv[i];
+    }
+    const double Rmix = R_U * ym;
+    const double p = rho * Rmix * T;
+    if ((unsigned)((int)(bits_of(p) >> 52) - 1023 + LIM) > 2u * LIM) return false;
+    const double iym = cl_rcp(ym);
+    i64 X62[NSP];
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < NSP; ++i) {
+        o.X[i] = ymol[i] * iym;
+        ok = fix_signed62(o.X[i], X62[i]) && ok;
+    }
+    if (!ok) return false;
+    o.T = T;
+    o.p = p;
+    o.cv = cv;
+    o.Rmix = Rmix;
+    o.a = cl_sqrt(cl_div((cv + Rmix) * p, cv * rho));
+#pragma unroll
+    for (int i = 0; i < NSP; ++i) {
+        o.h[i] = s.e[i] + g.Rs[i] * T;
+        o.es[i] = s.e[i];
+        o.cvs[i] = s.cv[i];
+        o.cvps[i] = s.cvp[i];
+    }
+    const i64 L58 = log58(T);
+    if (reactions) {
+        double conc[NSP];
+#pragma unroll
+        for (int i = 0; i < NSP; ++i) conc[i] = rho * ymol[i];
+        kinetics_fix(g, T, L58, xf_rcp(xf_of(T)), s, conc, o.wdot);
+    } else {
+#pragma unroll
+        for (int i = 0; i < NSP; ++i) o.wdot[i] = 0.0;
+    }
+    if constexpr (MIXED) {
+        transport_f32(g, T, f64_of_fixed((u64)L58, 58), p, s.cv, diffusion, o);
+        return true;
+    }
+    if (!diffusion)
+#pragma unroll
+        for (int i = 0; i < NSP; ++i) o.D[i] = 0.0;
+    return transport_fix(g, T, L58, p, s.cv, o.X, X62, diffusion, o.mu, o.k, o.D);
+}
+
+// The closure of the kernels.
+template <bool MIXED>
+__device__ __forceinline__ void closure_si_p(const GasDev& g, double rho, double e, const double* Y,
+                                             double T0, bool reactions, bool diffusion,
+                                             ClosureOut& o) {
+    if (g.fix.ok && closure_fix<MIXED>(g, rho, e, Y, T0, reactions, diffusion, o)) return;
+    ClosureOut c;
+    double y[NSP];
+#pragma unroll
+    for (int i = 0; i < NSP; ++i) y[i] = Y[i];
+    closure_general(g, rho, e, y, T0, reactions, diffusion, &c);
+    o = c;
+}
+#endif
 
 // ---- thermally perfect gas (HYP_GAS_TPG; Eqs. 22-25) ----
 // c_p(T) = c_p0 (1 + g1 s(Theta/T)) with g1 = (gamma_inf - 1)/gamma_inf and the harmonic-oscillator
@@ -1020,7 +967,7 @@ __host__ __device__ __forceinline__ void lte_closure(const GasDev& g, double rho
     const double lnT = log(T);
     if constexpr (MIXED) {
 #ifdef __CUDA_ARCH__
-        transport_f32(g, T, lnT, p, q.s, true, o);
+        transport_f32(g, T, lnT, p, q.s.cv, true, o);
 #endif
     } else {
         transport_f64(g, T, lnT, p, q.s, true, o);

@@ -311,10 +311,11 @@ FX i64 log58(double x) {
     return (i64)k * (i64)FIX_LN2_58 + (i64)row[1] + l;
 }
 
-// The binary64 nearest to v 2^-q for a signed v.
+// The binary64 nearest to v 2^-q for a signed v (the sign set in its bit: a negation would issue on
+// the binary64 pipe).
 FX double f64_of_signed(i64 v, int q) {
     const double x = f64_of_fixed((u64)(v < 0 ? -v : v), q);
-    return v < 0 ? -x : x;
+    return double_of(bits_of(x) | ((u64)v & 0x8000000000000000ull));
 }
 
 // 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of

@@ -137,19 +137,17 @@ struct hyp_grid {
     int nstate;
     long long off[NSP + 3];
     double *xi_c, *xi_f, *eta_c, *eta_f;
-    float* metf;                 // binary32 copies of the four metric arrays, in that order
     double *Uref, *sigma;
     uint8_t* mask;
     unsigned* status;
     double* pool;
     Scratch s;
     LineOp* ops;
-    double* opdata;
+    hyp::LineTail* opdata;
     LineJob* jobs;
     std::vector<LineJob> hjobs;  // host copy of the launch plan (the batched executor joins plans)
     int ph_start[PH_COUNT], ph_count[PH_COUNT], ph_blocks[PH_COUNT];
-    double* linetmp;
-    long long linetmp_n;
+    long long linetmp_n;         // doubles the size limit of hyp_rhs_noalloc adds (sweep_doubles)
     cudaStream_t stream;
     double Tw_nd;
     EventProfile* prof;

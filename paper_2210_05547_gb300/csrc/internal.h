@@ -21,7 +21,10 @@
 #define MAXLEV 6               // electronic levels per species
 #define MAXEPS 16              // distinct Lennard-Jones well depths of species pairs
 #define ETAB_N 64              // temperatures of the species-energy table (start of the T inversion)
-#define LINE_BLOCK 128         // threads per block of the line-operator kernel
+#define LSEG 8                 // rows of a line per thread of the line-operator kernel
+#define LINE_THREADS 288       // threads per block: fits lines of 2^k + 1 rows (k = 5 .. 11)
+#define LINE_MAX_LINES 72      // lines per block, at most (a thread for each of 4 closure rows)
+#define LINE_TAIL 40           // rows a line's end reaches into (rho^40 < 2^-63)
 
 namespace hyp {
 
@@ -143,27 +146,24 @@ struct hyp_gas {
 
 namespace hyp {
 
-// One compact line operator (Sec. 3.1): tridiagonal left-hand side with precomputed Thomas
-// factors, interior right-hand-side weights and explicit closure rows.
+// What the unknown start of q adds to the first rows of a line (lines.cu): row k of the interior gets
+// h_k Q, h_k = (-rho)^(k+1) (1 - rho^(2 (n - k))) / (1 - rho^2), Q = kappa (y_left + rho y_first).
+struct LineTail {
+    long long h[LINE_TAIL], kappa;               // in units of 2^-64, 2^-63
+    double hd[LINE_TAIL], kappa_d;
+};
+
+// One compact line operator (Sec. 3.1): tridiagonal (alpha, 1, alpha) on the interior rows, explicit
+// closure rows at the ends.
 struct LineOp {
     int m, n_in;                 // output and input points along the line
     int dir;                     // 0 centre->face, 1 face->centre
     int kind;                    // 0 interpolation, 1 first derivative
     int wall;                    // 1: known value at position 0 enters the closure rows
+    int periodic;                // every row interior, indices modulo m
+    int margin;                  // rows a chunk (or an extended periodic line) starts early
     int first_interior, last_interior;
-    double wi[4];                // interior weights on inputs at offsets -3/2, -1/2, +1/2, +3/2
-    const double* lower;         // device: sub-diagonal of each row
-    const double* cprime;        // device: Thomas c'
-    const double* minv;          // device: Thomas 1 / pivot
-    const double* wa;            // device, interior rows: weight of (f_{+1/2} +/- f_{-1/2}) / pivot
-    const double* wb;            // device, interior rows: weight of (f_{+3/2} +/- f_{-3/2}) / pivot
-    const double* lm;            // device: sub-diagonal / pivot
-    // Interior rows rc..last_interior have bitwise-constant factors (the Thomas recurrence of the
-    // Toeplitz interior reaches its fixed point within about 20 rows): wa, wb, lm, cprime there.
-    int rc;
-    double wac, wbc, lmc, cpc;
-    float wac_f, wbc_f, lmc_f, cpc_f;   // the same in binary32 (HYP_MIXED jobs)
-    float wac_l, wbc_l, lmc_l, cpc_l;   // their remainders: (x_f, x_l) is x as a double word
+    const LineTail* tail;        // device; null for periodic lines
     int ncl;                     // closure rows (<= 4)
     int crow[4], cstart[4], cnum[4];
     double cw[4][5];
@@ -175,15 +175,14 @@ struct LineJob {
     const double* in;            // input field, or an element offset into the state when in_state
     int in_state;
     double* out;
-    double* tmp;                 // forward-sweep storage, same layout as out, distinct from it
     long long in_ls, in_es, out_ls, out_es;
     int nlines;
-    int nseg;                    // segments per line (power of two dividing the block size)
+    // plan_line: lines per block (and 2^20 over it), segments per line (or chunk), output rows per
+    // chunk, chunks, blocks per chunk and in all
+    int nl, inv_nl, nseg, cstep, nchunk, groups, blocks;
     double wall_value;
-    double scale;                // +1 or -1
+    double scale;                // factor on the results (sign, and 1 / spacing along z)
     const double* metric;        // per output element along the line, nullable
-    const float* metric_f;       // binary32 copy of metric (HYP_MIXED jobs)
-    int f32ok;                   // under HYP_MIXED the constant-factor rows may run in binary32
     // three-dimensional grids: lines grouped by plane, line L starting at
     // (L / lpp) * plane stride + (L % lpp) * line stride (lpp = 0: one group)
     int lpp;
@@ -191,7 +190,11 @@ struct LineJob {
     const double* wall_arr;      // per-line wall values (line index), replacing wall_value
 };
 
+// Fill in how a job's lines are spread over thread blocks (a function of the operator and the line
+// count alone).
+void plan_line(const LineOp& op, LineJob& j);
+
 cudaError_t launch_lines(const LineJob* d_jobs, int njobs, int max_blocks, const double* U,
-                         cudaStream_t s, int mixed = 0);
+                         cudaStream_t s);
 
 }  // namespace hyp

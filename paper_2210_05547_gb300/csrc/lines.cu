@@ -1,623 +1,442 @@
-// Batched compact staggered line operators (Sec. 3.1): y = A^{-1} (B x) along grid lines.
+// Batched compact staggered line operators (Sec. 3.1): y = A^{-1} (B x) along grid lines, on
+// 64-bit fixed-point numbers.
 //
-// GB300 retires two FP64 FMAs per clock per SM, so one warp-wide FP64 instruction occupies an
-// SM sub-partition for 64 cycles: a Thomas sweep of one 2049-point line run by a single thread
-// takes about a millisecond. The work is therefore spread over segments of each line.
+// What bounds it: a tridiagonal solve costs about seven binary64 operations per point, and GB300
+// has one binary64 unit per SM (19 cycles per warp instruction), so the binary64 sweeps this file
+// held before ran at 125 cycles per 32 points with that unit 60-85% busy and the lines' length
+// (latency) behind it. The operators are linear with constant coefficients and each line's values
+// share a scale, so the solve runs on integers: a product with a constant takes three 32-bit
+// integer products (3 cycles), a sum less than one. Per line, the inputs are scaled by the power
+// of two above their largest magnitude to 62 bits (exact for values down to 2^-9 of it); results
+// are in units of 2^-59 of that magnitude, where binary64 rounds the largest values at 2^-53.
 //
-// Every line is cut into `nseg` segments that live in the same thread block. Thread k:
-//   1. runs the forward recurrence d_r = (rhs_r - l_r d_{r-1}) / piv_r from W rows before its
-//      segment (starting from 0 there; exact when that start is row 0) and stores d_r for its own
-//      rows in `tmp`;
-//   2. after a barrier, runs the back substitution y_r = d_r - c'_r y_{r+1} from W rows past its
-//      segment end (starting from y = d there; exact at the last row), reading the forward values
-//      its neighbours stored, and writes its own rows.
-// The factors satisfy |l_r / piv_r| <= 1/3 and |c'_r| <= 1/3, so the history dropped at the
-// start of either recurrence is scaled by at most 3^-W: W = 40 (interpolation, alpha = 3/10) and
-// W = 26 (derivative, alpha = 9/62, factor <= 0.148) leave it below 1e-19 of the values, under
-// FP64 rounding. Each segment reads only values written before the barrier by threads of its own
-// block, so results are deterministic.
+// One thread solves LSEG = 8 consecutive rows of a line in registers; the threads of a line sit
+// in one block and exchange end values, so nothing is stored between the forward and
+// the backward recurrence (the earlier sweeps wrote and read it, and re-ran 26-40 warm-up rows per
+// segment). With rho / (1 + rho^2) = alpha the interior rows factor into
+//     q_r = (1 + rho^2) rhs_r - rho q_{r-1},     y_r = q_r - rho y_{r+1}
+// with the same rho (1/3, 0.148) on every row. A thread runs both from zero; what enters from its
+// neighbours follows from their own end values, q_in = e_{-1} + rho^8 e_{-2} + ... (five terms,
+// rho^40 < 2^-63), likewise y_in, and their effect on row k, a_k q_in + b_k y_in, is added. The row before the first interior row is an
+// explicit closure row, as is the row after the last: the latter starts the backward recurrence,
+// the former fixes q's unknown start Q, whose effect h_k Q is added to the first rows.
+// Periodic lines wrap the exchange around (or, when 16 does not divide the period, extend the line
+// by three segments each way), lines of more than LINE_THREADS segments are cut into chunks with
+// such margins.
 //
-// Past the first ~20 interior rows the Thomas factors are bitwise constant (LineOp::rc), so those
-// rows take their factors from registers and only the field values come from memory. A thread
-// has only a few FP64 instructions per row and the grid holds a few warps per sub-partition, so
-// the rows of that constant stretch are software-pipelined: the loads for row r + 8 are issued
-// while row r is computed.
+// Inputs and, for lines along x (unit stride), results pass through shared memory, 17 words per
+// thread of 16 so that neither the threads' rows nor the coalesced copies meet bank conflicts;
+// neighbouring threads hold neighbouring lines, which keeps the few threads with closure rows in
+// one or two warps.
 //
-// Under HYP_MIXED that constant stretch leaves the FP64 pipe. Jobs marked f32ok (the
-// interpolations and derivatives that feed only the diffusive fluxes) run it in plain binary32:
-// inputs are rounded with integer instructions, the recurrences run on the FP32 pipe, the forward
-// values of those rows are kept as binary32 in the first half of their 8-byte storage slot, and
-// outputs are widened back to binary64. The other derivatives (those feeding the convective
-// fluxes, the pressure and the divergences) form the adjacent differences of their inputs in
-// binary64 and run the recurrence in binary32 on those derivative-sized values (fwd_rows_cdiff).
-// The other interpolations run it in double-word arithmetic (dword.cuh): each binary64 input is
-// split into a pair of binary32 numbers, and the recurrences carry their rounding errors in the
-// low word (error-free sums and FMA products, about 48 significand bits). The forward values are
-// kept as a binary32 pair in the 8-byte slot, and each output is the binary64 sum of its pair.
-// Closure rows and the first interior rows stay FP64.
-#include "dword.cuh"
-#include "fp32.cuh"
+// Lines with NaN, infinities or magnitudes above 2^899 run the same steps in binary64 (the whole
+// block), so that such values spread as far as a binary64 solve lets them.
+//
+// Measured (GB300): the 50 operators of the face phase at 1024 x 256 take 190 us (the binary64
+// sweeps 234, the binary32 and double-word ones 201), a phase of one or two operators 19-21 us (38-46); the
+// step of the 2048 x 256 shock case 6.69 -> 5.96 ms, of the 256 x 64 boundary layer 0.85 -> 0.57,
+// the 256 x 128 x 64 jet's right-hand side 12.2 -> 10.5. About 280 integer instructions a row
+// warp at 2.2 per clock and SM bound it; eight rows a thread (four blocks of 288 threads per SM)
+// against sixteen (three): 5.96 against 6.5 ms. Converting the results to binary64 on the binary64
+// pipe instead of with integers: 6.4.
+#include "fix64.cuh"
 #include "internal.h"
+#include "line_table.h"
 
 namespace hyp {
 namespace {
 
-constexpr int PF = 8;   // prefetch distance (rows) of the constant-factor loops
-// the same for the double-word rows (16 or 24 rows were measured slower: the registers cost more
-// resident warps than the earlier loads gain)
-constexpr int PF_DW = 8;
+struct LineConst {
+    int h, l;
+    double d;
+};
+enum { C_P24 = 16, C_P32 = 17, C_WA = 18, C_WB = 19, C_G = 20, C_A = 21 };
+// per kind: rho^1 .. rho^16, rho^24, rho^32, the right-hand side's weights, rho^2 / (1 - rho^2), and
+// |response| of a segment's rows to what enters its forward recurrence,
+// rho^(k+1) (1 - rho^(2 (LSEG - k))) / (1 - rho^2), the sign (-1)^(k+1)
+__constant__ LineConst c_line[2][C_A + LSEG] = {LINE_TABLE_BODY};
 
-__device__ __forceinline__ double closure_rhs(const LineOp& op, const double* __restrict__ in,
-                                              long long ies, int r, double wall) {
-    int c = 0;
-    while (op.crow[c] != r) ++c;
-    double v = op.gw[c] * wall;
-    const double* p = in + (long long)op.cstart[c] * ies;
-    for (int k = 0; k < op.cnum[c]; ++k) v += op.cw[c][k] * p[(long long)k * ies];
+// m >> s, zero for s >= 64.
+__device__ __forceinline__ u64 shift_down(u64 m, int s) {
+    u64 v;
+    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // PTX clamps the shift amount
     return v;
 }
 
-// Sliding window of the four inputs of an interior row: p0..p2 held, p3 the new one.
-struct Window {
-    double p0, p1, p2;
+struct Fix {                                     // y is held as y / 4
+    typedef i64 T;
+    int E;                                       // inputs below 2^E
+    // x in units of 2^(E - q), truncated
+    __device__ __forceinline__ T scaled(double x, int q) const {
+        const int hi = __double2hiint(x);
+        const u64 m = ((u64)__double_as_longlong(x) << 11) | 0x8000000000000000ull;
+        const i64 v = (i64)shift_down(m, 63 - q + E + 1023 - ((hi >> 20) & 0x7ff));
+        const i64 s = hi >> 31;
+        return (v ^ s) - s;
+    }
+    __device__ __forceinline__ T input(double x) const { return scaled(x, 62); }
+    __device__ __forceinline__ T closure(double x) const { return scaled(x, 60); }
+    // y as binary64, its sign flipped by `sign` (0 or the sign bit)
+    __device__ __forceinline__ double value(T y, unsigned sign) const {
+        const int s = (int)(y >> 63);
+        const u64 m = (u64)((y ^ (i64)s) - (i64)s);
+        const u32 h = (u32)(m >> 32);
+        if (h < 2u) return small(m, (unsigned)(s & 0x80000000) ^ sign);
+        const int z = __clz(h) - 1;                          // leading one to bit 62
+        const u64 v = ((m << z) + 0x200) >> 10;              // [2^52, 2^53]
+        return __longlong_as_double((i64)(v + ((u64)(u32)(E + 2 - z + 1022) << 52)) |
+                                    (i64)((u64)((unsigned)(s & 0x80000000) ^ sign) << 32));
+    }
+    // |y| < 2^33 units
+    __device__ __noinline__ double small(u64 m, unsigned sign) const {
+        return __longlong_as_double(__double_as_longlong(f64_of_fixed(m, 60 - E)) | (i64)((u64)sign << 32));
+    }
+    static __device__ __forceinline__ T flip(T a, int kind) { return kind ? -a : a; }
+    // a c, c = (h 2^32 + l) 2^-64 (the sum of cross products stays below 2^63)
+    static __device__ __forceinline__ T mul(T a, const LineConst& c) {
+        const int ah = (int)(a >> 32);
+        const i64 x = (i64)ah * c.l + (i64)((u64)(u32)a * (u32)c.h);
+        return (i64)ah * c.h + (x >> 32);
+    }
+    static __device__ __forceinline__ T mul(T a, const LineTail& t, int k) { return __mul64hi(a, t.h[k]); }
+    static __device__ __forceinline__ T start(T a, const LineTail& t) { return __mul64hi(a, t.kappa) << 1; }
 };
 
-template <int KIND>
-__device__ __forceinline__ double interior_row(double d, const Window& w, double p3, double wa,
-                                               double wb, double lm) {
-    if (KIND == 0) return fma(-lm, d, fma(wa, w.p1 + w.p2, wb * (w.p0 + p3)));
-    return fma(-lm, d, fma(wa, w.p2 - w.p1, wb * (p3 - w.p0)));
-}
+struct Dbl {
+    typedef double T;
+    static __device__ __forceinline__ T input(double x) { return x; }
+    static __device__ __forceinline__ T closure(double x) { return x; }
+    static __device__ __forceinline__ double value(T y, unsigned sign) { return sign ? -y : y; }
+    static __device__ __forceinline__ T flip(T a, int kind) { return kind ? -a : a; }
+    static __device__ __forceinline__ T mul(T a, const LineConst& c) { return a * c.d; }
+    static __device__ __forceinline__ T mul(T a, const LineTail& t, int k) { return a * t.hd[k]; }
+    static __device__ __forceinline__ T start(T a, const LineTail& t) { return a * t.kappa_d; }
+};
 
-__device__ __forceinline__ void shift(Window& w, double p3) {
-    w.p0 = w.p1;
-    w.p1 = w.p2;
-    w.p2 = p3;
-}
-
-// Interior rows r..r1 with per-row factors; `p` points at the new input of row r and is advanced
-// past row r1.
-template <int KIND, bool STORE>
-__device__ __forceinline__ void fwd_rows_var(int r, int r1, double& d, Window& w,
-                                             const double* __restrict__& p, long long ies,
-                                             const LineOp& op, double* __restrict__ tmp,
-                                             long long oes) {
-    const double* __restrict__ wa = op.wa;
-    const double* __restrict__ wb = op.wb;
-    const double* __restrict__ lm = op.lm;
-#pragma unroll 2
-    for (; r <= r1; ++r) {
-        const double p3 = *p;
-        p += ies;
-        d = interior_row<KIND>(d, w, p3, wa[r], wb[r], lm[r]);
-        if (STORE) tmp[(long long)r * oes] = d;
-        shift(w, p3);
-    }
-}
-
-// Interior rows r..r1 with the constant factors, inputs prefetched PF rows ahead.
-template <int KIND, bool STORE>
-__device__ __forceinline__ void fwd_rows_const(int r, int r1, double& d, Window& w,
-                                               const double* __restrict__& p, long long ies,
-                                               const LineOp& op, double* __restrict__ tmp,
-                                               long long oes) {
-    const int n = r1 - r + 1;
-    if (n <= 0) return;
-    const double wa = op.wac, wb = op.wbc, lm = op.lmc;
-    const double* __restrict__ pp = p;
-    double q[PF];
+// Closure row c of a line.
+__device__ __forceinline__ double closure_rhs(const LineOp& op, const double* __restrict__ in,
+                                              long long ies, int c, double wall) {
+    const double* p = in + (long long)op.cstart[c] * ies;
+    const int n = op.cnum[c];
+    double x[5];
 #pragma unroll
-    for (int k = 0; k < PF; ++k) q[k] = k < n ? pp[(long long)k * ies] : 0.0;
-    for (; r + PF - 1 <= r1; r += PF) {
+    for (int k = 0; k < 5; ++k) x[k] = k < n ? p[(long long)k * ies] : 0.0;
+    double v = op.gw[c] * wall;
 #pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const double p3 = q[k];
-            q[k] = r + PF + k <= r1 ? pp[(long long)(PF + k) * ies] : 0.0;
-            d = interior_row<KIND>(d, w, p3, wa, wb, lm);
-            if (STORE) tmp[(long long)(r + k) * oes] = d;
-            shift(w, p3);
+    for (int k = 0; k < 5; ++k)
+        if (k < n) v += op.cw[c][k] * x[k];
+    return v;
+}
+
+constexpr int SLOT = LSEG + 1;                   // words of shared memory per thread
+
+struct Shared {
+    double stage[LINE_THREADS * SLOT];           // inputs, then results of x lines
+    u64 ends[2][LINE_THREADS];                   // segments' end values, forward and backward
+    u64 start[LINE_MAX_LINES];                   // Q
+    double clos[LINE_MAX_LINES][4];              // the closure rows' values, in the operator's order
+    unsigned top[LINE_MAX_LINES];                // largest |input|, high word
+};
+
+// The thread's place: rows r0 .. r0 + 15 of a line, segment `seg` of `nseg`; the line's next
+// segment is `nl` threads on.
+struct Place {
+    int r0, seg, nseg, nl, line, lo, hi;
+    bool active, wrap;
+};
+
+template <class T>
+__device__ __forceinline__ u64 raw(T v) {
+    u64 u;
+    memcpy(&u, &v, 8);
+    return u;
+}
+
+template <class T>
+__device__ __forceinline__ T cooked(u64 u) {
+    T v;
+    memcpy(&v, &u, 8);
+    return v;
+}
+
+// What enters a segment from the five segments before it (way -1) or after it (way 1): the sum of
+// their end values times rho^(8 (i - 1)), rho^40 < 2^-63.
+constexpr int TERMS = 5;
+
+template <class N>
+__device__ __forceinline__ typename N::T carried(const u64* ends, const Place& P, int way,
+                                                 const LineConst* C) {
+    typename N::T v = 0;
+#pragma unroll
+    for (int i = 1; i <= TERMS; ++i) {
+        int s = P.seg + way * i;
+        if (P.wrap) {
+            s %= P.nseg;
+            s += s < 0 ? P.nseg : 0;
         }
-        pp += PF * ies;
+        typename N::T e = 0;
+        if ((unsigned)s < (unsigned)P.nseg) e = cooked<typename N::T>(ends[(int)threadIdx.x + (s - P.seg) * P.nl]);
+        const int p = LSEG * (i - 1);
+        if (i == 1) v = e;
+        else v += N::mul(e, C[p == 32 ? C_P32 : (p == 24 ? C_P24 : p - 1)]);
     }
-#pragma unroll
-    for (int k = 0; k < PF - 1; ++k) {
-        if (r + k <= r1) {
-            const double p3 = q[k];
-            d = interior_row<KIND>(d, w, p3, wa, wb, lm);
-            if (STORE) tmp[(long long)(r + k) * oes] = d;
-            shift(w, p3);
-        }
-    }
-    p += (long long)n * ies;
+    return v;
 }
 
-__device__ __forceinline__ float* slot32(double* p) { return reinterpret_cast<float*>(p); }
-__device__ __forceinline__ const float* slot32(const double* p) {
-    return reinterpret_cast<const float*>(p);
-}
-
-template <int KIND>
-__device__ __forceinline__ float interior_row32(float d, float p0, float p1, float p2, float p3,
-                                                float wa, float wb, float lm) {
-    if (KIND == 0) return fmaf(-lm, d, fmaf(wa, p1 + p2, wb * (p0 + p3)));
-    return fmaf(-lm, d, fmaf(wa, p2 - p1, wb * (p3 - p0)));
-}
-
-// The constant-factor rows r..r1 in binary32 (f32ok jobs under HYP_MIXED).
-template <int KIND, bool STORE>
-__device__ __forceinline__ void fwd_rows_const32(int r, int r1, double& d, Window& w,
-                                                 const double* __restrict__& p, long long ies,
-                                                 const LineOp& op, double* __restrict__ tmp,
-                                                 long long oes) {
-    const int n = r1 - r + 1;
-    if (n <= 0) return;
-    const float wa = op.wac_f, wb = op.wbc_f, lm = op.lmc_f;
-    const double* __restrict__ pp = p;
-    float df = f32_of(d), p0 = f32_of(w.p0), p1 = f32_of(w.p1), p2 = f32_of(w.p2);
-    double q[PF];   // raw prefetched inputs; rounded when used so the load latency stays hidden
+// The solve and its output, once the inputs are in shared memory.
+template <class N>
+__device__ __forceinline__ void solve(const N& num, const LineJob& J, const LineOp& op, const Place& P,
+                                      Shared& sh, double* __restrict__ out) {
+    typedef typename N::T T;
+    const int kind = op.kind, fi = op.first_interior, li = op.last_interior, tid = threadIdx.x;
+    const LineConst* C = c_line[kind];
+    const bool left = !op.periodic && P.lo == 0;         // uniform per block
+    const bool first = left && P.active && P.seg == 0;
+    const int rr = P.active ? li + 1 - P.r0 : LSEG;      // the right closure row, if in this segment
+    const double* own = sh.stage + tid * SLOT;
+    const int next = P.seg + 1 < P.nseg ? tid + P.nl : (P.wrap ? tid - (P.nseg - 1) * P.nl : tid);
+    const double* nxt = sh.stage + (P.active ? next : tid) * SLOT;
+    // forward: f0 f1 f2 f3 at offsets -3/2 .. +3/2 of row r; g the same, negated for a derivative
+    T q[LSEG];
+    T g0 = N::flip(num.input(own[0]), kind), g1 = N::flip(num.input(own[1]), kind);
+    T f2 = num.input(own[2]), p = 0;
 #pragma unroll
-    for (int k = 0; k < PF; ++k) q[k] = k < n ? pp[(long long)k * ies] : 0.0;
-    for (; r + PF - 1 <= r1; r += PF) {
+    for (int k = 0; k < LSEG; ++k) {
+        const T f3 = num.input(k + 3 < LSEG ? own[k + 3] : nxt[k + 3 - LSEG]);
+        p = N::mul(f2 + g1, C[C_WA]) + N::mul(f3 + g0, C[C_WB]) - N::mul(p, C[0]);
+        if (k < 2 && first && k < fi) p = 0;             // q starts after the left closure rows
+        q[k] = p;
+        g0 = g1;
+        g1 = N::flip(f2, kind);
+        f2 = f3;
+    }
+    sh.ends[0][tid] = raw(p);
+    if (rr < LSEG) {                                     // the line ends here
+        const T yr = num.closure(rr >= 0 ? sh.clos[P.line][fi] : 0.0);
 #pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const float p3 = f32_of(q[k]);
-            q[k] = r + PF + k <= r1 ? pp[(long long)(PF + k) * ies] : 0.0;
-            df = interior_row32<KIND>(df, p0, p1, p2, p3, wa, wb, lm);
-            if (STORE) *slot32(tmp + (long long)(r + k) * oes) = df;
-            p0 = p1;
-            p1 = p2;
-            p2 = p3;
-        }
-        pp += PF * ies;
+        for (int k = 0; k < LSEG; ++k)
+            if (k >= rr) q[k] = k == rr ? yr : 0;
     }
+    // backward
+    T y = 0;
 #pragma unroll
-    for (int k = 0; k < PF - 1; ++k) {
-        if (r + k <= r1) {
-            const float p3 = f32_of(q[k]);
-            df = interior_row32<KIND>(df, p0, p1, p2, p3, wa, wb, lm);
-            if (STORE) *slot32(tmp + (long long)(r + k) * oes) = df;
-            p0 = p1;
-            p1 = p2;
-            p2 = p3;
-        }
-    }
-    d = f64_of(df);
-    w.p0 = f64_of(p0);
-    w.p1 = f64_of(p1);
-    w.p2 = f64_of(p2);
-    p += (long long)n * ies;
-}
-
-// The row's right-hand side is formed off the recurrence's dependency chain; the recurrence step
-// itself is dw_step (one binary32 product and sum on the chain of the high word).
-template <int KIND>
-__device__ __forceinline__ dword interior_row_dw(dword d, dword p0, dword p1, dword p2, dword p3,
-                                                 dword wa, dword wb, dword lm) {
-    const dword s1 = KIND == 0 ? dw_add(p1, p2) : dw_sub(p2, p1);
-    const dword s2 = KIND == 0 ? dw_add(p0, p3) : dw_sub(p3, p0);
-    return dw_step(d, dw_add(dw_mul(wa, s1), dw_mul(wb, s2)), lm);
-}
-
-// The constant-factor rows r..r1 in double-word arithmetic (jobs not marked f32ok under
-// HYP_MIXED). The window keeps each input both as binary64 (handed back to the FP64 rows that
-// follow) and as a double word.
-template <int KIND, bool STORE>
-__device__ __forceinline__ void fwd_rows_constdw(int r, int r1, double& d, Window& w,
-                                                 const double* __restrict__& p, long long ies,
-                                                 const LineOp& op, double* __restrict__ tmp,
-                                                 long long oes) {
-    const int n = r1 - r + 1;
-    if (n <= 0) return;
-    const dword wa{op.wac_f, op.wac_l}, wb{op.wbc_f, op.wbc_l}, lm{op.lmc_f, op.lmc_l};
-    const double* __restrict__ pp = p;
-    dword dd = dw_of(d), p0 = dw_of(w.p0), p1 = dw_of(w.p1), p2 = dw_of(w.p2);
-    double q[PF_DW];
-#pragma unroll
-    for (int k = 0; k < PF_DW; ++k) q[k] = k < n ? pp[(long long)k * ies] : 0.0;
-    for (; r + PF_DW - 1 <= r1; r += PF_DW) {
-#pragma unroll
-        for (int k = 0; k < PF_DW; ++k) {
-            const double x3 = q[k];
-            const dword p3 = dw_of(x3);
-            q[k] = r + PF_DW + k <= r1 ? pp[(long long)(PF_DW + k) * ies] : 0.0;
-            dd = interior_row_dw<KIND>(dd, p0, p1, p2, p3, wa, wb, lm);
-            if (STORE) dw_store(tmp + (long long)(r + k) * oes, dd);
-            p0 = p1;
-            p1 = p2;
-            p2 = p3;
-            shift(w, x3);
-        }
-        pp += PF_DW * ies;
-    }
-#pragma unroll
-    for (int k = 0; k < PF_DW - 1; ++k) {
-        if (r + k <= r1) {
-            const double x3 = q[k];
-            const dword p3 = dw_of(x3);
-            dd = interior_row_dw<KIND>(dd, p0, p1, p2, p3, wa, wb, lm);
-            if (STORE) dw_store(tmp + (long long)(r + k) * oes, dd);
-            p0 = p1;
-            p1 = p2;
-            p2 = p3;
-            shift(w, x3);
-        }
-    }
-    d = dw_to_f64(dd);
-    p += (long long)n * ies;
-}
-
-// The constant-factor rows r..r1 of a derivative (KIND 1) under HYP_MIXED, jobs not marked
-// f32ok. The row's right-hand side wa (p2 - p1) + wb (p3 - p0) is built from the adjacent
-// differences of the inputs: each difference is formed in binary64 and rounded to binary32. A
-// difference of neighbours within a factor of two is exact in binary64, else within an ulp of
-// itself. p3 - p0 is the sum of three adjacent differences. The recurrence then runs in binary32
-// on derivative-sized values. Their rounding is relative to the derivative, not to the field it
-// differentiates: the cancellation that made binary32 inputs miss the error bound happens in
-// the binary64 differences.
-template <bool STORE>
-__device__ __forceinline__ void fwd_rows_cdiff(int r, int r1, double& d, Window& w,
-                                               const double* __restrict__& p, long long ies,
-                                               const LineOp& op, double* __restrict__ tmp,
-                                               long long oes) {
-    const int n = r1 - r + 1;
-    if (n <= 0) return;
-    const float wa = op.wac_f, wb = op.wbc_f, lm = op.lmc_f;
-    const double* __restrict__ pp = p;
-    float df = f32_of(d);
-    float e1 = f32_of(w.p1 - w.p0), e2 = f32_of(w.p2 - w.p1);
-    double q[PF];
-#pragma unroll
-    for (int k = 0; k < PF; ++k) q[k] = k < n ? pp[(long long)k * ies] : 0.0;
-    for (; r + PF - 1 <= r1; r += PF) {
-#pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const double x3 = q[k];
-            q[k] = r + PF + k <= r1 ? pp[(long long)(PF + k) * ies] : 0.0;
-            const float e3 = f32_of(x3 - w.p2);
-            const float rhs = fmaf(wa, e2, __fmul_rn(wb, __fadd_rn(__fadd_rn(e1, e2), e3)));
-            df = fmaf(-lm, df, rhs);
-            if (STORE) *slot32(tmp + (long long)(r + k) * oes) = df;
-            e1 = e2;
-            e2 = e3;
-            shift(w, x3);
-        }
-        pp += PF * ies;
-    }
-#pragma unroll
-    for (int k = 0; k < PF - 1; ++k) {
-        if (r + k <= r1) {
-            const double x3 = q[k];
-            const float e3 = f32_of(x3 - w.p2);
-            const float rhs = fmaf(wa, e2, __fmul_rn(wb, __fadd_rn(__fadd_rn(e1, e2), e3)));
-            df = fmaf(-lm, df, rhs);
-            if (STORE) *slot32(tmp + (long long)(r + k) * oes) = df;
-            e1 = e2;
-            e2 = e3;
-            shift(w, x3);
-        }
-    }
-    d = f64_of(df);
-    p += (long long)n * ies;
-}
-
-// Forward sweep over rows r..r1 of one kind of region (closure / per-row / constant interior).
-template <int KIND, bool STORE, int MODE>
-__device__ __forceinline__ void fwd_span(int r, int r1, double& d, Window& w,
-                                         const double* __restrict__ in,
-                                         const double* __restrict__& p, long long ies,
-                                         const LineOp& op, double wall, double* __restrict__ tmp,
-                                         long long oes) {
-    if (r > r1) return;
-    const int fi = op.first_interior, li = op.last_interior, rc = op.rc;
-    const int base = op.dir == 0 ? -2 : -1;
-    // left closure rows
-    for (; r <= r1 && r < fi; ++r) {
-        d = (closure_rhs(op, in, ies, r, wall) - op.lower[r] * d) * op.minv[r];
-        if (STORE) tmp[(long long)r * oes] = d;
-    }
-    if (r > r1) return;
-    if (r <= li) {
-        // (re)load the window when entering the interior here
-        if (p == nullptr) {
-            const double* q = in + (long long)(r + base) * ies;
-            w.p0 = q[0];
-            w.p1 = q[ies];
-            w.p2 = q[2 * ies];
-            p = q + 3 * ies;
-        }
-        const int rv = min(r1, min(li, rc - 1));
-        if (r <= rv) {
-            fwd_rows_var<KIND, STORE>(r, rv, d, w, p, ies, op, tmp, oes);
-            r = rv + 1;
-        }
-        const int rcn = min(r1, li);
-        if (r <= rcn) {
-            if constexpr (MODE == 1) fwd_rows_const32<KIND, STORE>(r, rcn, d, w, p, ies, op, tmp, oes);
-            else if constexpr (MODE == 2) fwd_rows_constdw<KIND, STORE>(r, rcn, d, w, p, ies, op, tmp, oes);
-            else if constexpr (MODE == 3) fwd_rows_cdiff<STORE>(r, rcn, d, w, p, ies, op, tmp, oes);
-            else fwd_rows_const<KIND, STORE>(r, rcn, d, w, p, ies, op, tmp, oes);
-            r = rcn + 1;
-        }
-    }
-    // right closure rows
-    for (; r <= r1; ++r) {
-        d = (closure_rhs(op, in, ies, r, wall) - op.lower[r] * d) * op.minv[r];
-        if (STORE) tmp[(long long)r * oes] = d;
-    }
-}
-
-// Output modes of the back substitution: 0 none (warm-up rows), 1 y, 2 -y, 3 y met, 4 -y met.
-template <int OM>
-__device__ __forceinline__ void put(double* __restrict__ out, long long oes, int r, double y,
-                                    double m) {
-    if (OM == 1) out[(long long)r * oes] = y;
-    if (OM == 2) out[(long long)r * oes] = -y;
-    if (OM == 3) out[(long long)r * oes] = y * m;
-    if (OM == 4) out[(long long)r * oes] = -y * m;
-}
-
-// Back substitution over rows r0 >= r >= r1 (descending) with per-row c'.
-template <int OM>
-__device__ __forceinline__ void back_rows_var(int r0, int r1, double& y,
-                                              const double* __restrict__ tmp, long long oes,
-                                              const double* __restrict__ cpr,
-                                              const double* __restrict__ met,
-                                              double* __restrict__ out) {
-#pragma unroll 2
-    for (int r = r0; r >= r1; --r) {
-        y = tmp[(long long)r * oes] - cpr[r] * y;
-        put<OM>(out, oes, r, y, OM >= 3 ? met[r] : 0.0);
-    }
-}
-
-// Back substitution over rows r0 >= r >= r1 with the constant c', loads prefetched PF rows ahead.
-template <int OM>
-__device__ __forceinline__ void back_rows_const(int r0, int r1, double& y,
-                                                const double* __restrict__ tmp, long long oes,
-                                                double cc, const double* __restrict__ met,
-                                                double* __restrict__ out) {
-    const int n = r0 - r1 + 1;
-    if (n <= 0) return;
-    double q[PF], mq[PF];
-#pragma unroll
-    for (int k = 0; k < PF; ++k) {
-        q[k] = k < n ? tmp[(long long)(r0 - k) * oes] : 0.0;
-        mq[k] = (OM >= 3 && k < n) ? met[r0 - k] : 0.0;
-    }
-    int r = r0;
-    for (; r - PF + 1 >= r1; r -= PF) {
-#pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const double t = q[k], m = mq[k];
-            const int rn = r - PF - k;
-            q[k] = rn >= r1 ? tmp[(long long)rn * oes] : 0.0;
-            if (OM >= 3) mq[k] = rn >= r1 ? met[rn] : 0.0;
-            y = fma(-cc, y, t);
-            put<OM>(out, oes, r - k, y, m);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PF - 1; ++k) {
-        if (r - k >= r1) {
-            y = fma(-cc, y, q[k]);
-            put<OM>(out, oes, r - k, y, mq[k]);
-        }
-    }
-}
-
-template <int OM>
-__device__ __forceinline__ void put32(double* __restrict__ out, long long oes, int r, float y,
-                                      float m) {
-    if (OM == 1) out[(long long)r * oes] = f64_of(y);
-    if (OM == 2) out[(long long)r * oes] = f64_of(-y);
-    if (OM == 3) out[(long long)r * oes] = f64_of(y * m);
-    if (OM == 4) out[(long long)r * oes] = f64_of(-y * m);
-}
-
-// The constant-factor rows r0 >= r >= r1 in binary32, reading the binary32 forward values.
-template <int OM>
-__device__ __forceinline__ void back_rows_const32(int r0, int r1, double& y,
-                                                  const double* __restrict__ tmp, long long oes,
-                                                  float cc, const float* __restrict__ met,
-                                                  double* __restrict__ out) {
-    const int n = r0 - r1 + 1;
-    if (n <= 0) return;
-    float yf = f32_of(y);
-    float q[PF], mq[PF];
-#pragma unroll
-    for (int k = 0; k < PF; ++k) {
-        q[k] = k < n ? *slot32(tmp + (long long)(r0 - k) * oes) : 0.0f;
-        mq[k] = (OM >= 3 && k < n) ? met[r0 - k] : 0.0f;
-    }
-    int r = r0;
-    for (; r - PF + 1 >= r1; r -= PF) {
-#pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const float t = q[k], m = mq[k];
-            const int rn = r - PF - k;
-            q[k] = rn >= r1 ? *slot32(tmp + (long long)rn * oes) : 0.0f;
-            if (OM >= 3) mq[k] = rn >= r1 ? met[rn] : 0.0f;
-            yf = fmaf(-cc, yf, t);
-            put32<OM>(out, oes, r - k, yf, m);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PF - 1; ++k) {
-        if (r - k >= r1) {
-            yf = fmaf(-cc, yf, q[k]);
-            put32<OM>(out, oes, r - k, yf, mq[k]);
-        }
-    }
-    y = f64_of(yf);
-}
-
-// The constant-factor rows r0 >= r >= r1 in double-word arithmetic, reading the double-word
-// forward values; each output is the binary64 sum of its pair (times the metric in binary64).
-template <int OM>
-__device__ __forceinline__ void back_rows_constdw(int r0, int r1, double& y,
-                                                  const double* __restrict__ tmp, long long oes,
-                                                  dword cc, const double* __restrict__ met,
-                                                  double* __restrict__ out) {
-    const int n = r0 - r1 + 1;
-    if (n <= 0) return;
-    dword yd = dw_of(y);
-    dword q[PF_DW];
-    double mq[PF_DW];
-#pragma unroll
-    for (int k = 0; k < PF_DW; ++k) {
-        q[k] = k < n ? dw_load(tmp + (long long)(r0 - k) * oes) : dword{0.0f, 0.0f};
-        mq[k] = (OM >= 3 && k < n) ? met[r0 - k] : 0.0;
-    }
-    int r = r0;
-    for (; r - PF_DW + 1 >= r1; r -= PF_DW) {
-#pragma unroll
-        for (int k = 0; k < PF_DW; ++k) {
-            const dword t = q[k];
-            const double m = mq[k];
-            const int rn = r - PF_DW - k;
-            q[k] = rn >= r1 ? dw_load(tmp + (long long)rn * oes) : dword{0.0f, 0.0f};
-            if (OM >= 3) mq[k] = rn >= r1 ? met[rn] : 0.0;
-            yd = dw_step(yd, t, cc);
-            if (OM != 0) put<OM>(out, oes, r - k, dw_to_f64(yd), m);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PF_DW - 1; ++k) {
-        if (r - k >= r1) {
-            yd = dw_step(yd, q[k], cc);
-            if (OM != 0) put<OM>(out, oes, r - k, dw_to_f64(yd), mq[k]);
-        }
-    }
-    y = dw_to_f64(yd);
-}
-
-// Back substitution over rows r0 >= r >= r1, split at the constant-factor stretch.
-template <int OM, int MODE>
-__device__ __forceinline__ void back_span(int r0, int r1, double& y, const LineOp& op,
-                                          const double* __restrict__ tmp, long long oes,
-                                          const double* __restrict__ met,
-                                          const float* __restrict__ met_f,
-                                          double* __restrict__ out) {
-    if (r0 < r1) return;
-    const int li = op.last_interior, rc = op.rc;
-    const int a = max(r1, li + 1);            // rows above the interior (right closure)
-    if (r0 >= a) back_rows_var<OM>(r0, a, y, tmp, oes, op.cprime, met, out);
-    const int c0 = min(r0, li), c1 = max(r1, rc);
-    if (c0 >= c1) {
-        if (MODE == 1 || MODE == 3) back_rows_const32<OM>(c0, c1, y, tmp, oes, op.cpc_f, met_f, out);
-        else if (MODE == 2)
-            back_rows_constdw<OM>(c0, c1, y, tmp, oes, dword{op.cpc_f, op.cpc_l}, met, out);
-        else back_rows_const<OM>(c0, c1, y, tmp, oes, op.cpc, met, out);
-    }
-    const int v0 = min(r0, rc - 1);
-    if (v0 >= r1) back_rows_var<OM>(v0, r1, y, tmp, oes, op.cprime, met, out);
-}
-
-template <int KIND, int MODE>
-__device__ __forceinline__ void forward(const LineJob& J, const LineOp& op,
-                                        const double* __restrict__ in, double* __restrict__ tmp,
-                                        int s, int e, int W, double wall) {
-    const int fs = max(0, s - W);
-    const long long ies = J.in_es, oes = J.out_es;
-    double d = 0.0;
-    Window w{0.0, 0.0, 0.0};
-    const double* __restrict__ p = nullptr;
-    fwd_span<KIND, false, MODE>(fs, s - 1, d, w, in, p, ies, op, wall, tmp, oes);
-    fwd_span<KIND, true, MODE>(s, e, d, w, in, p, ies, op, wall, tmp, oes);
-}
-
-template <int OM, int MODE>
-__device__ __forceinline__ void backward(const LineOp& op, const double* __restrict__ tmp,
-                                         long long oes, const double* __restrict__ met,
-                                         const float* __restrict__ met_f,
-                                         double* __restrict__ out, int s, int e, int be) {
-    // the last row is a closure row (FP64 storage) or, for lines without one, an interior row
-    const bool last_c = MODE != 0 && be >= op.rc && be <= op.last_interior;
-    double y;
-    if (last_c && (MODE == 1 || MODE == 3)) y = f64_of(*slot32(tmp + (long long)be * oes));
-    else if (last_c) y = dw_to_f64(dw_load(tmp + (long long)be * oes));
-    else y = tmp[(long long)be * oes];
-    if (be <= e) put<OM>(out, oes, be, y, OM >= 3 ? met[be] : 0.0);
-    back_span<0, MODE>(be - 1, e + 1, y, op, tmp, oes, met, met_f, out);   // warm-up rows
-    back_span<OM, MODE>(min(be - 1, e), s, y, op, tmp, oes, met, met_f, out);
-}
-
-template <int MODE>
-__device__ __forceinline__ void run_line(const LineJob& J, const LineOp& op,
-                                         const double* __restrict__ in, double* __restrict__ out,
-                                         double* __restrict__ tmp, int s, int e, int m, int W,
-                                         bool active, double wall) {
-    if (active && s <= e) {
-        if constexpr (MODE == 3) forward<1, MODE>(J, op, in, tmp, s, e, W, wall);   // derivatives only
-        else if (op.kind == 0) forward<0, MODE>(J, op, in, tmp, s, e, W, wall);
-        else forward<1, MODE>(J, op, in, tmp, s, e, W, wall);
+    for (int k = LSEG - 1; k >= 0; --k) {
+        y = q[k] - N::mul(y, C[0]);
+        q[k] = y;
     }
     __syncthreads();
-    if (active && s <= e) {
-        const int be = min(e + W, m - 1);
-        const double* __restrict__ met = J.metric;
-        const float* __restrict__ met_f = J.metric_f;
-        const bool neg = J.scale < 0.0;
-        const long long oes = J.out_es;
-        if (met) {
-            if (neg) backward<4, MODE>(op, tmp, oes, met, met_f, out, s, e, be);
-            else backward<3, MODE>(op, tmp, oes, met, met_f, out, s, e, be);
-        } else {
-            if (neg) backward<2, MODE>(op, tmp, oes, met, met_f, out, s, e, be);
-            else backward<1, MODE>(op, tmp, oes, met, met_f, out, s, e, be);
+    const T qin = carried<N>(sh.ends[0], P, -1, C);
+    if (rr >= LSEG) {
+#pragma unroll
+        for (int k = 0; k < LSEG; ++k) {
+            const T c = N::mul(qin, C[C_A + k]);
+            q[k] = (k & 1) ? q[k] + c : q[k] - c;
+        }
+    } else {                                             // rows from rr on do not respond
+        const T qe = qin + N::mul(qin, C[C_G]);
+#pragma unroll
+        for (int k = 0; k < LSEG; ++k) {
+            if (k >= rr) continue;
+            const T c = N::mul(qe, C[k]) - N::mul(qe, C[2 * rr - k]);
+            q[k] = (k & 1) ? q[k] + c : q[k] - c;
+        }
+    }
+    sh.ends[1][tid] = raw(q[0]);
+    __syncthreads();
+    const T yin = carried<N>(sh.ends[1], P, 1, C);
+#pragma unroll
+    for (int k = 0; k < LSEG; ++k) {
+        const T c = N::mul(yin, C[LSEG - 1 - k]);
+        q[k] = ((LSEG - k) & 1) ? q[k] - c : q[k] + c;
+    }
+    if (left) {
+        if (first) {
+            const T Yl = num.closure(sh.clos[P.line][fi - 1]);
+            sh.start[P.line] = raw(N::start(Yl + N::mul(fi == 1 ? q[1] : q[2], C[0]), op.tail[0]));
+        }
+        __syncthreads();
+        if (P.active && P.seg < LINE_TAIL / LSEG) {
+            const T Q = cooked<T>(sh.start[P.line]);
+#pragma unroll
+            for (int k = 0; k < LSEG; ++k) {
+                const int i = P.r0 + k - fi;
+                if (i >= 0 && i < LINE_TAIL) q[k] += N::mul(Q, op.tail[0], i);
+            }
+        }
+    }
+    // output: sign and constant factor, then the metric
+    const double scale = J.scale;
+    const unsigned sign = (unsigned)__double2hiint(scale) & 0x80000000u;
+    const bool scaled = ((unsigned)__double2hiint(scale) & 0x7fffffffu) != 0x3ff00000u || __double2loint(scale);
+    const double* __restrict__ met = J.metric;
+    const bool edge = P.r0 < fi || rr < LSEG || P.r0 < P.lo || P.r0 + LSEG > P.hi;
+    double* st = sh.stage + tid * SLOT;
+    double* __restrict__ o = out + (long long)P.r0 * J.out_es;
+    const bool xl = J.in_es == 1;
+#pragma unroll
+    for (int k = 0; k < LSEG; ++k) {
+        double v = num.value(q[k], sign);
+        bool put = P.active;
+        if (edge) {
+            const int r = P.r0 + k;
+            put = put && r >= P.lo && r < P.hi;
+            if (put && (r < fi || r > li)) {
+                v = sh.clos[P.line][r < fi ? r : fi + r - li - 1];
+                if (sign) v = -v;
+            }
+        }
+        if (scaled) v *= fabs(scale);
+        if (xl) {
+            st[k] = v;
+        } else if (put) {
+            if (met) v *= met[P.r0 + k];
+            *o = v;
+        }
+        o += J.out_es;
+    }
+    if (xl) {
+        __syncthreads();
+        if (P.active) {
+            const int row0 = P.r0 - P.seg * LSEG;
+            for (unsigned j = P.seg; j < (unsigned)(P.nseg * LSEG); j += P.nseg) {
+                const int r = row0 + (int)j;
+                if (r < P.lo || r >= P.hi) continue;
+                double v = sh.stage[((j / LSEG) * P.nl + P.line) * SLOT + (j % LSEG)];
+                if (met) v *= met[r];
+                out[r] = v;
+            }
         }
     }
 }
 
-// One instantiation per precision: the FP64 one carries only the binary64 sweeps (and keeps its
-// registers), the HYP_MIXED one the binary32 and double-word sweeps beside the binary64 rows.
-template <bool MIXED>
-__global__ void __launch_bounds__(LINE_BLOCK) k_lines(const LineJob* __restrict__ jobs,
-                                                                       const double* __restrict__ U) {
+// The rare binary64 form, out of line.
+__device__ __noinline__ void solve_wild(const LineJob& J, const LineOp& op, const Place& P, Shared& sh,
+                                        double* __restrict__ out) {
+    solve<Dbl>(Dbl(), J, op, P, sh, out);
+}
+
+__device__ __forceinline__ unsigned magnitude(double x) {
+    return (unsigned)__double2hiint(x) & 0x7fffffffu;
+}
+
+__global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __restrict__ jobs,
+                                                           const double* __restrict__ U) {
+    __shared__ Shared sh;
     const LineJob& J = jobs[blockIdx.y];
-    const int nseg = J.nseg;
-    const int lpb = blockDim.x / nseg;                  // lines per block
-    const int seg = threadIdx.x / lpb;
-    const int line = blockIdx.x * lpb + (threadIdx.x - seg * lpb);
-    const bool active = line < J.nlines;
     const LineOp& op = *J.op;
-    const int m = op.m;
-    const int L = (m + nseg - 1) / nseg;
-    const int s = seg * L;
-    const int e = min(s + L, m) - 1;
-    const int W = op.kind == 0 ? 40 : 26;
-    long long ioff, ooff;
-    if (J.lpp) {
-        const int k = line / J.lpp, l = line - k * J.lpp;
-        ioff = k * J.in_ps + (long long)l * J.in_ls;
-        ooff = k * J.out_ps + (long long)l * J.out_ls;
+    const int nl = J.nl, nseg = J.nseg, tid = threadIdx.x;
+    const int chunk = J.nchunk == 1 ? 0 : blockIdx.x / J.groups;
+    const int group = blockIdx.x - chunk * J.groups;
+    if (group >= J.groups) return;
+    Place P;
+    P.lo = chunk * J.cstep;                              // output rows [lo, hi)
+    if (P.lo >= op.m) return;
+    P.hi = min(op.m, P.lo + J.cstep);
+    P.nseg = nseg;
+    P.nl = nl;
+    P.seg = (tid * J.inv_nl) >> 20;                      // tid / nl
+    P.line = tid - P.seg * nl;
+    P.wrap = op.periodic && !op.margin;
+    const int line = group * nl + P.line;
+    P.active = P.seg < nseg && line < J.nlines;
+    const int row0 = P.lo - (P.lo > 0 || op.periodic ? op.margin : 0);
+    P.r0 = row0 + P.seg * LSEG;
+    auto offset = [&](int l, long long ls, long long ps) {
+        if (!J.lpp) return (long long)l * ls;
+        const int k = l / J.lpp;
+        return k * ps + (long long)(l - k * J.lpp) * ls;
+    };
+    const double* __restrict__ base_in = J.in_state ? U + (size_t)J.in : J.in;
+    const double* __restrict__ in = base_in + (P.active ? offset(line, J.in_ls, J.in_ps) : 0);
+    double* __restrict__ out = J.out + (P.active ? offset(line, J.out_ls, J.out_ps) : 0);
+    const double wall = (J.wall_arr && P.active) ? J.wall_arr[line] : J.wall_value;
+    if (tid < LINE_MAX_LINES) sh.top[tid] = 0;
+    __syncthreads();
+
+    // inputs: row r reads r + base .. r + base + 3
+    const int base = op.dir == 0 ? -2 : -1, n_in = op.n_in;
+    unsigned top = op.wall ? magnitude(wall) : 0u;
+    double* st = sh.stage + tid * SLOT;
+    if (!P.active) {
+#pragma unroll
+        for (int k = 0; k < LSEG; ++k) st[k] = 0.0;
+    } else if (J.in_es == 1) {
+        const int j0 = row0 + base;
+        for (unsigned j = P.seg; j < (unsigned)(nseg * LSEG); j += nseg) {
+            const int i = j0 + (int)j;
+            const double v = (unsigned)i < (unsigned)n_in ? in[i] : 0.0;
+            sh.stage[((j / LSEG) * nl + P.line) * SLOT + (j % LSEG)] = v;
+            top = max(top, magnitude(v));
+        }
     } else {
-        ioff = (long long)line * J.in_ls;
-        ooff = (long long)line * J.out_ls;
+        const long long ies = J.in_es;
+        int j = P.r0 + base;
+        if (op.periodic) {
+            j %= n_in;
+            j += j < 0 ? n_in : 0;
+#pragma unroll
+            for (int k = 0; k < LSEG; ++k) {
+                const double v = in[j * ies];
+                st[k] = v;
+                top = max(top, magnitude(v));
+                j = j + 1 == n_in ? 0 : j + 1;
+            }
+        } else {
+            const double* __restrict__ p = in + j * ies;
+#pragma unroll
+            for (int k = 0; k < LSEG; ++k) {
+                const double v = (unsigned)(j + k) < (unsigned)n_in ? *p : 0.0;
+                st[k] = v;
+                top = max(top, magnitude(v));
+                p += ies;
+            }
+        }
     }
-    const double* __restrict__ in = (J.in_state ? U + (size_t)J.in : J.in) + ioff;
-    double* __restrict__ out = J.out + ooff;
-    double* __restrict__ tmp = J.tmp + ooff;
-    const double wall = (J.wall_arr && active) ? J.wall_arr[line] : J.wall_value;
-    // uniform per block: every thread of a block works on the same job
-    if constexpr (MIXED) {
-        if (J.f32ok) run_line<1>(J, op, in, out, tmp, s, e, m, W, active, wall);
-        else if (op.kind == 1) run_line<3>(J, op, in, out, tmp, s, e, m, W, active, wall);
-        else run_line<2>(J, op, in, out, tmp, s, e, m, W, active, wall);
-    } else {
-        run_line<0>(J, op, in, out, tmp, s, e, m, W, active, wall);
+    if (P.active) atomicMax(&sh.top[P.line], top);
+    // the closure rows, one per thread from the block's end
+    if (!op.periodic && LINE_THREADS - 1 - tid < nl * op.ncl) {
+        const int i = LINE_THREADS - 1 - tid, c = (i * J.inv_nl) >> 20, l = i - c * nl;
+        const int ln = group * nl + l;
+        if (ln < J.nlines)
+            sh.clos[l][c] = closure_rhs(op, base_in + offset(ln, J.in_ls, J.in_ps), J.in_es, c,
+                                        J.wall_arr ? J.wall_arr[ln] : J.wall_value);
     }
+    if (__syncthreads_or(P.active && top >= (unsigned)(1023 + 899) << 20)) {
+        solve_wild(J, op, P, sh, out);
+        return;
+    }
+    Fix num;
+    num.E = max((int)(sh.top[P.line < nl && P.active ? P.line : 0] >> 20) - 1022, -960);
+    solve<Fix>(num, J, op, P, sh, out);
 }
 
 }  // namespace
 
+void plan_line(const LineOp& op, LineJob& j) {
+    // two rows more than the line has: the last interior row's inputs then lie in the line's own
+    // segments
+    const int segs = op.periodic ? (op.m + LSEG - 1) / LSEG : (op.m + 2) / LSEG + 1;
+    const int extra = op.margin ? 2 * (op.margin / LSEG) : 0;
+    if (segs + (op.periodic ? extra : 0) <= LINE_THREADS) {
+        j.nseg = segs + (op.periodic ? extra : 0);
+        j.cstep = op.m;
+        j.nchunk = 1;
+    } else {
+        j.nseg = LINE_THREADS;
+        j.cstep = (LINE_THREADS - extra) * LSEG;
+        j.nchunk = (op.m + j.cstep - 1) / j.cstep;
+    }
+    j.nl = LINE_THREADS / j.nseg;
+    if (j.nl > LINE_MAX_LINES) j.nl = LINE_MAX_LINES;
+    j.inv_nl = (1 << 20) / j.nl + 1;
+    j.groups = (j.nlines + j.nl - 1) / j.nl;
+    j.blocks = j.groups * j.nchunk;
+}
+
 cudaError_t launch_lines(const LineJob* d_jobs, int njobs, int max_blocks, const double* U,
-                         cudaStream_t s, int mixed) {
+                         cudaStream_t s) {
     if (njobs == 0) return cudaSuccess;
-    dim3 block(LINE_BLOCK);
-    dim3 grid(max_blocks, njobs);
-    if (mixed) k_lines<true><<<grid, block, 0, s>>>(d_jobs, U);
-    else k_lines<false><<<grid, block, 0, s>>>(d_jobs, U);
+    k_lines<<<dim3(max_blocks, njobs), LINE_THREADS, 0, s>>>(d_jobs, U);
     return cudaGetLastError();
 }
 

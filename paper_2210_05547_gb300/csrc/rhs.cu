@@ -277,20 +277,13 @@ void lagrange(const double* nodes, int n, double x, bool deriv, double* w) {
 }
 
 // Build one operator: kind 0 interpolation / 1 derivative; dir 0 centre->face / 1 face->centre.
-LineOp make_op(int kind, int dir, int n, int wall, std::vector<double>& data) {
+// tails: receives the operator's LineTail; op.tail holds its index until the device array exists.
+LineOp make_op(int kind, int dir, int n, int wall, std::vector<LineTail>& tails) {
     LineOp op;
     memset(&op, 0, sizeof(op));
     op.kind = kind;
     op.dir = dir;
     op.wall = wall;
-    double alpha, a, b;
-    if (kind == 0) { alpha = 3.0 / 10.0; a = 3.0 / 2.0; b = 1.0 / 10.0; }
-    else { alpha = 9.0 / 62.0; a = 63.0 / 62.0; b = 17.0 / 62.0; }
-    if (kind == 0) {
-        op.wi[0] = b / 2.0; op.wi[1] = a / 2.0; op.wi[2] = a / 2.0; op.wi[3] = b / 2.0;
-    } else {
-        op.wi[0] = -b / 3.0; op.wi[1] = -a; op.wi[2] = a; op.wi[3] = b / 3.0;
-    }
     std::vector<double> in_pos, out_pos;
     if (dir == 0) {
         op.m = n + 1;
@@ -308,14 +301,8 @@ LineOp make_op(int kind, int dir, int n, int wall, std::vector<double>& data) {
         op.last_interior = n - 2;
     }
     const int m = op.m;
-    std::vector<double> lower(m, 0.0), upper(m, 0.0);
     for (int r = 0; r < m; ++r) {
-        const bool interior = r >= op.first_interior && r <= op.last_interior;
-        if (interior) {
-            if (r > 0) lower[r] = alpha;
-            if (r < m - 1) upper[r] = alpha;
-            continue;
-        }
+        if (r >= op.first_interior && r <= op.last_interior) continue;
         const int c = op.ncl++;
         op.crow[c] = r;
         const bool left = r < op.first_interior;
@@ -338,51 +325,28 @@ LineOp make_op(int kind, int dir, int n, int wall, std::vector<double>& data) {
             for (int k = 0; k < 5; ++k) op.cw[c][k] = w[k];
         }
     }
-    // Thomas factors of the unit-diagonal tridiagonal matrix
-    std::vector<double> cp(m), mi(m);
-    for (int r = 0; r < m; ++r) {
-        const double piv = 1.0 - (r > 0 ? lower[r] * cp[r - 1] : 0.0);
-        mi[r] = 1.0 / piv;
-        cp[r] = upper[r] * mi[r];
+    op.margin = m + 2 >= LINE_THREADS * LSEG ? LINE_TAIL : 0;   // cut into chunks (plan_line)
+    // rho / (1 + rho^2) = alpha = 3/10 (interpolation), 9/62 (derivative)
+    const long double rho = kind == 0 ? 1.0L / 3.0L : (31.0L - sqrtl(880.0L)) / 9.0L;
+    const int ni = op.last_interior - op.first_interior + 1;
+    LineTail tail;
+    memset(&tail, 0, sizeof(tail));
+    // |h_k| = rho^(k+1) (1 - rho^(2 (ni - k))) / (1 - rho^2), by products from the far end
+    long double up = rho, far = 1.0L, h0 = 0.0L;
+    for (int k = 0; k < ni && k < 1000; ++k) far *= rho * rho;   // rho^(2 ni), 0 for long lines
+    if (ni > 1000) far = 0.0L;
+    for (int k = 0; k < LINE_TAIL && k < ni; ++k) {
+        const long double h = (k & 1 ? 1.0L : -1.0L) * up * (1.0L - far) / (1.0L - rho * rho);
+        if (k == 0) h0 = h;
+        tail.h[k] = llrintl(ldexpl(h, 64));
+        tail.hd[k] = (double)h;
+        up *= rho;
+        far /= rho * rho;
     }
-    // interior weights folded with the pivot: d_r = wa_r (f1 +/- f0) + wb_r (f3 +/- f_-1) - lm_r d_{r-1}
-    std::vector<double> wa(m), wb(m), lm(m);
-    for (int r = 0; r < m; ++r) {
-        wa[r] = (kind == 0 ? op.wi[1] : op.wi[2]) * mi[r];
-        wb[r] = (kind == 0 ? op.wi[0] : op.wi[3]) * mi[r];
-        lm[r] = lower[r] * mi[r];
-    }
-    // first row of the constant tail of the interior factors
-    const int li = op.last_interior;
-    op.rc = li + 1;
-    if (li >= op.first_interior) {
-        int r = li;
-        while (r - 1 >= op.first_interior && wa[r - 1] == wa[li] && wb[r - 1] == wb[li] &&
-               lm[r - 1] == lm[li] && cp[r - 1] == cp[li])
-            --r;
-        op.rc = r;
-        op.wac = wa[li];
-        op.wbc = wb[li];
-        op.lmc = lm[li];
-        op.cpc = cp[li];
-        op.wac_f = (float)op.wac;
-        op.wbc_f = (float)op.wbc;
-        op.lmc_f = (float)op.lmc;
-        op.cpc_f = (float)op.cpc;
-        op.wac_l = (float)(op.wac - (double)op.wac_f);
-        op.wbc_l = (float)(op.wbc - (double)op.wbc_f);
-        op.lmc_l = (float)(op.lmc - (double)op.lmc_f);
-        op.cpc_l = (float)(op.cpc - (double)op.cpc_f);
-    }
-    // store offsets into data (fixed up to device pointers later)
-    const size_t base = data.size();
-    for (auto* v : {&lower, &cp, &mi, &wa, &wb, &lm}) data.insert(data.end(), v->begin(), v->end());
-    op.lower = (const double*)(base);
-    op.cprime = (const double*)(base + m);
-    op.minv = (const double*)(base + 2 * m);
-    op.wa = (const double*)(base + 3 * m);
-    op.wb = (const double*)(base + 4 * m);
-    op.lm = (const double*)(base + 5 * m);
+    tail.kappa = llrintl(ldexpl(1.0L / (1.0L - rho * h0), 63));
+    tail.kappa_d = (double)(1.0L / (1.0L - rho * h0));
+    op.tail = (const LineTail*)(size_t)tails.size();
+    tails.push_back(tail);
     return op;
 }
 
@@ -526,59 +490,29 @@ struct PlanBuilder {
             j.out_es = d.pitch(tout);
             j.nlines = d.pitch(tin);
         }
-        j.nseg = hops[op].m;   // line length for now; replaced by the segment count in finish()
         j.wall_value = wall_value;
         j.scale = scale;
         j.metric = metric;
+        plan_line(hops[op], j);
         jobs.push_back(j);
         out_size.push_back(d.size(tout));
         ph_count[cur]++;
+        ph_blocks[cur] = std::max(ph_blocks[cur], j.blocks);
     }
-    // the last job added feeds only diffusive fluxes: binary32 allowed under HYP_MIXED
-    void f32() { jobs.back().f32ok = 1; }
-    // Segment counts (at most 260 points per segment, more segments when a phase has too few
-    // threads to occupy the GPU), forward-sweep storage and block counts per phase. Returns the
-    // tmp doubles needed by the largest phase.
-    long long finish() {
-        long long need = 0;
-        long long face_need = 0;
-        for (int k = ph_start[PH_FACE]; k < ph_start[PH_FACE] + ph_count[PH_FACE]; ++k)
-            face_need += out_size[k];
+    // Sum of the output sizes of the largest phase (the phases that run beside the face phase
+    // counted with it): the size limit of hyp_rhs_noalloc counts this many doubles beside the
+    // scratch fields.
+    long long sweep_doubles() const {
+        long long need = 0, face = 0;
         for (int ph = 0; ph < PH_COUNT; ++ph) {
-            const int a = ph_start[ph], b = a + ph_count[ph];
-            std::vector<int> nseg(ph_count[ph]);
-            long long threads = 0;
-            for (int k = a; k < b; ++k) {
-                const int m = jobs[k].nseg;
-                int ns = 1;
-                while (ns < LINE_BLOCK / 2 && (m + ns - 1) / ns > 260) ns *= 2;
-                nseg[k - a] = ns;
-                threads += (long long)jobs[k].nlines * ns;
-            }
-            while (threads < 40960) {
-                bool grew = false;
-                threads = 0;
-                for (int k = a; k < b; ++k) {
-                    const int m = jobs[k].nseg;
-                    if (nseg[k - a] < LINE_BLOCK / 2 && (m + 2 * nseg[k - a] - 1) / (2 * nseg[k - a]) >= 32) {
-                        nseg[k - a] *= 2;
-                        grew = true;
-                    }
-                    threads += (long long)jobs[k].nlines * nseg[k - a];
-                }
-                if (!grew) break;
-            }
-            // phases that run beside the face phase on the second stream take storage past it
-            const bool beside_face = ph == PH_MU1 || ph == PH_MU2 || ph == PH_FACEB;
-            long long off = beside_face ? face_need : 0;
-            for (int k = a; k < b; ++k) {
-                jobs[k].nseg = nseg[k - a];
-                jobs[k].tmp = (double*)(size_t)off;   // relative; fixed up by the caller
-                off += out_size[k];
-                const int lpb = LINE_BLOCK / jobs[k].nseg;
-                ph_blocks[ph] = std::max(ph_blocks[ph], (jobs[k].nlines + lpb - 1) / lpb);
-            }
-            need = std::max(need, off);
+            long long n = 0;
+            for (int k = ph_start[ph]; k < ph_start[ph] + ph_count[ph]; ++k) n += out_size[k];
+            if (ph == PH_FACE) face = n;
+        }
+        for (int ph = 0; ph < PH_COUNT; ++ph) {
+            long long n = ph == PH_MU1 || ph == PH_MU2 || ph == PH_FACEB ? face : 0;
+            for (int k = ph_start[ph]; k < ph_start[ph] + ph_count[ph]; ++k) n += out_size[k];
+            need = std::max(need, n);
         }
         return need;
     }
@@ -659,8 +593,6 @@ static void free_grid(hyp_grid* G) {
     cudaFree(G->ops);
     cudaFree(G->opdata);
     cudaFree(G->jobs);
-    cudaFree(G->linetmp);
-    cudaFree(G->metf);
     free_streams(G);
     if (G->prof) {
         for (auto e : G->prof->ev) cudaEventDestroy(e);
@@ -855,7 +787,7 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
         return cuda_fail(err, "cudaMalloc(grid)");
     }
     // operators
-    std::vector<double> opdata;
+    std::vector<LineTail> opdata;
     std::vector<LineOp> hops(NOPS);
     hops[OX_ICF] = make_op(0, 0, nx, 0, opdata);
     hops[OX_DCF] = make_op(1, 0, nx, 0, opdata);
@@ -867,20 +799,13 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     hops[OY_DFC] = make_op(1, 1, ny, 0, opdata);
     hops[OY_ICFW] = make_op(0, 0, ny, 1, opdata);
     hops[OY_DCFW] = make_op(1, 0, ny, 1, opdata);
-    err = cudaMalloc(&G->opdata, opdata.size() * sizeof(double));
+    err = cudaMalloc(&G->opdata, opdata.size() * sizeof(LineTail));
     if (err == cudaSuccess) err = cudaMalloc(&G->ops, NOPS * sizeof(LineOp));
     if (err != cudaSuccess) {
         free_grid(G);
         return cuda_fail(err, "cudaMalloc(operators)");
     }
-    for (auto& op : hops) {
-        op.lower = G->opdata + (size_t)op.lower;
-        op.cprime = G->opdata + (size_t)op.cprime;
-        op.minv = G->opdata + (size_t)op.minv;
-        op.wa = G->opdata + (size_t)op.wa;
-        op.wb = G->opdata + (size_t)op.wb;
-        op.lm = G->opdata + (size_t)op.lm;
-    }
+    for (auto& op : hops) op.tail = G->opdata + (size_t)op.tail;
     // plans
     PlanBuilder B;
     B.G = G;
@@ -899,8 +824,6 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     B.add(OY_ICF, S.rho_xf, NXF, S.rho_cn, NCN, nullptr);
     B.add(OX_IFC, S.mux_f, NXF, S.mux_c, NC, nullptr);
     B.add(OY_IFC, S.mvy_f, NYF, S.mvy_c, NC, nullptr);
-    // (the velocity gradients feed the artificial-diffusivity sensors, whose fourth differences
-    // would amplify binary32 rounding: they stay FP64 in every mode)
     B.begin(PH_AD1);
     B.add(OY_IFC, S.dudy_cn, NCN, S.dudy_t, NXF, nullptr);
     B.add(OY_IFC, S.dvdx_cn, NCN, S.dvdx_t, NXF, nullptr);
@@ -909,61 +832,39 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     B.add(OX_IFC, S.dvdx_t, NXF, S.dvdx_c, NC, nullptr);
     B.begin(PH_MU1);
     B.add(OX_ICF, S.mu_e, NC, S.mu_xf, NXF, nullptr);
-    B.f32();
     B.begin(PH_MU2);
     B.add(OY_ICF, S.mu_xf, NXF, S.mu_cn, NCN, nullptr);
-    B.f32();
     B.begin(PH_FACE);
     for (int sp = 0; sp < NSP; ++sp) {
         B.add(OX_ICF, S.Y[sp], NC, S.Yx[sp], NXF, nullptr);
         B.add(OX_ICF, S.G[sp], NC, S.Gx[sp], NXF, nullptr);
-        B.f32();
-        B.add(OX_ICF, S.h[sp], NC, S.hx[sp], NXF, nullptr);
-        B.f32();
-        B.add(OX_DCF, S.X[sp], NC, S.dXdx[sp], NXF, G->xi_f);
-        B.f32();
-        B.add(OY_ICF, S.Y[sp], NC, S.Yy[sp], NYF, nullptr);
+            B.add(OX_ICF, S.h[sp], NC, S.hx[sp], NXF, nullptr);
+            B.add(OX_DCF, S.X[sp], NC, S.dXdx[sp], NXF, G->xi_f);
+            B.add(OY_ICF, S.Y[sp], NC, S.Yy[sp], NYF, nullptr);
         B.add(OY_ICF, S.G[sp], NC, S.Gy[sp], NYF, nullptr);
-        B.f32();
-        B.add(OY_ICF, S.h[sp], NC, S.hy[sp], NYF, nullptr);
-        B.f32();
-        B.add(OY_DCF, S.X[sp], NC, S.dXdy[sp], NYF, G->eta_f);
-        B.f32();
-    }
+            B.add(OY_ICF, S.h[sp], NC, S.hy[sp], NYF, nullptr);
+            B.add(OY_DCF, S.X[sp], NC, S.dXdy[sp], NYF, G->eta_f);
+        }
     B.add(OX_ICF, S.H, NC, S.Hx, NXF, nullptr);
     B.add(OX_ICF, S.K, NC, S.Kx, NXF, nullptr);
-    B.f32();
     B.add(OX_ICF, S.tau_xx, NC, S.txx_x, NXF, nullptr);
-    B.f32();
     B.add(OX_ICF, S.v_c, NC, S.v_x, NXF, nullptr);
-    B.f32();
     B.add(OX_DCF, S.T, NC, S.dTdx, NXF, G->xi_f);
-    B.f32();
     B.add(OY_ICF, S.H, NC, S.Hy, NYF, nullptr);
     B.add(OY_ICF, S.K, NC, S.Ky, NYF, nullptr);
-    B.f32();
     B.add(OY_ICF, S.tau_yy, NC, S.tyy_y, NYF, nullptr);
-    B.f32();
     B.add(y_icf_u, S.u_c, NC, S.u_y, NYF, nullptr, 1.0, 0.0);
-    B.f32();
     B.add(wall ? OY_DCFW : OY_DCF, S.T, NC, S.dTdy, NYF, G->eta_f, 1.0, G->Tw_nd);
-    B.f32();
     if (G->view().sm) {
         // face temperature and pressure for the binary coefficients of Eq. (17)
         B.add(OX_ICF, S.T, NC, S.Tx, NXF, nullptr);
-        B.f32();
-        B.add(OX_ICF, S.p, NC, S.px, NXF, nullptr);
-        B.f32();
-        B.add(OY_ICF, S.T, NC, S.Ty, NYF, nullptr);
-        B.f32();
-        B.add(OY_ICF, S.p, NC, S.py, NYF, nullptr);
-        B.f32();
-    }
+            B.add(OX_ICF, S.p, NC, S.px, NXF, nullptr);
+            B.add(OY_ICF, S.T, NC, S.Ty, NYF, nullptr);
+            B.add(OY_ICF, S.p, NC, S.py, NYF, nullptr);
+        }
     B.begin(PH_FACEB);
     B.add(OY_IFC, S.tau_xy, NCN, S.txy_x, NXF, nullptr);
-    B.f32();
     B.add(OX_IFC, S.tau_xy, NCN, S.txy_y, NYF, nullptr);
-    B.f32();
     B.begin(PH_DIV);
     for (int sp = 1; sp < NSP; ++sp) {
         B.add(OX_DFC, S.Fsx[sp], NXF, S.DX + G->off[sp], NC, G->xi_c, -1.0);
@@ -984,39 +885,21 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     B.add(OY_ICF, soff(0), NC, S.rho_yf, NYF, nullptr, 1.0, 0.0, 1);
     B.add(OX_DFC, soff(NSP + 1), NXF, S.DX + G->off[0], NC, G->xi_c, -1.0, 0.0, 1);
     B.add(OY_DFC, soff(NSP + 2), NYF, S.DY + G->off[0], NC, G->eta_c, -1.0, 0.0, 1);
-    const long long tmp_need = B.finish();
+    G->linetmp_n = B.sweep_doubles();
     memcpy(G->ph_start, B.ph_start, sizeof(B.ph_start));
     memcpy(G->ph_count, B.ph_count, sizeof(B.ph_count));
     memcpy(G->ph_blocks, B.ph_blocks, sizeof(B.ph_blocks));
-    G->linetmp_n = tmp_need;
-    err = cudaMalloc(&G->linetmp, tmp_need * sizeof(double));
-    if (err == cudaSuccess) err = cudaMalloc(&G->jobs, B.jobs.size() * sizeof(LineJob));
+    err = cudaMalloc(&G->jobs, B.jobs.size() * sizeof(LineJob));
     if (err != cudaSuccess) {
         free_grid(G);
         return cuda_fail(err, "cudaMalloc(jobs)");
     }
-    if (err == cudaSuccess) err = cudaMalloc(&G->metf, (2 * (nx + ny) + 2) * sizeof(float));
-    if (err != cudaSuccess) {
-        free_grid(G);
-        return cuda_fail(err, "cudaMalloc(metrics)");
-    }
-    std::vector<float> metf_h;
-    for (const auto* v : {&xi_c, &xi_f, &eta_c, &eta_f})
-        for (double x : *v) metf_h.push_back((float)x);
-    const double* met_d[4] = {G->xi_c, G->xi_f, G->eta_c, G->eta_f};
-    const long long met_off[4] = {0, nx, 2LL * nx + 1, 2LL * nx + 1 + ny};
-    for (auto& j : B.jobs) {
-        j.tmp = G->linetmp + (size_t)j.tmp;
-        for (int k = 0; k < 4; ++k)
-            if (j.metric == met_d[k]) j.metric_f = G->metf + met_off[k];
-    }
     // uploads
 #define UP(dst, src, bytes) HYP_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s))
-    UP(G->opdata, opdata.data(), opdata.size() * sizeof(double));
+    UP(G->opdata, opdata.data(), opdata.size() * sizeof(LineTail));
     UP(G->ops, hops.data(), NOPS * sizeof(LineOp));
     UP(G->jobs, B.jobs.data(), B.jobs.size() * sizeof(LineJob));
     G->hjobs = B.jobs;
-    UP(G->metf, metf_h.data(), metf_h.size() * sizeof(float));
     UP(G->xi_c, xi_c.data(), nx * sizeof(double));
     UP(G->xi_f, xi_f.data(), (nx + 1) * sizeof(double));
     UP(G->eta_c, eta_c.data(), ny * sizeof(double));
@@ -1110,9 +993,8 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     const long long nc = d.size(NC);
     cudaError_t e1 = cudaSuccess;
     const bool mixed = precision == HYP_MIXED;
-    const int mx = mixed ? 1 : 0;
     TIMED(KID_LINES_STATE, e1 = launch_lines(G->jobs + G->ph_start[PH_P1], G->ph_count[PH_P1],
-                                             G->ph_blocks[PH_P1], U, s, mx));
+                                             G->ph_blocks[PH_P1], U, s));
     HYP_CUDA(e1);
     TIMED(KID_FACE_VEL, (k_face_vel<<<blocks_for(d.size(NXF) + d.size(NYF), 256), 256, 0, s>>>(v, U, S)));
     // fork: velocity gradients and the artificial-diffusivity line phases do not need the closure
@@ -1126,15 +1008,12 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     HYP_CUDA(cudaGetLastError());
     G->cache_valid = 1;
     TIMED_ON(s2, KID_LINES_VELGRAD, e1 = launch_lines(G->jobs + G->ph_start[PH_P3], G->ph_count[PH_P3],
-                                                      G->ph_blocks[PH_P3], U, s2, mx));
+                                                      G->ph_blocks[PH_P3], U, s2));
     HYP_CUDA(e1);
     if (v.ad) {
-        // the two small interpolation phases of the sensors' cross derivatives run in binary64 in
-        // both precisions: with two jobs their lines cannot fill the GPU, and at that occupancy the
-        // binary64 recurrence (one FMA per row on its chain) beats the double-word one
-        TIMED_ON(s2, KID_LINES_AD, e1 = launch_lines(G->jobs + G->ph_start[PH_AD1], 2, G->ph_blocks[PH_AD1], U, s2, 0));
+        TIMED_ON(s2, KID_LINES_AD, e1 = launch_lines(G->jobs + G->ph_start[PH_AD1], 2, G->ph_blocks[PH_AD1], U, s2));
         HYP_CUDA(e1);
-        TIMED_ON(s2, KID_LINES_AD, e1 = launch_lines(G->jobs + G->ph_start[PH_AD2], 2, G->ph_blocks[PH_AD2], U, s2, 0));
+        TIMED_ON(s2, KID_LINES_AD, e1 = launch_lines(G->jobs + G->ph_start[PH_AD2], 2, G->ph_blocks[PH_AD2], U, s2));
         HYP_CUDA(e1);
         TIMED_ON(s2, KID_AD_PREP, (k_ad_prep<<<blocks_for(nc, 256), 256, 0, s2>>>(v, S)));
     }
@@ -1157,17 +1036,17 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     // fork: viscosity to the corners, shear stress and its face interpolants beside the face phase
     HYP_CUDA(cudaEventRecord(G->fork[1], s));
     HYP_CUDA(cudaStreamWaitEvent(s2, G->fork[1], 0));
-    TIMED_ON(s2, KID_LINES_MU, e1 = launch_lines(G->jobs + G->ph_start[PH_MU1], 1, G->ph_blocks[PH_MU1], U, s2, mx));
+    TIMED_ON(s2, KID_LINES_MU, e1 = launch_lines(G->jobs + G->ph_start[PH_MU1], 1, G->ph_blocks[PH_MU1], U, s2));
     HYP_CUDA(e1);
-    TIMED_ON(s2, KID_LINES_MU, e1 = launch_lines(G->jobs + G->ph_start[PH_MU2], 1, G->ph_blocks[PH_MU2], U, s2, mx));
+    TIMED_ON(s2, KID_LINES_MU, e1 = launch_lines(G->jobs + G->ph_start[PH_MU2], 1, G->ph_blocks[PH_MU2], U, s2));
     HYP_CUDA(e1);
     TIMED_ON(s2, KID_STRESS_CN, (k_stress_cn<<<blocks_for(d.size(NCN), 256), 256, 0, s2>>>(v, S)));
     TIMED_ON(s2, KID_LINES_FACE, e1 = launch_lines(G->jobs + G->ph_start[PH_FACEB], G->ph_count[PH_FACEB],
-                                                   G->ph_blocks[PH_FACEB], U, s2, mx));
+                                                   G->ph_blocks[PH_FACEB], U, s2));
     HYP_CUDA(e1);
     HYP_CUDA(cudaEventRecord(G->join[1], s2));
     TIMED(KID_LINES_FACE, e1 = launch_lines(G->jobs + G->ph_start[PH_FACE], G->ph_count[PH_FACE],
-                                            G->ph_blocks[PH_FACE], U, s, mx));
+                                            G->ph_blocks[PH_FACE], U, s));
     HYP_CUDA(e1);
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[1], 0));
     if (v.sm) {
@@ -1178,7 +1057,7 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
         TIMED(KID_FLUX, (k_flux<false><<<blocks_for(d.size(NYF), 128), 128, 0, s>>>(g, sc, v, U, S, 1)));
     }
     TIMED(KID_LINES_DIV, e1 = launch_lines(G->jobs + G->ph_start[PH_DIV], G->ph_count[PH_DIV],
-                                           G->ph_blocks[PH_DIV], U, s, mx));
+                                           G->ph_blocks[PH_DIV], U, s));
     HYP_CUDA(e1);
     const AssembleArgs aa{S.DX, S.DY, S.SRC, G->sigma, G->Uref, G->mask,
                           rk ? Urk : (double*)U, dUdt, dQ, rk, A, Bc, dt};
@@ -1408,22 +1287,19 @@ static __device__ __align__(256) double g_noalloc_scratch[HYP_NOALLOC_DOUBLES];
 static double* g_noalloc_base[HYP_NOALLOC_MAX_DEVICES];
 static std::mutex g_noalloc_mutex;
 
-// Copy of a launch plan whose field pointers into the grid's scratch pool or line-sweep storage
-// are moved to the same offsets in the static array (one thread per job).
+// Copy of a launch plan whose field pointers into the grid's scratch pool are moved to the same
+// offsets in the static array (one thread per job).
 __global__ void k_relocate_jobs(const LineJob* __restrict__ src, LineJob* __restrict__ dst, int n,
-                                const double* pool, long long pool_n, const double* linetmp,
-                                long long linetmp_n, double* base, double* tmp_base) {
+                                const double* pool, long long pool_n, double* base) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     auto relocate = [&](const double* p) -> double* {
         if (p >= pool && p < pool + pool_n) return base + (p - pool);
-        if (p >= linetmp && p < linetmp + linetmp_n) return tmp_base + (p - linetmp);
         return const_cast<double*>(p);
     };
     LineJob j = src[k];
     if (!j.in_state) j.in = relocate(j.in);
     j.out = relocate(j.out);
-    j.tmp = relocate(j.tmp);
     dst[k] = j;
 }
 
@@ -1463,24 +1339,22 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
     double* base = nullptr;
     int rc = noalloc_base(&base);
     if (rc) return rc;
-    double* tmp_base = base + scratch_n;
     LineJob* djobs = (LineJob*)(base + scratch_n + G->linetmp_n);
     auto relocate = [&](const double* p) -> double* {
         if (p >= G->pool && p < G->pool + scratch_n) return base + (p - G->pool);
-        if (p >= G->linetmp && p < G->linetmp + G->linetmp_n) return tmp_base + (p - G->linetmp);
         return const_cast<double*>(p);
     };
     // the grid's launch plan, copied on the device with its scratch pointers moved into the
     // static array (no host buffer, no synchronisation)
     k_relocate_jobs<<<blocks_for(njobs, 64), 64, 0, s>>>(G->jobs, djobs, njobs, G->pool, scratch_n,
-                                                         G->linetmp, G->linetmp_n, base, tmp_base);
+                                                         base);
     HYP_CUDA(cudaGetLastError());
     Scratch S = G->s;
     double** fields = reinterpret_cast<double**>(&S);
     for (size_t k = 0; k < sizeof(Scratch) / sizeof(double*); ++k) fields[k] = relocate(fields[k]);
     // every call starts from cleared scratch, as a newly built grid does (the array keeps the last
     // call's contents, possibly of another grid); the Newton iteration starts at 1000 K
-    HYP_CUDA(cudaMemsetAsync(base, 0, (scratch_n + G->linetmp_n) * sizeof(double), s));
+    HYP_CUDA(cudaMemsetAsync(base, 0, scratch_n * sizeof(double), s));
     const long long nc = G->d.size(NC);
     k_fill<<<blocks_for(nc, 256), 256, 0, s>>>(S.Tcache, nc, 1000.0);
     HYP_CUDA(cudaGetLastError());

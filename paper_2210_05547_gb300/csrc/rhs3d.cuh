@@ -14,12 +14,8 @@
 // artificial-diffusivity sensors (fourth differences and Gaussian filter periodic in z), stresses
 // at centres and edges, species and energy fluxes on the three face families, divergences in
 // three directions. Lines along x and y run through the segmented line kernel of the
-// two-dimensional path (lines.cu; lines along y grouped by z-plane); lines along z are periodic:
-// every row is interior, so the forward and backward recurrences run with the operator's
-// constant factors around the ring, one thread per line, started W rows early from zero (W = 40
-// for the interpolation, factor 1/3, and 26 for the derivative, factor 0.148: the dropped history
-// is below 1e-19 of the values, and the result is the periodic solution to rounding). Each phase
-// batches up to eight independent line jobs of one kind per launch; the velocity-gradient and
+// two-dimensional path (lines.cu; lines along y grouped by z-plane); lines along z are periodic
+// (every row interior) and go through it too. Each phase is one launch; the velocity-gradient and
 // artificial-diffusivity phases run on a second stream beside the closure, and the viscosity
 // phase, the stresses and their face values there beside the other face values.
 //
@@ -40,150 +36,21 @@ struct Sh3 {
     __host__ __device__ long long size(int t) const { return plane(t) * nz; }
 };
 
-// One batched line operation over a 3-D array.
+// One line operation over a 3-D array.
 struct Line3 {
-    const LineOp* op;          // x or y operator (device); unused along z
+    int op;                    // operator (Grid3::ops)
     int axis, tin, tout;       // 0 x, 1 y, 2 z; array shapes of input and output
     const double* in;
     double* out;
     const double* metric;      // x, y: per output point along the line (nullable)
     double scale;              // z lines: includes the metric zeta
-    double wall;               // y lines with a wall operator: wall value, or per line:
-    const double* wall_arr;    //   wall value of line (k, i) at k * nx + i
-    int kind, dir;             // z lines: 0 interpolation / 1 derivative; 0 c->f / 1 f->c
-    double wa, wb, lm, cp;     // z lines: the operator's constant factors
-    int job;                   // x, y lines: index of the segmented line job (Grid3::jobs)
-    int f32;                   // feeds only diffusive fluxes: binary32 rows under HYP_MIXED
+    const double* wall_arr;    // y lines with a wall operator, nullable: wall value of line (k, i)
+                               // at k * nx + i (else 0)
 };
 
-
-__device__ __forceinline__ double row3(int kind, double p0, double p1, double p2, double p3,
-                                       double wa, double wb, double lm, double d) {
-    if (kind == 0) return fma(-lm, d, fma(wa, p1 + p2, wb * (p0 + p3)));
-    return fma(-lm, d, fma(wa, p2 - p1, wb * (p3 - p0)));
-}
-
-// Periodic lines along z: one thread per line, one job of the batch per blockIdx.y. The four
-// stencil values slide through registers and the plane index wraps with a counter (one load per
-// row, no integer division in the loop).
-constexpr int BATCH3 = 8;      // line jobs per launch (x/y jobs: forward-sweep slots)
-struct ZBatch {
-    Line3 L[BATCH3];
-};
-
-struct ZRing {
-    int n, W3, r0, b0;         // period, warm-up rows, first stencil row, first warm-up back row
-    long long plane;
-    __device__ ZRing(const Line3& L, const Sh3& sh) {
-        plane = sh.plane(L.tin);
-        n = sh.nz;
-        W3 = L.kind == 0 ? 40 : 26;   // as the segmented solver: dropped history < 1e-19
-        const int o = L.dir == 0 ? 2 : 1;          // first stencil row of output row t: t - o
-        r0 = ((-W3 - o) % n + n) % n;
-        b0 = (n - 1 + W3) % n;
-    }
-};
-
-__device__ __forceinline__ void zline64(const Line3& L, const ZRing& z,
-                                        const double* __restrict__ in, double* __restrict__ out) {
-    const long long plane = z.plane;
-    const int n = z.n, W3 = z.W3;
-    int r = z.r0;
-    auto next = [&]() {
-        const double v = in[(long long)r * plane];
-        r = r + 1 == n ? 0 : r + 1;
-        return v;
-    };
-    double p0 = next(), p1 = next(), p2 = next();
-    double d = 0.0;
-    for (int t = -W3; t < 0; ++t) {      // warm-up: rows n - W3 .. n - 1 of the period
-        const double p3 = next();
-        d = row3(L.kind, p0, p1, p2, p3, L.wa, L.wb, L.lm, d);
-        p0 = p1;
-        p1 = p2;
-        p2 = p3;
-    }
-    for (int t = 0; t < n; ++t) {
-        const double p3 = next();
-        d = row3(L.kind, p0, p1, p2, p3, L.wa, L.wb, L.lm, d);
-        out[(long long)t * plane] = d;
-        p0 = p1;
-        p1 = p2;
-        p2 = p3;
-    }
-    // back substitution: warm-up over rows W3 - 1 .. 0 of the next period, then the period
-    int b = z.b0;
-    double y = out[(long long)b * plane];
-    for (int k = 1; k < W3; ++k) {
-        b = b == 0 ? n - 1 : b - 1;
-        y = out[(long long)b * plane] - L.cp * y;
-    }
-    for (int t = n - 1; t >= 0; --t) {
-        y = out[(long long)t * plane] - L.cp * y;
-        out[(long long)t * plane] = L.scale * y;
-    }
-}
-
-__device__ __forceinline__ float* zslot(double* p) { return reinterpret_cast<float*>(p); }
-
-// The same in binary32 (HYP_MIXED, lines feeding only diffusive fluxes): inputs rounded with the
-// integer conversions of fp32.cuh, forward values kept as binary32 in the first half of their
-// output slot, outputs widened back to binary64.
-__device__ __forceinline__ void zline32(const Line3& L, const ZRing& z,
-                                        const double* __restrict__ in, double* __restrict__ out) {
-    const long long plane = z.plane;
-    const int n = z.n, W3 = z.W3;
-    const float wa = f32_of(L.wa), wb = f32_of(L.wb), lm = f32_of(L.lm), cp = f32_of(L.cp),
-                sc = f32_of(L.scale);
-    auto row = [&](float p0, float p1, float p2, float p3, float d) {
-        if (L.kind == 0) return fmaf(-lm, d, fmaf(wa, p1 + p2, wb * (p0 + p3)));
-        return fmaf(-lm, d, fmaf(wa, p2 - p1, wb * (p3 - p0)));
-    };
-    int r = z.r0;
-    auto next = [&]() {
-        const float v = f32_of(in[(long long)r * plane]);
-        r = r + 1 == n ? 0 : r + 1;
-        return v;
-    };
-    float p0 = next(), p1 = next(), p2 = next();
-    float d = 0.0f;
-    for (int t = -W3; t < 0; ++t) {
-        const float p3 = next();
-        d = row(p0, p1, p2, p3, d);
-        p0 = p1;
-        p1 = p2;
-        p2 = p3;
-    }
-    for (int t = 0; t < n; ++t) {
-        const float p3 = next();
-        d = row(p0, p1, p2, p3, d);
-        *zslot(out + (long long)t * plane) = d;
-        p0 = p1;
-        p1 = p2;
-        p2 = p3;
-    }
-    int b = z.b0;
-    float y = *zslot(out + (long long)b * plane);
-    for (int k = 1; k < W3; ++k) {
-        b = b == 0 ? n - 1 : b - 1;
-        y = fmaf(-cp, y, *zslot(out + (long long)b * plane));
-    }
-    for (int t = n - 1; t >= 0; --t) {
-        y = fmaf(-cp, y, *zslot(out + (long long)t * plane));
-        out[(long long)t * plane] = f64_of(sc * y);
-    }
-}
-
-__global__ void __launch_bounds__(128) k_line3z(ZBatch B, Sh3 sh, int mixed) {
-    const Line3& L = B.L[blockIdx.y];
-    const ZRing z(L, sh);
-    const bool f32 = mixed && L.f32;      // uniform per block
-    for (long long line = blockIdx.x * (long long)blockDim.x + threadIdx.x; line < z.plane;
-         line += (long long)gridDim.x * blockDim.x) {
-        if (f32) zline32(L, z, L.in + line, L.out + line);
-        else zline64(L, z, L.in + line, L.out + line);
-    }
-}
+// Operators of a three-dimensional grid: the x and y ones of two dimensions, then the periodic z
+// ones [kind][dir].
+constexpr int OZ = NOPS, NOPS3 = NOPS + 4;
 
 struct Grid3 {
     Sh3 sh;
@@ -217,33 +84,26 @@ struct Grid3 {
     double *Uref, *sigma;
     uint8_t* mask;
     double *xi_c, *xi_f, *eta_c, *eta_f, *Tw;
-    float* metf;               // binary32 copies of xi_c, xi_f, eta_c, eta_f (HYP_MIXED line jobs)
     LineOp* ops;
-    double* opdata;
-    Line3 zop[2][2];           // periodic z operators [kind][dir] (constants only)
-    struct Plan3* plan;        // host: the line jobs of each phase
-    LineJob* jobs;             // device: the x and y lines as segmented line jobs (lines.cu)
-    double* ltmp;              // their forward-sweep storage (jobs run one after another)
+    LineTail* opdata;
+    struct Plan3* plan;        // host: the launches of each phase
+    LineJob* jobs;             // device: their line jobs (lines.cu)
 };
 
-// One launch of a phase: up to BATCH3 consecutive entries of its line list, all periodic z lines
-// (k_line3z) or all x/y line jobs (k_lines, contiguous in Grid3::jobs).
+// One launch of a phase: consecutive entries of Grid3::jobs, `blocks` the most of any.
 struct Launch3 {
-    int z;
-    int first, count;
-    int blocks;                // x/y: blocks per job, the largest of the batch
+    int first, count, blocks;
 };
 
 struct Phase3 {
     std::vector<Line3> lines;
     std::vector<Launch3> launches;
-    int slot_base = 0;         // first forward-sweep buffer of its x/y jobs
 };
 
 // face: the face values that do not need the stresses; faceb: the stresses' face values, which
-// run with mu on the second stream beside face (so their x/y jobs take other sweep buffers)
+// run with mu and mu2 on the second stream beside face
 struct Plan3 {
-    Phase3 p1, p3, ad1, ad2, mu, face, faceb, divs;
+    Phase3 p1, p3, ad1, ad2, mu, mu2, face, faceb, divs;
 };
 
 struct View3 {
@@ -700,8 +560,6 @@ void free_grid3(Grid3* g) {
     if (!g) return;
     delete g->plan;
     cudaFree(g->jobs);
-    cudaFree(g->ltmp);
-    cudaFree(g->metf);
     cudaFree(g->pool);
     cudaFree(g->mask);
     cudaFree(g->ops);
@@ -727,27 +585,10 @@ View3 view3(const hyp_grid* G, const Grid3* g) {
     return v;
 }
 
-// The launches of one phase in order; `state`: the z lines' `in` is an element offset into U (the
-// x and y jobs resolve theirs in the line kernel).
-int launch3(const Grid3* g, const Phase3& ph, const double* U, bool state, int mixed,
-            cudaStream_t s) {
-    for (const Launch3& b : ph.launches) {
-        if (b.z) {
-            ZBatch zb;
-            memset(&zb, 0, sizeof(zb));
-            long long n = 0;
-            for (int i = 0; i < b.count; ++i) {
-                zb.L[i] = ph.lines[b.first + i];
-                if (state) zb.L[i].in = U + (size_t)zb.L[i].in;
-                n = std::max(n, g->sh.plane(zb.L[i].tin));
-            }
-            const int bx = (int)std::min<long long>((n + 127) / 128, 152LL * 64);
-            k_line3z<<<dim3(bx, b.count), 128, 0, s>>>(zb, g->sh, mixed);
-        } else {
-            HYP_CUDA(launch_lines(g->jobs + ph.lines[b.first].job, b.count, b.blocks, U, s, mixed));
-        }
-    }
-    HYP_CUDA(cudaGetLastError());
+// The launches of one phase.
+int launch3(const Grid3* g, const Phase3& ph, const double* U, cudaStream_t s) {
+    for (const Launch3& b : ph.launches)
+        HYP_CUDA(launch_lines(g->jobs + b.first, b.count, b.blocks, U, s));
     return HYP_OK;
 }
 
@@ -760,7 +601,7 @@ int run_rhs3(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUdt, int
     const GasDev& gd = gas->dev;
     const Plan3& pl = *g->plan;
     const int mx = precision == HYP_MIXED ? 1 : 0;
-    int rc = launch3(g, pl.p1, U, true, mx, s);
+    int rc = launch3(g, pl.p1, U, s);
     if (rc) return rc;
     k_fv3<<<blocks3(g->nxf + g->nyf + g->nc), 256, 0, s>>>(*g, v, U);
     // fork: velocity gradients and the artificial-diffusivity line phases do not need the closure
@@ -774,10 +615,10 @@ int run_rhs3(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUdt, int
     prof_end(G, slot, s);
     HYP_CUDA(cudaGetLastError());
     g->cache_valid = 1;
-    if ((rc = launch3(g, pl.p3, U, false, mx, s2))) return rc;
+    if ((rc = launch3(g, pl.p3, U, s2))) return rc;
     if (v.ad) {
-        if ((rc = launch3(g, pl.ad1, U, false, mx, s2))) return rc;
-        if ((rc = launch3(g, pl.ad2, U, false, mx, s2))) return rc;
+        if ((rc = launch3(g, pl.ad1, U, s2))) return rc;
+        if ((rc = launch3(g, pl.ad2, U, s2))) return rc;
         k_adprep3<<<blocks3(g->nc), 256, 0, s2>>>(*g);
         HYP_CUDA(cudaGetLastError());
     }
@@ -796,16 +637,17 @@ int run_rhs3(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUdt, int
     // face values
     HYP_CUDA(cudaEventRecord(G->fork[1], s));
     HYP_CUDA(cudaStreamWaitEvent(s2, G->fork[1], 0));
-    if ((rc = launch3(g, pl.mu, U, false, mx, s2))) return rc;
+    if ((rc = launch3(g, pl.mu, U, s2))) return rc;
+    if ((rc = launch3(g, pl.mu2, U, s2))) return rc;
     k_stress3<<<blocks3(g->nc + g->nxy + g->nxf + g->nyf), 256, 0, s2>>>(*g);
     HYP_CUDA(cudaGetLastError());
-    if ((rc = launch3(g, pl.faceb, U, false, mx, s2))) return rc;
+    if ((rc = launch3(g, pl.faceb, U, s2))) return rc;
     HYP_CUDA(cudaEventRecord(G->join[1], s2));
-    if ((rc = launch3(g, pl.face, U, false, mx, s))) return rc;
+    if ((rc = launch3(g, pl.face, U, s))) return rc;
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[1], 0));
     k_flux3<<<blocks3(g->nxf + g->nyf + g->nc), 128, 0, s>>>(gd, *g, v, U);
     HYP_CUDA(cudaGetLastError());
-    if ((rc = launch3(g, pl.divs, U, false, mx, s))) return rc;
+    if ((rc = launch3(g, pl.divs, U, s))) return rc;
     Assemble3 a;
     a.DX = g->DX;
     a.DY = g->DY;
@@ -936,8 +778,8 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
         return fail(HYP_ERR_ARG, "internal: 3-D scratch pool too small");
     }
     // ---------------- operators ----------------
-    std::vector<double> opdata;
-    std::vector<LineOp> hops(NOPS);
+    std::vector<LineTail> opdata;
+    std::vector<LineOp> hops(NOPS3);
     hops[OX_ICF] = make_op(0, 0, nx, 0, opdata);
     hops[OX_DCF] = make_op(1, 0, nx, 0, opdata);
     hops[OX_IFC] = make_op(0, 1, nx, 0, opdata);
@@ -948,41 +790,26 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
     hops[OY_DFC] = make_op(1, 1, ny, 0, opdata);
     hops[OY_ICFW] = make_op(0, 0, ny, 1, opdata);
     hops[OY_DCFW] = make_op(1, 0, ny, 1, opdata);
-    err = cudaMalloc(&g->opdata, opdata.size() * sizeof(double));
-    if (err == cudaSuccess) err = cudaMalloc(&g->ops, NOPS * sizeof(LineOp));
+    err = cudaMalloc(&g->opdata, opdata.size() * sizeof(LineTail));
+    if (err == cudaSuccess) err = cudaMalloc(&g->ops, NOPS3 * sizeof(LineOp));
     if (err != cudaSuccess) {
         free_grid3(g);
         G->g3 = nullptr;
         return cuda_fail(err, "cudaMalloc(3-D operators)");
     }
-    for (auto& op : hops) {
-        op.lower = g->opdata + (size_t)op.lower;
-        op.cprime = g->opdata + (size_t)op.cprime;
-        op.minv = g->opdata + (size_t)op.minv;
-        op.wa = g->opdata + (size_t)op.wa;
-        op.wb = g->opdata + (size_t)op.wb;
-        op.lm = g->opdata + (size_t)op.lm;
-    }
-    // periodic z operators: the fixed point of the Thomas recurrence of (alpha, 1, alpha)
+    for (int k = 0; k < NOPS; ++k) hops[k].tail = g->opdata + (size_t)hops[k].tail;
+    // periodic z operators: every row interior
     for (int kind = 0; kind < 2; ++kind)
         for (int dir = 0; dir < 2; ++dir) {
-            const double alpha = kind == 0 ? 3.0 / 10.0 : 9.0 / 62.0;
-            const double wa0 = kind == 0 ? 3.0 / 4.0 : 63.0 / 62.0;          // a/2 or a
-            const double wb0 = kind == 0 ? 1.0 / 20.0 : 17.0 / 62.0 / 3.0;   // b/2 or b/3
-            double cp = 0.0, mi = 1.0;
-            for (int it = 0; it < 400; ++it) {
-                mi = 1.0 / (1.0 - alpha * cp);
-                cp = alpha * mi;
-            }
-            Line3& L = g->zop[kind][dir];
-            memset(&L, 0, sizeof(L));
-            L.axis = 2;
-            L.kind = kind;
-            L.dir = dir;
-            L.wa = wa0 * mi;
-            L.wb = wb0 * mi;
-            L.lm = alpha * mi;
-            L.cp = cp;
+            LineOp& op = hops[OZ + 2 * kind + dir];
+            memset(&op, 0, sizeof(op));
+            op.m = op.n_in = nz;
+            op.kind = kind;
+            op.dir = dir;
+            op.periodic = 1;
+            op.margin = nz % LSEG || nz > LINE_THREADS * LSEG ? LINE_TAIL : 0;
+            op.first_interior = -(1 << 28);
+            op.last_interior = 1 << 28;
         }
     // ---------------- host geometry ----------------
     std::vector<double> xc(nx), xf(nx + 1), yc(ny), yf(ny + 1), xi_c(nx), xi_f(nx + 1), eta_c(ny),
@@ -1058,7 +885,7 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
     auto xy = [&](int opid, int axis, const double* in, int tin, double* out, int tout,
                   const double* metric, double scale = 1.0, const double* wall_arr = nullptr) {
         Line3 L = base;
-        L.op = g->ops + opid;
+        L.op = opid;
         L.axis = axis;
         L.in = in;
         L.tin = tin;
@@ -1066,12 +893,13 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
         L.tout = tout;
         L.metric = metric;
         L.scale = scale;
-        L.wall = 0.0;
         L.wall_arr = wall_arr;
         return L;
     };
     auto zl = [&](int kind, int dir, const double* in, int t, double* out, double scale = 1.0) {
-        Line3 L = g->zop[kind][dir];
+        Line3 L = base;
+        L.op = OZ + 2 * kind + dir;
+        L.axis = 2;
         L.in = in;
         L.tin = L.tout = t;
         L.out = out;
@@ -1125,59 +953,51 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
               zl(0, 1, g->tc[1], C3, g->dwdx_c),
               zl(0, 1, g->tc[2], C3, g->dvdz_c),
               zl(0, 1, g->tc[3], C3, g->dwdy_c)};
-    // under HYP_MIXED the jobs feeding only the diffusive fluxes (viscosities, diffusion and
-    // conduction coefficients, gradients of X_s and T, stresses, the velocities of the viscous
-    // work) run their rows in binary32; those feeding the convective fluxes stay FP64
-    auto f = [](Line3 L) {
-        L.f32 = 1;
-        return L;
-    };
-    pl.mu.lines = {f(xy(OX_ICF, 0, g->mu_e, C3, g->mu_xf, XF3, nullptr)),
-                   f(xy(OY_ICF, 1, g->mu_e, C3, g->mu_yf, YF3, nullptr))};
-    // edge viscosities from the face ones (the jobs of a list run in order on one stream)
-    pl.mu.lines.push_back(f(zl(0, 0, g->mu_xf, XF3, g->mu_xz)));
-    pl.mu.lines.push_back(f(zl(0, 0, g->mu_yf, YF3, g->mu_yz)));
-    pl.mu.lines.push_back(f(xy(OY_ICF, 1, g->mu_xf, XF3, g->mu_xy, XY3, nullptr)));
+    pl.mu.lines = {xy(OX_ICF, 0, g->mu_e, C3, g->mu_xf, XF3, nullptr),
+                   xy(OY_ICF, 1, g->mu_e, C3, g->mu_yf, YF3, nullptr)};
+    // edge viscosities from the face ones
+    pl.mu2.lines = {zl(0, 0, g->mu_xf, XF3, g->mu_xz), zl(0, 0, g->mu_yf, YF3, g->mu_yz),
+                    xy(OY_ICF, 1, g->mu_xf, XF3, g->mu_xy, XY3, nullptr)};
     std::vector<Line3>& F = pl.face.lines;
     std::vector<Line3>& FB = pl.faceb.lines;
     for (int sp = 0; sp < NSP; ++sp) {
         F.push_back(xy(OX_ICF, 0, g->Y[sp], C3, g->Yx[sp], XF3, nullptr));
-        F.push_back(f(xy(OX_ICF, 0, g->G[sp], C3, g->Gx[sp], XF3, nullptr)));
-        F.push_back(f(xy(OX_ICF, 0, g->h[sp], C3, g->hx[sp], XF3, nullptr)));
-        F.push_back(f(xy(OX_DCF, 0, g->X[sp], C3, g->dXdx[sp], XF3, g->xi_f)));
+        F.push_back(xy(OX_ICF, 0, g->G[sp], C3, g->Gx[sp], XF3, nullptr));
+        F.push_back(xy(OX_ICF, 0, g->h[sp], C3, g->hx[sp], XF3, nullptr));
+        F.push_back(xy(OX_DCF, 0, g->X[sp], C3, g->dXdx[sp], XF3, g->xi_f));
         F.push_back(xy(OY_ICF, 1, g->Y[sp], C3, g->Yy[sp], YF3, nullptr));
-        F.push_back(f(xy(OY_ICF, 1, g->G[sp], C3, g->Gy[sp], YF3, nullptr)));
-        F.push_back(f(xy(OY_ICF, 1, g->h[sp], C3, g->hy[sp], YF3, nullptr)));
-        F.push_back(f(xy(OY_DCF, 1, g->X[sp], C3, g->dXdy[sp], YF3, g->eta_f)));
+        F.push_back(xy(OY_ICF, 1, g->G[sp], C3, g->Gy[sp], YF3, nullptr));
+        F.push_back(xy(OY_ICF, 1, g->h[sp], C3, g->hy[sp], YF3, nullptr));
+        F.push_back(xy(OY_DCF, 1, g->X[sp], C3, g->dXdy[sp], YF3, g->eta_f));
         F.push_back(zl(0, 0, g->Y[sp], C3, g->Yz[sp]));
-        F.push_back(f(zl(0, 0, g->G[sp], C3, g->Gz[sp])));
-        F.push_back(f(zl(0, 0, g->h[sp], C3, g->hz[sp])));
-        F.push_back(f(zl(1, 0, g->X[sp], C3, g->dXdz[sp], ze)));
+        F.push_back(zl(0, 0, g->G[sp], C3, g->Gz[sp]));
+        F.push_back(zl(0, 0, g->h[sp], C3, g->hz[sp]));
+        F.push_back(zl(1, 0, g->X[sp], C3, g->dXdz[sp], ze));
     }
     F.push_back(xy(OX_ICF, 0, g->H, C3, g->Hx, XF3, nullptr));
-    F.push_back(f(xy(OX_ICF, 0, g->K, C3, g->Kx, XF3, nullptr)));
-    F.push_back(f(xy(OX_DCF, 0, g->T, C3, g->dTdx, XF3, g->xi_f)));
-    FB.push_back(f(xy(OX_ICF, 0, g->tau_xx, C3, g->txx_x, XF3, nullptr)));
-    F.push_back(f(xy(OX_ICF, 0, g->v_c, C3, g->v_x, XF3, nullptr)));
-    F.push_back(f(xy(OX_ICF, 0, g->w_c, C3, g->w_x, XF3, nullptr)));
-    FB.push_back(f(xy(OY_IFC, 1, g->tau_xy, XY3, g->txy_x, XF3, nullptr)));
-    FB.push_back(f(zl(0, 1, g->tau_xz, XF3, g->txz_x)));
+    F.push_back(xy(OX_ICF, 0, g->K, C3, g->Kx, XF3, nullptr));
+    F.push_back(xy(OX_DCF, 0, g->T, C3, g->dTdx, XF3, g->xi_f));
+    FB.push_back(xy(OX_ICF, 0, g->tau_xx, C3, g->txx_x, XF3, nullptr));
+    F.push_back(xy(OX_ICF, 0, g->v_c, C3, g->v_x, XF3, nullptr));
+    F.push_back(xy(OX_ICF, 0, g->w_c, C3, g->w_x, XF3, nullptr));
+    FB.push_back(xy(OY_IFC, 1, g->tau_xy, XY3, g->txy_x, XF3, nullptr));
+    FB.push_back(zl(0, 1, g->tau_xz, XF3, g->txz_x));
     F.push_back(xy(OY_ICF, 1, g->H, C3, g->Hy, YF3, nullptr));
-    F.push_back(f(xy(OY_ICF, 1, g->K, C3, g->Ky, YF3, nullptr)));
-    F.push_back(f(xy(ydcfw, 1, g->T, C3, g->dTdy, YF3, g->eta_f, 1.0, wall ? g->Tw : nullptr)));
-    FB.push_back(f(xy(OY_ICF, 1, g->tau_yy, C3, g->tyy_y, YF3, nullptr)));
-    F.push_back(f(xy(yicfw, 1, g->u_c, C3, g->u_y, YF3, nullptr)));
-    F.push_back(f(xy(yicfw, 1, g->w_c, C3, g->w_y, YF3, nullptr)));
-    FB.push_back(f(xy(OX_IFC, 0, g->tau_xy, XY3, g->txy_y, YF3, nullptr)));
-    FB.push_back(f(zl(0, 1, g->tau_yz, YF3, g->tyz_y)));
+    F.push_back(xy(OY_ICF, 1, g->K, C3, g->Ky, YF3, nullptr));
+    F.push_back(xy(ydcfw, 1, g->T, C3, g->dTdy, YF3, g->eta_f, 1.0, wall ? g->Tw : nullptr));
+    FB.push_back(xy(OY_ICF, 1, g->tau_yy, C3, g->tyy_y, YF3, nullptr));
+    F.push_back(xy(yicfw, 1, g->u_c, C3, g->u_y, YF3, nullptr));
+    F.push_back(xy(yicfw, 1, g->w_c, C3, g->w_y, YF3, nullptr));
+    FB.push_back(xy(OX_IFC, 0, g->tau_xy, XY3, g->txy_y, YF3, nullptr));
+    FB.push_back(zl(0, 1, g->tau_yz, YF3, g->tyz_y));
     F.push_back(zl(0, 0, g->H, C3, g->Hz));
-    F.push_back(f(zl(0, 0, g->K, C3, g->Kz)));
-    F.push_back(f(zl(1, 0, g->T, C3, g->dTdz, ze)));
-    FB.push_back(f(zl(0, 0, g->tau_zz, C3, g->tzz_z)));
-    F.push_back(f(zl(0, 0, g->u_c, C3, g->u_z)));
-    F.push_back(f(zl(0, 0, g->v_c, C3, g->v_z)));
-    FB.push_back(f(xy(OX_IFC, 0, g->tau_xz, XF3, g->txz_z, C3, nullptr)));
-    FB.push_back(f(xy(OY_IFC, 1, g->tau_yz, YF3, g->tyz_z, C3, nullptr)));
+    F.push_back(zl(0, 0, g->K, C3, g->Kz));
+    F.push_back(zl(1, 0, g->T, C3, g->dTdz, ze));
+    FB.push_back(zl(0, 0, g->tau_zz, C3, g->tzz_z));
+    F.push_back(zl(0, 0, g->u_c, C3, g->u_z));
+    F.push_back(zl(0, 0, g->v_c, C3, g->v_z));
+    FB.push_back(xy(OX_IFC, 0, g->tau_xz, XF3, g->txz_z, C3, nullptr));
+    FB.push_back(xy(OY_IFC, 1, g->tau_yz, YF3, g->tyz_z, C3, nullptr));
     std::vector<Line3>& D = pl.divs.lines;
     for (int sp = 1; sp < NSP; ++sp) {
         D.push_back(xy(OX_DFC, 0, g->Fsx[sp], XF3, g->DX + g->off[sp], C3, g->xi_c, -1.0));
@@ -1196,103 +1016,47 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
     D.push_back(xy(OX_DFC, 0, g->Gxz, XF3, g->DX + g->off[NSP + 3], C3, g->xi_c, -1.0));
     D.push_back(xy(OY_DFC, 1, g->Gyz, YF3, g->DY + g->off[NSP + 3], C3, g->eta_c, -1.0));
     D.push_back(zl(1, 0, g->Gzz, C3, g->DZ + g->off[NSP + 3], -ze));
-    // launches: the independent phases put their x/y lines before their z lines and batch each
-    // kind; the viscosity phase keeps its order (its edge values come from its face values)
-    Phase3* phases[] = {&pl.p1, &pl.p3, &pl.ad1, &pl.ad2, &pl.mu, &pl.face, &pl.faceb, &pl.divs};
-    pl.mu.slot_base = pl.faceb.slot_base = BATCH3;
-    for (Phase3* ph : phases) {
-        std::vector<Line3>& V = ph->lines;
-        if (ph != &pl.mu)
-            std::stable_partition(V.begin(), V.end(), [](const Line3& L) { return L.axis != 2; });
-        for (size_t i = 0; i < V.size();) {
-            const int z = V[i].axis == 2;
-            size_t e = i;
-            while (e < V.size() && (V[e].axis == 2) == z && e - i < (size_t)BATCH3) ++e;
-            ph->launches.push_back(Launch3{z, (int)i, (int)(e - i), 0});
-            i = e;
-        }
-    }
-    // x and y lines as segmented line jobs: plane groups for y; per launch, segments as in two
-    // dimensions (lines split while the launch has fewer than 40960 threads); one forward-sweep
-    // buffer per position in a launch
+    // one launch per phase: the lines of a phase are independent of each other
     {
-        // binary32 copies of the metrics for the jobs that run binary32 rows
-        err = cudaMalloc(&g->metf, (2 * (nx + ny) + 2) * sizeof(float));
-        if (err != cudaSuccess) return cuda_fail(err, "cudaMalloc(3-D binary32 metrics)");
-        const double* met_d[4] = {g->xi_c, g->xi_f, g->eta_c, g->eta_f};
-        const long long met_off[4] = {0, nx, 2LL * nx + 1, 2LL * nx + 1 + ny};
         std::vector<LineJob> lj;
-        std::vector<int> slot;
-        long long tmp_n = 0;
-        int slots = 1;
-        for (Phase3* ph : phases)
-            for (Launch3& b : ph->launches) {
-                if (b.z) continue;
-                const int j0 = (int)lj.size();
-                std::vector<int> ns(b.count), m(b.count);
-                long long threads = 0;
-                for (int i = 0; i < b.count; ++i) {
-                    Line3& L = ph->lines[b.first + i];
-                    m[i] = hops[L.op - g->ops].m;
-                    LineJob j;
-                    memset(&j, 0, sizeof(j));
-                    j.op = L.op;
-                    j.in_state = ph == &pl.p1 ? 1 : 0;
-                    j.in = L.in;
-                    j.out = L.out;
-                    j.scale = L.scale;
-                    j.metric = L.metric;
-                    j.wall_value = L.wall;
-                    j.wall_arr = L.wall_arr;
-                    j.f32ok = L.f32;
-                    for (int k = 0; k < 4; ++k)
-                        if (L.metric && L.metric == met_d[k]) j.metric_f = g->metf + met_off[k];
-                    if (L.axis == 0) {
-                        j.in_ls = sh.pitch(L.tin);
-                        j.out_ls = sh.pitch(L.tout);
-                        j.in_es = j.out_es = 1;
-                        j.nlines = sh.rows(L.tin) * nz;
-                    } else {
-                        j.lpp = sh.pitch(L.tin);
-                        j.in_ls = j.out_ls = 1;
-                        j.in_es = sh.pitch(L.tin);
-                        j.out_es = sh.pitch(L.tout);
-                        j.in_ps = sh.plane(L.tin);
-                        j.out_ps = sh.plane(L.tout);
-                        j.nlines = sh.pitch(L.tin) * nz;
-                    }
-                    ns[i] = 1;
-                    while (ns[i] < LINE_BLOCK / 2 && (m[i] + ns[i] - 1) / ns[i] > 260) ns[i] *= 2;
-                    threads += (long long)j.nlines * ns[i];
-                    tmp_n = std::max(tmp_n, sh.size(L.tout));
-                    L.job = (int)lj.size();
-                    lj.push_back(j);
-                    slot.push_back(ph->slot_base + i);
+        for (Phase3* ph : {&pl.p1, &pl.p3, &pl.ad1, &pl.ad2, &pl.mu, &pl.mu2, &pl.face, &pl.faceb, &pl.divs}) {
+            Launch3 b{(int)lj.size(), (int)ph->lines.size(), 0};
+            for (const Line3& L : ph->lines) {
+                LineJob j;
+                memset(&j, 0, sizeof(j));
+                j.op = g->ops + L.op;
+                j.in_state = ph == &pl.p1 ? 1 : 0;
+                j.in = L.in;
+                j.out = L.out;
+                j.scale = L.scale;
+                j.metric = L.metric;
+                j.wall_arr = L.wall_arr;
+                if (L.axis == 0) {
+                    j.in_ls = sh.pitch(L.tin);
+                    j.out_ls = sh.pitch(L.tout);
+                    j.in_es = j.out_es = 1;
+                    j.nlines = sh.rows(L.tin) * nz;
+                } else if (L.axis == 1) {
+                    j.lpp = sh.pitch(L.tin);
+                    j.in_ls = j.out_ls = 1;
+                    j.in_es = sh.pitch(L.tin);
+                    j.out_es = sh.pitch(L.tout);
+                    j.in_ps = sh.plane(L.tin);
+                    j.out_ps = sh.plane(L.tout);
+                    j.nlines = sh.pitch(L.tin) * nz;
+                } else {
+                    j.in_ls = j.out_ls = 1;
+                    j.in_es = j.out_es = sh.plane(L.tin);
+                    j.nlines = (int)sh.plane(L.tin);
                 }
-                while (threads < 40960) {
-                    bool grew = false;
-                    threads = 0;
-                    for (int i = 0; i < b.count; ++i) {
-                        if (ns[i] < LINE_BLOCK / 2 && (m[i] + 2 * ns[i] - 1) / (2 * ns[i]) >= 32) {
-                            ns[i] *= 2;
-                            grew = true;
-                        }
-                        threads += (long long)lj[j0 + i].nlines * ns[i];
-                    }
-                    if (!grew) break;
-                }
-                for (int i = 0; i < b.count; ++i) {
-                    LineJob& j = lj[j0 + i];
-                    j.nseg = ns[i];
-                    const int lpb = LINE_BLOCK / ns[i];
-                    b.blocks = std::max(b.blocks, (j.nlines + lpb - 1) / lpb);
-                }
-                slots = std::max(slots, ph->slot_base + b.count);
+                plan_line(hops[L.op], j);
+                b.blocks = std::max(b.blocks, j.blocks);
+                lj.push_back(j);
             }
-        err = cudaMalloc(&g->ltmp, (size_t)slots * tmp_n * sizeof(double));
-        if (err == cudaSuccess) err = cudaMalloc(&g->jobs, lj.size() * sizeof(LineJob));
+            ph->launches.push_back(b);
+        }
+        err = cudaMalloc(&g->jobs, lj.size() * sizeof(LineJob));
         if (err != cudaSuccess) return cuda_fail(err, "cudaMalloc(3-D line jobs)");
-        for (size_t k = 0; k < lj.size(); ++k) lj[k].tmp = g->ltmp + (size_t)slot[k] * tmp_n;
         HYP_CUDA(cudaMemcpyAsync(g->jobs, lj.data(), lj.size() * sizeof(LineJob), cudaMemcpyHostToDevice, s));
         HYP_CUDA(cudaStreamSynchronize(s));
     }
@@ -1304,16 +1068,12 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
     }
     // ---------------- uploads, reference, initial state ----------------
 #define UP3(dst, src, bytes) HYP_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s))
-    UP3(g->ops, hops.data(), NOPS * sizeof(LineOp));
-    UP3(g->opdata, opdata.data(), opdata.size() * sizeof(double));
+    UP3(g->ops, hops.data(), NOPS3 * sizeof(LineOp));
+    UP3(g->opdata, opdata.data(), opdata.size() * sizeof(LineTail));
     UP3(g->xi_c, xi_c.data(), nx * sizeof(double));
     UP3(g->xi_f, xi_f.data(), (nx + 1) * sizeof(double));
     UP3(g->eta_c, eta_c.data(), ny * sizeof(double));
     UP3(g->eta_f, eta_f.data(), (ny + 1) * sizeof(double));
-    std::vector<float> metf_h;
-    for (const auto* v : {&xi_c, &xi_f, &eta_c, &eta_f})
-        for (double x : *v) metf_h.push_back((float)x);
-    UP3(g->metf, metf_h.data(), metf_h.size() * sizeof(float));
     UP3(g->Tw, Tw.data(), Tw.size() * sizeof(double));
     k_reference3<<<blocks3(g->nstate), 128, 0, s>>>(gd, P, *desc, jet, *g);
     const bool noisy = cas->noise && cas->noise_amp > 0;

@@ -530,7 +530,7 @@ extern "C" const char* hyp_last_error(void) { return g_last_error.c_str(); }
 namespace gaskern {
 
 template <bool MIXED>
-__global__ void __launch_bounds__(128) k_thermo_eval(
+__global__ void __launch_bounds__(128, SWEEP_MIN_BLOCKS) k_thermo_eval(
     const __grid_constant__ GasDev g, int64_t n, const double* __restrict__ rho, const double* __restrict__ e,
     const double* __restrict__ Y, double* __restrict__ T, double* __restrict__ p,
     double* __restrict__ wdot, double* __restrict__ mu, double* __restrict__ kk,

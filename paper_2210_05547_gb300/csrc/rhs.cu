@@ -363,7 +363,7 @@ enum OpId { OX_ICF, OX_DCF, OX_IFC, OX_DFC, OY_ICF, OY_DCF, OY_IFC, OY_DFC, OY_I
 // executor's kernel holds them, so that both pass the shared closure_point the same kinds of
 // pointers.
 template <bool MIXED, bool LTE>
-__global__ void __launch_bounds__(128, CLOSURE_MIN_BLOCKS) k_closure(const __grid_constant__ GasDev g,
+__global__ void __launch_bounds__(128, closure_min_blocks<MIXED, LTE>()) k_closure(const __grid_constant__ GasDev g,
                                                     const Scales sc, const GridView v,
                                                     const double* __restrict__ U, const Scratch s) {
     __shared__ Scales sh_sc;

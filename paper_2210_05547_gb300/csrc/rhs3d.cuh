@@ -141,7 +141,7 @@ __global__ void k_fv3(Grid3 g, View3 v, const double* __restrict__ U) {
 }
 
 template <bool MIXED>
-__global__ void __launch_bounds__(128) k_closure3(const __grid_constant__ GasDev gd, const Scales sc, const Grid3 g, View3 v,
+__global__ void __launch_bounds__(128, closure_min_blocks<MIXED>()) k_closure3(const __grid_constant__ GasDev gd, const Scales sc, const Grid3 g, View3 v,
                                                   const double* __restrict__ U) {
     const bool cneq = sc.kind == HYP_GAS_CNEQ;
     RANGE3(g.nc) {

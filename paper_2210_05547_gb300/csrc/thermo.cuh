@@ -520,6 +520,15 @@ __host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho,
 
 namespace hyp {
 
+// Resident blocks of 128 threads per SM the closure kernels are compiled for. The integer closure
+// waits on its own chains, so warps pay, until the registers of four blocks (128) spill too much:
+// 2048 x 256 step FP64 5.80 ms with three blocks, 5.94 with four and five; mixed 5.09, 4.98, 5.18;
+// eleven-species right-hand side (512 x 128) 0.97, 0.78, 0.79; 256 x 128 x 64 jet 10.05, 10.17, 10.13
+// (10.54 unbounded); 4,000,037 states of the sweep 6.26, 5.26, 5.92, eleven species 1.15, 0.87, 0.94.
+template <bool MIXED, bool LTE = false>
+constexpr int closure_min_blocks() { return (NSP > 5 || MIXED) && !LTE ? 4 : 3; }
+constexpr int SWEEP_MIN_BLOCKS = 4;
+
 #ifdef __CUDACC__
 // The binary64 closure out of line: the states and gases that closure_fix.cuh does not take.
 static __device__ __noinline__ void closure_general(const GasDev& g, double rho, double e, const double* Y,

@@ -109,10 +109,9 @@ __global__ void kb_ad_raw(const BatchItem* __restrict__ items, BatchDev B) {
     });
 }
 
-template <bool MIXED>
 __global__ void kb_gauss(const BatchItem* __restrict__ items, BatchDev B, int dir) {
     for_tiles(items, B, SP_GAUSS, [&](const BatchItem& it, long long lo, long long hi) {
-        if (it.v.ad) gauss_body<MIXED>(it.v, it.s, dir, lo, hi, blockDim.x);
+        if (it.v.ad) gauss_body(it.v, it.s, dir, lo, hi, blockDim.x);
     });
 }
 
@@ -255,10 +254,12 @@ int rebuild(hyp_batch* b, cudaStream_t s) {
         it.n[SP_NC] = nc;
         it.n[SP_FACES] = G->d.size(hyp::NXF) + G->d.size(hyp::NYF);
         it.n[SP_NCN] = G->d.size(hyp::NCN);
-        // the binary32 filter's threads take every field of a point (gauss_body)
-        it.n[SP_GAUSS] = b->precision == HYP_MIXED ? nc : (long long)AD_FIELDS * nc;
+        // runs of four along x or along y, whichever is more (the bodies stop at their own count)
+        it.n[SP_GAUSS] = (long long)AD_FIELDS * std::max(hyp::gauss_runs(G->d.nx, G->d.ny, 0),
+                                                         hyp::gauss_runs(G->d.nx, G->d.ny, 1));
         it.n[SP_STATE] = G->nstate;
-        it.n[SP_FILTER] = G->cas.filter_sigma > 0.0 ? G->nstate : 0;
+        it.n[SP_FILTER] = !(G->cas.filter_sigma > 0.0) ? 0
+                          : std::max(hyp::filter_runs(G->d.nx, G->d.ny, 0), hyp::filter_runs(G->d.nx, G->d.ny, 1));
     }
     for (int sp = 0; sp < SP_COUNT; ++sp) {
         int* ts = b->h_tstart.data() + (size_t)sp * (n + 1);
@@ -357,13 +358,8 @@ int launch_step(hyp_batch* b, cudaStream_t s) {
         HYP_CUDA(cudaEventRecord(b->join[0], s2));
         HYP_CUDA(cudaStreamWaitEvent(s, b->join[0], 0));
         kb_ad_raw<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
-        if (mixed) {
-            kb_gauss<true><<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 0);
-            kb_gauss<true><<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 1);
-        } else {
-            kb_gauss<false><<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 0);
-            kb_gauss<false><<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 1);
-        }
+        kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 0);
+        kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 1);
         kb_ad_combine<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
         kb_stress_c<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
         HYP_CUDA(cudaGetLastError());

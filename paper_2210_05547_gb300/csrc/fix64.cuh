@@ -318,6 +318,59 @@ FX double f64_of_signed(i64 v, int q) {
     return double_of(bits_of(x) | ((u64)v & 0x8000000000000000ull));
 }
 
+// ---- fixed-point numbers of a common scale (line solver, filters): values below 2^E in magnitude ----
+
+#ifdef __CUDACC__
+// m >> s, zero for s >= 64.
+__device__ __forceinline__ u64 shift_down(u64 m, int s) {
+    u64 v;
+    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // PTX clamps the shift amount
+    return v;
+}
+
+__device__ __forceinline__ unsigned magnitude(double x) {    // high word of |x|
+    return (unsigned)__double2hiint(x) & 0x7fffffffu;
+}
+
+// Values whose largest high word is `top`: too large (or not finite) for a common scale, or its E.
+__device__ __forceinline__ bool scale_wild(unsigned top) { return top >= (unsigned)(1023 + 899) << 20; }
+__device__ __forceinline__ int scale_of(unsigned top) { return max((int)(top >> 20) - 1022, -960); }
+
+// x in units of 2^(E - q), truncated towards zero.
+__device__ __forceinline__ i64 to_scale(double x, int E, int q) {
+    const int hi = __double2hiint(x);
+    const u64 m = ((u64)__double_as_longlong(x) << 11) | 0x8000000000000000ull;
+    const i64 v = (i64)shift_down(m, 63 - q + E + 1023 - ((hi >> 20) & 0x7ff));
+    const i64 s = hi >> 31;
+    return (v ^ s) - s;
+}
+
+// The binary64 nearest to m 2^(E - q) for m < 2^33, its sign bit set by `sign`.
+__device__ __noinline__ inline double small_from_scale(u64 m, int E, int q, unsigned sign) {
+    return double_of(bits_of(f64_of_fixed(m, q - E)) | (u64)sign << 32);
+}
+
+// The binary64 nearest to y 2^(E - q), |y| < 2^63, its sign flipped by `sign` (0 or the sign bit).
+__device__ __forceinline__ double from_scale(i64 y, int E, int q, unsigned sign = 0) {
+    const int s = (int)(y >> 63);
+    const u64 m = (u64)((y ^ (i64)s) - (i64)s);
+    const u32 h = (u32)(m >> 32);
+    const unsigned sg = (unsigned)(s & 0x80000000) ^ sign;
+    if (h < 2u) return small_from_scale(m, E, q, sg);
+    const int z = __clz(h) - 1;                          // leading one to bit 62
+    const u64 v = ((m << z) + 0x200) >> 10;              // [2^52, 2^53]
+    return double_of((v + ((u64)(u32)(E + 62 - q - z + 1022) << 52)) | (u64)sg << 32);
+}
+
+// a c 2^-64 for a constant c = h 2^32 + l (h >= 0), |a| h and |a| l small enough that the sum of
+// cross products stays below 2^63.
+__device__ __forceinline__ i64 mul_const(i64 a, int h, int l) {
+    const int ah = (int)(a >> 32);
+    const i64 x = (i64)ah * l + (i64)((u64)(u32)a * (u32)h);
+    return (i64)ah * h + (x >> 32);
+}
+#endif
+
 // 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of
 // the same range (positive under the roots): one rounding, within 0.51 ulp.
 FX bool fix_in_range(double b) {

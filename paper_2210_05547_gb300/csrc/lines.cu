@@ -56,48 +56,14 @@ enum { C_P24 = 16, C_P32 = 17, C_WA = 18, C_WB = 19, C_G = 20, C_A = 21 };
 // rho^(k+1) (1 - rho^(2 (LSEG - k))) / (1 - rho^2), the sign (-1)^(k+1)
 __constant__ LineConst c_line[2][C_A + LSEG] = {LINE_TABLE_BODY};
 
-// m >> s, zero for s >= 64.
-__device__ __forceinline__ u64 shift_down(u64 m, int s) {
-    u64 v;
-    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // PTX clamps the shift amount
-    return v;
-}
-
 struct Fix {                                     // y is held as y / 4
     typedef i64 T;
     int E;                                       // inputs below 2^E
-    // x in units of 2^(E - q), truncated
-    __device__ __forceinline__ T scaled(double x, int q) const {
-        const int hi = __double2hiint(x);
-        const u64 m = ((u64)__double_as_longlong(x) << 11) | 0x8000000000000000ull;
-        const i64 v = (i64)shift_down(m, 63 - q + E + 1023 - ((hi >> 20) & 0x7ff));
-        const i64 s = hi >> 31;
-        return (v ^ s) - s;
-    }
-    __device__ __forceinline__ T input(double x) const { return scaled(x, 62); }
-    __device__ __forceinline__ T closure(double x) const { return scaled(x, 60); }
-    // y as binary64, its sign flipped by `sign` (0 or the sign bit)
-    __device__ __forceinline__ double value(T y, unsigned sign) const {
-        const int s = (int)(y >> 63);
-        const u64 m = (u64)((y ^ (i64)s) - (i64)s);
-        const u32 h = (u32)(m >> 32);
-        if (h < 2u) return small(m, (unsigned)(s & 0x80000000) ^ sign);
-        const int z = __clz(h) - 1;                          // leading one to bit 62
-        const u64 v = ((m << z) + 0x200) >> 10;              // [2^52, 2^53]
-        return __longlong_as_double((i64)(v + ((u64)(u32)(E + 2 - z + 1022) << 52)) |
-                                    (i64)((u64)((unsigned)(s & 0x80000000) ^ sign) << 32));
-    }
-    // |y| < 2^33 units
-    __device__ __noinline__ double small(u64 m, unsigned sign) const {
-        return __longlong_as_double(__double_as_longlong(f64_of_fixed(m, 60 - E)) | (i64)((u64)sign << 32));
-    }
+    __device__ __forceinline__ T input(double x) const { return to_scale(x, E, 62); }
+    __device__ __forceinline__ T closure(double x) const { return to_scale(x, E, 60); }
+    __device__ __forceinline__ double value(T y, unsigned sign) const { return from_scale(y, E, 60, sign); }
     static __device__ __forceinline__ T flip(T a, int kind) { return kind ? -a : a; }
-    // a c, c = (h 2^32 + l) 2^-64 (the sum of cross products stays below 2^63)
-    static __device__ __forceinline__ T mul(T a, const LineConst& c) {
-        const int ah = (int)(a >> 32);
-        const i64 x = (i64)ah * c.l + (i64)((u64)(u32)a * (u32)c.h);
-        return (i64)ah * c.h + (x >> 32);
-    }
+    static __device__ __forceinline__ T mul(T a, const LineConst& c) { return mul_const(a, c.h, c.l); }
     static __device__ __forceinline__ T mul(T a, const LineTail& t, int k) { return __mul64hi(a, t.h[k]); }
     static __device__ __forceinline__ T start(T a, const LineTail& t) { return __mul64hi(a, t.kappa) << 1; }
 };
@@ -315,10 +281,6 @@ __device__ __noinline__ void solve_wild(const LineJob& J, const LineOp& op, cons
     solve<Dbl>(Dbl(), J, op, P, sh, out);
 }
 
-__device__ __forceinline__ unsigned magnitude(double x) {
-    return (unsigned)__double2hiint(x) & 0x7fffffffu;
-}
-
 __global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __restrict__ jobs,
                                                            const double* __restrict__ U) {
     __shared__ Shared sh;
@@ -401,12 +363,12 @@ __global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __rest
             sh.clos[l][c] = closure_rhs(op, base_in + offset(ln, J.in_ls, J.in_ps), J.in_es, c,
                                         J.wall_arr ? J.wall_arr[ln] : J.wall_value);
     }
-    if (__syncthreads_or(P.active && top >= (unsigned)(1023 + 899) << 20)) {
+    if (__syncthreads_or(P.active && scale_wild(top))) {
         solve_wild(J, op, P, sh, out);
         return;
     }
     Fix num;
-    num.E = max((int)(sh.top[P.line < nl && P.active ? P.line : 0] >> 20) - 1022, -960);
+    num.E = scale_of(sh.top[P.active ? P.line : 0]);
     solve<Fix>(num, J, op, P, sh, out);
 }
 

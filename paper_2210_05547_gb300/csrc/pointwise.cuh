@@ -280,68 +280,74 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
     }
 }
 
-// Gaussian filter of the eight raw diffusivities along x (dir 0) or y (dir 1); indices clamp.
-// FP64: index range field f * nc + point, one field value per thread (the filter is bound by the
-// FP64 pipe, nine operations a point; the threads' independent loads hide the latency).
-// MIXED: in binary32 (truncated inputs, binary32 weights and sums, the result widened exactly)
-// over the points, each thread filtering every field at its point, so the point's indices and
-// clamped neighbours are computed once for the eight fields (integer work bounds the binary32
-// form). The filtered fields are the artificial diffusivities, nonnegative and entering only the
-// diffusive fluxes, where the few 2^-24 of relative error are immaterial.
-template <bool MIXED>
+// Gaussian filter of the raw diffusivities along x (dir 0) or y (dir 1); indices clamp. Nine
+// binary64 operations a point on a unit that takes 19 cycles each bound the plain form (80 us a
+// pass at 2048 x 256). Here a thread filters four neighbours on 62-bit integers scaled by the
+// largest of their twelve inputs, which share the conversions: 36 us (binary32 in the mixed path before: 37). Inputs that are not finite or
+// huge take the plain form.
+constexpr int RUN = 4;                                   // outputs per thread, here and in the filter
+
+// the weights c_gauss in units of 2^-64, as the words (h, l) of mul_const
+static __constant__ int c_gauss_h[5] = {1476809260, 1024362956, 330904695, 49378868, 4432499};
+static __constant__ int c_gauss_l[5] = {1060485752, 721130311, -710525454, -721130311, 180282578};
+
+// in(i): input i of the line, indices clamped or wrapped by the caller; put(k, v): output pos + k
+template <class In, class Put>
+__device__ __forceinline__ void gauss_run(int pos, const In& in, const Put& put) {
+    double x[RUN + 8];
+    unsigned top = 0;
+#pragma unroll
+    for (int k = 0; k < RUN + 8; ++k) {
+        x[k] = in(pos - 4 + k);
+        top = max(top, magnitude(x[k]));
+    }
+    if (scale_wild(top)) {
+#pragma unroll
+        for (int o = 0; o < RUN; ++o) {
+            double acc = c_gauss[0] * x[o + 4];
+#pragma unroll
+            for (int d = 1; d <= 4; ++d) acc += c_gauss[d] * (x[o + 4 - d] + x[o + 4 + d]);
+            put(o, acc);
+        }
+        return;
+    }
+    const int E = scale_of(top);
+    i64 v[RUN + 8];
+#pragma unroll
+    for (int k = 0; k < RUN + 8; ++k) v[k] = to_scale(x[k], E, 62);
+#pragma unroll
+    for (int o = 0; o < RUN; ++o) {
+        i64 acc = mul_const(v[o + 4], c_gauss_h[0], c_gauss_l[0]);
+#pragma unroll
+        for (int d = 1; d <= 4; ++d)
+            acc += mul_const(v[o + 4 - d] + v[o + 4 + d], c_gauss_h[d], c_gauss_l[d]);
+        put(o, from_scale(acc, E, 62));
+    }
+}
+
+// Runs of four per field along dir: the index range of gauss_body.
+__host__ __device__ __forceinline__ int gauss_runs(int nx, int ny, int dir) {
+    return dir == 0 ? ny * ((nx + RUN - 1) / RUN) : (ny + RUN - 1) / RUN * nx;
+}
+
 __device__ __forceinline__ void gauss_body(const GridView& v, const Scratch& s, int dir,
                                            long long lo, long long hi, long long stride) {
-    if constexpr (MIXED) {
-        for (long long li = lo + threadIdx.x; li < hi; li += stride) {
-            const int idx = (int)li;
-            const int j = idx / v.nx, i = idx - j * v.nx;
-            int nb[8];                                   // neighbours -4..-1, +1..+4, clamped
-            if (dir == 0) {
-#pragma unroll
-                for (int d = 1; d <= 4; ++d) {
-                    nb[d - 1] = j * v.nx + max(i - d, 0);
-                    nb[3 + d] = j * v.nx + min(i + d, v.nx - 1);
-                }
-            } else {
-#pragma unroll
-                for (int d = 1; d <= 4; ++d) {
-                    nb[d - 1] = max(j - d, 0) * v.nx + i;
-                    nb[3 + d] = min(j + d, v.ny - 1) * v.nx + i;
-                }
-            }
-#pragma unroll 2
-            for (int f = 0; f < AD_FIELDS; ++f) {
-                const double* __restrict__ in = dir == 0 ? s.raw[f] : s.filt[f];
-                double* __restrict__ out = dir == 0 ? s.filt[f] : s.raw[f];
-                float acc = __fmul_rn(c_gauss_f[0], f32_trunc(in[idx]));
-#pragma unroll
-                for (int d = 1; d <= 4; ++d)
-                    acc = fmaf(c_gauss_f[d], __fadd_rn(f32_trunc(in[nb[d - 1]]), f32_trunc(in[nb[3 + d]])),
-                               acc);
-                out[idx] = f64_of(acc);
-            }
-        }
-    } else {
-        const long long n = (long long)v.nx * v.ny;
-        for (long long li = lo + threadIdx.x; li < hi; li += stride) {
-            const int f = (int)(li / n);
-            const int idx = (int)(li - f * n);
-            const double* __restrict__ in = dir == 0 ? s.raw[f] : s.filt[f];
-            double* __restrict__ out = dir == 0 ? s.filt[f] : s.raw[f];
-            const int j = idx / v.nx, i = idx - j * v.nx;
-            double acc = c_gauss[0] * in[idx];
-            if (dir == 0) {
-                const double* r = in + (long long)j * v.nx;
-#pragma unroll
-                for (int d = 1; d <= 4; ++d)
-                    acc += c_gauss[d] * (r[max(i - d, 0)] + r[min(i + d, v.nx - 1)]);
-            } else {
-#pragma unroll
-                for (int d = 1; d <= 4; ++d)
-                    acc += c_gauss[d] * (in[(long long)max(j - d, 0) * v.nx + i] +
-                                         in[(long long)min(j + d, v.ny - 1) * v.nx + i]);
-            }
-            out[idx] = acc;
+    const int n = gauss_runs(v.nx, v.ny, dir), qx = (v.nx + RUN - 1) / RUN;
+    hi = min(hi, (long long)AD_FIELDS * n);
+    for (long long li = lo + threadIdx.x; li < hi; li += stride) {
+        const int f = (int)((unsigned)li / (unsigned)n), r = (int)li - f * n;
+        if (dir == 0) {
+            const int j = r / qx, i = (r - j * qx) * RUN;
+            const double* __restrict__ in = s.raw[f] + (long long)j * v.nx;
+            double* __restrict__ out = s.filt[f] + (long long)j * v.nx;
+            gauss_run(i, [&](int k) { return in[min(max(k, 0), v.nx - 1)]; },
+                      [&](int k, double y) { if (i + k < v.nx) out[i + k] = y; });
+        } else {
+            const int q = r / v.nx, i = r - q * v.nx, j = q * RUN;
+            const double* __restrict__ in = s.filt[f] + i;
+            double* __restrict__ out = s.raw[f] + i;
+            gauss_run(j, [&](int k) { return in[(long long)min(max(k, 0), v.ny - 1) * v.nx]; },
+                      [&](int k, double y) { if (j + k < v.ny) out[(long long)(j + k) * v.nx] = y; });
         }
     }
 }
@@ -523,42 +529,91 @@ static __constant__ double c_filter_w[5][11] = {
     {-1.0 / 1024, 10.0 / 1024, -45.0 / 1024, 120.0 / 1024, -210.0 / 1024, 252.0 / 1024,
      -210.0 / 1024, 120.0 / 1024, -45.0 / 1024, 10.0 / 1024, -1.0 / 1024}};
 
+// Runs of four entries along dir in the three sections of the state: the index range of filter_body.
+__host__ __device__ __forceinline__ long long filter_runs(int nx, int ny, int dir) {
+    if (dir == 0)
+        return ((NSP + 1) * (long long)ny + ny + 1) * ((nx + RUN - 1) / RUN) + (long long)ny * ((nx + RUN) / RUN);
+    return ((NSP + 1) * (long long)nx + nx + 1) * ((ny + RUN - 1) / RUN) + (long long)nx * ((ny + RUN) / RUN);
+}
+
+// The plain form took twelve binary64 operations an entry (96 us a pass at 2048 x 256). A thread
+// takes four entries of a line: away from the ends the tenth difference is formed on integers, whose
+// weights 252, 210, 120, 45, 10, 1 are exact, in units of 2^-52 of the largest input; one FMA with
+// the entry itself (binary64) finishes: 43 us. Entries near the ends, and inputs that are not finite
+// or huge, take the plain form.
 __device__ __forceinline__ void filter_body(int nx, int ny, const double* __restrict__ in,
                                             double* __restrict__ out, int dir, double sigma,
                                             long long lo, long long hi, long long stride) {
-    const long long nc = (long long)nx * ny;
-    const long long nxf = (long long)(nx + 1) * ny;
+    const int across = dir == 0 ? ny : nx, along = dir == 0 ? nx : ny;
+    const long long q0 = (along + RUN - 1) / RUN, q1 = (along + RUN) / RUN;   // runs per line
+    // sections: centres, the faces with one more entry across, the faces with one more along
+    const long long nc = (long long)nx * ny, nxf = (long long)(nx + 1) * ny;
+    const long long n0 = (NSP + 1) * (long long)across * q0, n1 = (across + 1) * q0;
+    hi = min(hi, n0 + n1 + across * q1);
     for (long long idx = lo + threadIdx.x; idx < hi; idx += stride) {
-        long long local;
-        int pitch, rows;
-        if (idx < (NSP + 1) * nc) {
-            local = idx % nc;
-            pitch = nx;
-            rows = ny;
-        } else if (idx < (NSP + 1) * nc + nxf) {
-            local = idx - (NSP + 1) * nc;
-            pitch = nx + 1;
-            rows = ny;
+        long long t = idx, base, q = q0;
+        int pitch = nx, n = along;
+        bool xf = false;
+        if (idx < n0) {
+            base = 0;
+        } else if (idx < n0 + n1) {
+            t = idx - n0;
+            xf = dir == 1;                               // one more across: x-faces' columns
+            base = (NSP + 1) * nc + (xf ? 0 : nxf);
         } else {
-            local = idx - (NSP + 1) * nc - nxf;
-            pitch = nx;
-            rows = ny + 1;
+            t = idx - n0 - n1;
+            q = q1;
+            n = along + 1;
+            xf = dir == 0;
+            base = (NSP + 1) * nc + (xf ? 0 : nxf);
         }
-        const int row = (int)(local / pitch), col = (int)(local - (long long)row * pitch);
-        const int pos = dir == 0 ? col : row;
-        const int n = dir == 0 ? pitch : rows;
-        const long long st = dir == 0 ? 1 : pitch;
-        const int m = min(min(pos, n - 1 - pos), 5);
-        const double f = in[idx];
-        if (m == 0) {
-            out[idx] = f;
-            continue;
+        if (xf) pitch = nx + 1;
+        // dir 0: line = row (of a field), run fastest; dir 1: column fastest, then run, then field
+        long long first, st;
+        int pos;
+        if (dir == 0) {
+            const long long line = t / q;
+            pos = (int)(t - line * q) * RUN;
+            first = base + line * pitch;
+            st = 1;
+        } else {
+            const long long field = t / (q * pitch), r = t - field * q * pitch;
+            const int run = (int)(r / pitch), col = (int)(r - (long long)run * pitch);
+            pos = run * RUN;
+            first = base + field * n * pitch + col;
+            st = pitch;
         }
-        const double* w = c_filter_w[m - 1];
-        const double* p = in + idx - m * st;
-        double acc = 0.0;
-        for (int k = 0; k <= 2 * m; ++k) acc = fma(w[k], p[k * st], acc);
-        out[idx] = fma(-sigma, acc, f);
+        const double* __restrict__ p = in + first;
+        double x[RUN + 10];
+        unsigned top = 0;
+#pragma unroll
+        for (int k = 0; k < RUN + 10; ++k) {
+            x[k] = p[min(max(pos - 5 + k, 0), n - 1) * st];
+            top = max(top, magnitude(x[k]));
+        }
+        const bool wild = scale_wild(top);
+        const int E = scale_of(top);
+        i64 v[RUN + 10];
+#pragma unroll
+        for (int k = 0; k < RUN + 10; ++k) v[k] = to_scale(x[k], E, 52);
+#pragma unroll
+        for (int o = 0; o < RUN; ++o) {
+            const int at = pos + o;
+            if (at >= n) continue;
+            const int m = min(min(at, n - 1 - at), 5);
+            const double f = x[o + 5];
+            double acc = 0.0;
+            if (m == 5 && !wild) {
+                i64 d = 252 * v[o + 5] - 210 * (v[o + 4] + v[o + 6]) + 120 * (v[o + 3] + v[o + 7]) -
+                        45 * (v[o + 2] + v[o + 8]) + 10 * (v[o + 1] + v[o + 9]) - (v[o] + v[o + 10]);
+                acc = from_scale(d, E, 62);              // over 1024
+            } else if (m > 0) {
+                const double* w = c_filter_w[m - 1];
+                const double* c = p + (at - m) * st;
+                for (int k = 0; k <= 2 * m; ++k) acc = fma(w[k], c[k * st], acc);
+            }
+            out[first + at * st] = m == 0 ? f : fma(-sigma, acc, f);
+        }
     }
 }
 

@@ -402,9 +402,8 @@ __global__ void k_ad_raw(int cneq, GridView v, const double* __restrict__ U, Scr
     ad_raw_body(cneq != 0, v, U, s, GRID_RANGE((long long)v.nx * v.ny));
 }
 
-template <bool MIXED>
 __global__ void k_gauss(GridView v, Scratch s, int dir) {
-    gauss_body<MIXED>(v, s, dir, GRID_RANGE((MIXED ? 1LL : (long long)AD_FIELDS) * v.nx * v.ny));
+    gauss_body(v, s, dir, GRID_RANGE((long long)AD_FIELDS * gauss_runs(v.nx, v.ny, dir)));
 }
 
 __global__ void k_ad_combine(GridView v, Scratch s) {
@@ -427,9 +426,9 @@ __global__ void k_flux(GasDev g, Scales sc, GridView v, const double* __restrict
 
 __global__ void k_assemble(long long n, AssembleArgs a) { assemble_body(a, GRID_RANGE(n)); }
 
-__global__ void k_filter(int nx, int ny, long long nstate, const double* __restrict__ in,
+__global__ void k_filter(int nx, int ny, const double* __restrict__ in,
                          double* __restrict__ out, int dir, double sigma) {
-    filter_body(nx, ny, in, out, dir, sigma, GRID_RANGE(nstate));
+    filter_body(nx, ny, in, out, dir, sigma, GRID_RANGE(filter_runs(nx, ny, dir)));
 }
 
 __global__ void k_fill(double* p, long long n, double val) {
@@ -1021,14 +1020,8 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[0], 0));
     if (v.ad) {
         TIMED(KID_AD_RAW, (k_ad_raw<<<blocks_for(nc, 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S)));
-        const int gg = blocks_for(mixed ? nc : AD_FIELDS * nc, 256);
-        if (mixed) {
-            TIMED(KID_AD_GAUSS, (k_gauss<true><<<gg, 256, 0, s>>>(v, S, 0)));
-            TIMED(KID_AD_GAUSS, (k_gauss<true><<<gg, 256, 0, s>>>(v, S, 1)));
-        } else {
-            TIMED(KID_AD_GAUSS, (k_gauss<false><<<gg, 256, 0, s>>>(v, S, 0)));
-            TIMED(KID_AD_GAUSS, (k_gauss<false><<<gg, 256, 0, s>>>(v, S, 1)));
-        }
+        for (int dir = 0; dir < 2; ++dir)
+            TIMED(KID_AD_GAUSS, (k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir)));
         TIMED(KID_AD_COMBINE, (k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
         HYP_CUDA(cudaGetLastError());
     }
@@ -1095,9 +1088,9 @@ extern "C" int hyp_grid_temperature(const hyp_grid* grid, int64_t n_T, double* T
 // The state filter after the last RK stage: x pass into the scratch state vector, y pass back.
 static int launch_filter(hyp_grid* G, double* U, cudaStream_t s) {
     const double sigma = G->cas.filter_sigma;
-    const int blocks = blocks_for(G->nstate, 256);
-    TIMED(KID_FILTER, (k_filter<<<blocks, 256, 0, s>>>(G->d.nx, G->d.ny, G->nstate, U, G->s.R, 0, sigma)));
-    TIMED(KID_FILTER, (k_filter<<<blocks, 256, 0, s>>>(G->d.nx, G->d.ny, G->nstate, G->s.R, U, 1, sigma)));
+    const int nx = G->d.nx, ny = G->d.ny;
+    TIMED(KID_FILTER, (k_filter<<<blocks_for(filter_runs(nx, ny, 0), 256), 256, 0, s>>>(nx, ny, U, G->s.R, 0, sigma)));
+    TIMED(KID_FILTER, (k_filter<<<blocks_for(filter_runs(nx, ny, 1), 256), 256, 0, s>>>(nx, ny, G->s.R, U, 1, sigma)));
     HYP_CUDA(cudaGetLastError());
     return HYP_OK;
 }
@@ -1376,9 +1369,8 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
         HYP_CUDA(lines(PH_AD2, 2));
         k_ad_prep<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
         k_ad_raw<<<blocks_for(nc, 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S);
-        const int gg = blocks_for(AD_FIELDS * nc, 256);
-        k_gauss<false><<<gg, 256, 0, s>>>(v, S, 0);
-        k_gauss<false><<<gg, 256, 0, s>>>(v, S, 1);
+        for (int dir = 0; dir < 2; ++dir)
+            k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir);
         k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
         HYP_CUDA(cudaGetLastError());
     }

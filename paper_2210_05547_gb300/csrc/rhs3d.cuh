@@ -296,58 +296,44 @@ __global__ void k_adraw3(Grid3 g, View3 v, const double* __restrict__ U, int cne
 }
 
 // Gaussian filter of the raw diffusivities along one axis (x, y clamped; z periodic):
-// pass 0 raw -> filt (x), 1 filt -> raw (y), 2 raw -> filt (z). MIXED: in binary32 as gauss_body
-// (pointwise.cuh) does for two-dimensional grids.
-template <typename R, bool MIXED>
-__device__ __forceinline__ R gauss3_load(const double* p) {
-    if constexpr (MIXED) return f32_trunc(*p);
-    else return *p;
-}
-
-__device__ __forceinline__ float gauss3_fma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double gauss3_fma(double a, double b, double c) { return fma(a, b, c); }
-
-template <bool MIXED>
+// pass 0 raw -> filt (x), 1 filt -> raw (y), 2 raw -> filt (z), runs of four (gauss_run).
 __global__ void k_gauss3(Grid3 g, int axis) {
-    using R = typename std::conditional<MIXED, float, double>::type;
     const Sh3 s = g.sh;
-    const long long n = g.nc, pl = (long long)s.nx * s.ny;
-    const R* w;
-    if constexpr (MIXED) w = c_gauss_f;
-    else w = c_gauss;
-    // FP64: one field value per thread (field-major index range, as gauss_body); binary32: every
-    // field of a point per thread
-    RANGE3(MIXED ? n : (long long)AD_FIELDS * n) {
-        const int f0 = MIXED ? 0 : (int)(q / n);
-        const long long idx = q - (long long)f0 * n;
-        const int i = (int)(idx % s.nx);
-        const long long t = idx / s.nx;
-        const int j = (int)(t % s.ny), k = (int)(t / s.ny);
-        long long nb[8];                                 // neighbours -4..-1, +1..+4 (indices)
-#pragma unroll
-        for (int d = 1; d <= 4; ++d) {
-            if (axis == 0) {
-                nb[d - 1] = idx - i + max(i - d, 0);
-                nb[3 + d] = idx - i + min(i + d, s.nx - 1);
-            } else if (axis == 1) {
-                nb[d - 1] = idx + (long long)(max(j - d, 0) - j) * s.nx;
-                nb[3 + d] = idx + (long long)(min(j + d, s.ny - 1) - j) * s.nx;
-            } else {
-                nb[d - 1] = idx + (long long)(((k - d) % s.nz + s.nz) % s.nz - k) * pl;
-                nb[3 + d] = idx + (long long)((k + d) % s.nz - k) * pl;
-            }
+    const long long pl = (long long)s.nx * s.ny;
+    const int qx = (s.nx + RUN - 1) / RUN, qy = (s.ny + RUN - 1) / RUN, qz = (s.nz + RUN - 1) / RUN;
+    // runs per field: along x the run is fastest, else the column
+    const long long n = axis == 0 ? (long long)qx * s.ny * s.nz : (axis == 1 ? (long long)s.nx * qy * s.nz : pl * qz);
+    RANGE3((long long)AD_FIELDS * n) {
+        const int f = (int)(q / n);
+        const long long r = q - f * n;
+        const double* __restrict__ in = axis == 1 ? g.filt[f] : g.raw[f];
+        double* __restrict__ out = axis == 1 ? g.raw[f] : g.filt[f];
+        long long first, st;
+        int pos, len;
+        if (axis == 0) {
+            const long long line = r / qx;
+            pos = (int)(r - line * qx) * RUN;
+            first = line * s.nx;
+            st = 1;
+            len = s.nx;
+        } else if (axis == 1) {
+            const int i = (int)(r % s.nx);
+            const long long t = r / s.nx;
+            pos = (int)(t % qy) * RUN;
+            first = t / qy * pl + i;
+            st = s.nx;
+            len = s.ny;
+        } else {
+            pos = (int)(r / pl) * RUN;
+            first = r % pl;
+            st = pl;
+            len = s.nz;
         }
-        for (int f = f0; f < (MIXED ? AD_FIELDS : f0 + 1); ++f) {
-            const double* __restrict__ in = axis == 1 ? g.filt[f] : g.raw[f];
-            double* __restrict__ out = axis == 1 ? g.raw[f] : g.filt[f];
-            R acc = w[0] * gauss3_load<R, MIXED>(in + idx);
-#pragma unroll
-            for (int d = 1; d <= 4; ++d)
-                acc = gauss3_fma(w[d], gauss3_load<R, MIXED>(in + nb[d - 1]) +
-                                           gauss3_load<R, MIXED>(in + nb[3 + d]), acc);
-            if constexpr (MIXED) out[idx] = f64_of(acc);
-            else out[idx] = acc;
-        }
+        const double* __restrict__ line = in + first;
+        double* __restrict__ to = out + first;
+        const auto put = [&](int k, double y) { if (pos + k < len) to[(pos + k) * st] = y; };
+        if (axis < 2) gauss_run(pos, [&](int k) { return line[min(max(k, 0), len - 1) * st]; }, put);
+        else gauss_run(pos, [&](int k) { return line[((k % len + len) % len) * st]; }, put);
     }
 }
 
@@ -600,7 +586,6 @@ int run_rhs3(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUdt, int
     const View3 v = view3(G, g);
     const GasDev& gd = gas->dev;
     const Plan3& pl = *g->plan;
-    const int mx = precision == HYP_MIXED ? 1 : 0;
     int rc = launch3(g, pl.p1, U, s);
     if (rc) return rc;
     k_fv3<<<blocks3(g->nxf + g->nyf + g->nc), 256, 0, s>>>(*g, v, U);
@@ -626,10 +611,8 @@ int run_rhs3(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUdt, int
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[0], 0));
     if (v.ad) {
         k_adraw3<<<blocks3(g->nc), 256, 0, s>>>(*g, v, U, gd.kind == HYP_GAS_CNEQ);
-        for (int ax = 0; ax < 3; ++ax) {
-            if (mx) k_gauss3<true><<<blocks3(g->nc), 256, 0, s>>>(*g, ax);
-            else k_gauss3<false><<<blocks3(AD_FIELDS * g->nc), 256, 0, s>>>(*g, ax);
-        }
+        for (int ax = 0; ax < 3; ++ax)
+            k_gauss3<<<blocks3(AD_FIELDS * ((g->nc + RUN - 1) / RUN)), 256, 0, s>>>(*g, ax);
         k_adcombine3<<<blocks3(g->nc), 256, 0, s>>>(*g);
         HYP_CUDA(cudaGetLastError());
     }

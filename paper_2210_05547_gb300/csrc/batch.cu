@@ -104,7 +104,7 @@ __global__ void kb_ad_prep(const BatchItem* __restrict__ items, BatchDev B) {
 }
 
 __global__ void kb_ad_raw(const BatchItem* __restrict__ items, BatchDev B) {
-    for_tiles(items, B, SP_NC, [&](const BatchItem& it, long long lo, long long hi) {
+    for_tiles(items, B, SP_GAUSS, [&](const BatchItem& it, long long lo, long long hi) {
         if (it.v.ad) ad_raw_body(it.cneq != 0, it.v, it.U, it.s, lo, hi, blockDim.x);
     });
 }
@@ -357,7 +357,7 @@ int launch_step(hyp_batch* b, cudaStream_t s) {
         kb_ad_prep<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s2>>>(b->d_items, B);
         HYP_CUDA(cudaEventRecord(b->join[0], s2));
         HYP_CUDA(cudaStreamWaitEvent(s, b->join[0], 0));
-        kb_ad_raw<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
+        kb_ad_raw<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B);
         kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 0);
         kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 1);
         kb_ad_combine<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);

@@ -399,7 +399,7 @@ __global__ void k_ad_prep(GridView v, Scratch s) {
 }
 
 __global__ void k_ad_raw(int cneq, GridView v, const double* __restrict__ U, Scratch s) {
-    ad_raw_body(cneq != 0, v, U, s, GRID_RANGE((long long)v.nx * v.ny));
+    ad_raw_body(cneq != 0, v, U, s, GRID_RANGE((long long)AD_FIELDS * gauss_runs(v.nx, v.ny, 0)));
 }
 
 __global__ void k_gauss(GridView v, Scratch s, int dir) {
@@ -1019,7 +1019,7 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     HYP_CUDA(cudaEventRecord(G->join[0], s2));
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[0], 0));
     if (v.ad) {
-        TIMED(KID_AD_RAW, (k_ad_raw<<<blocks_for(nc, 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S)));
+        TIMED(KID_AD_RAW, (k_ad_raw<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, 0), 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S)));
         for (int dir = 0; dir < 2; ++dir)
             TIMED(KID_AD_GAUSS, (k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir)));
         TIMED(KID_AD_COMBINE, (k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
@@ -1368,7 +1368,7 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
         HYP_CUDA(lines(PH_AD1, 2));
         HYP_CUDA(lines(PH_AD2, 2));
         k_ad_prep<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
-        k_ad_raw<<<blocks_for(nc, 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S);
+        k_ad_raw<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, 0), 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S);
         for (int dir = 0; dir < 2; ++dir)
             k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir);
         k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);

@@ -115,15 +115,10 @@ __global__ void kb_gauss(const BatchItem* __restrict__ items, BatchDev B, int di
     });
 }
 
-__global__ void kb_ad_combine(const BatchItem* __restrict__ items, BatchDev B) {
-    for_tiles(items, B, SP_NC, [&](const BatchItem& it, long long lo, long long hi) {
-        if (it.v.ad) ad_combine_body(it.s, lo, hi, blockDim.x);
-    });
-}
-
 __global__ void kb_stress_c(const BatchItem* __restrict__ items, BatchDev B) {
     for_tiles(items, B, SP_NC, [&](const BatchItem& it, long long lo, long long hi) {
-        stress_c_body(it.s, lo, hi, blockDim.x);
+        if (it.v.ad) stress_c_body<true>(it.s, lo, hi, blockDim.x);
+        else stress_c_body<false>(it.s, lo, hi, blockDim.x);
     });
 }
 
@@ -134,9 +129,9 @@ __global__ void kb_stress_cn(const BatchItem* __restrict__ items, BatchDev B) {
 }
 
 template <bool SMK>
-__global__ void kb_flux(GasDev g, const BatchItem* __restrict__ items, BatchDev B) {
+__global__ void kb_flux(const __grid_constant__ GasDev g, const BatchItem* __restrict__ items, BatchDev B) {
     for_tiles(items, B, SP_FACES, [&](const BatchItem& it, long long lo, long long hi) {
-        flux_body<SMK>(g, it.sc, it.v, it.U, it.s, -1, lo, hi, blockDim.x);
+        flux_body<SMK>(g, it.sc, it.v, it.U, it.s, lo, hi, blockDim.x);
     });
 }
 
@@ -360,7 +355,6 @@ int launch_step(hyp_batch* b, cudaStream_t s) {
         kb_ad_raw<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B);
         kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 0);
         kb_gauss<<<grid_for_tiles(b, SP_GAUSS, pw), 256, 0, s>>>(b->d_items, B, 1);
-        kb_ad_combine<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
         kb_stress_c<<<grid_for_tiles(b, SP_NC, pw), 256, 0, s>>>(b->d_items, B);
         HYP_CUDA(cudaGetLastError());
         HYP_CUDA(cudaEventRecord(b->fork[1], s));

@@ -423,26 +423,28 @@ __device__ __forceinline__ void gauss_body(const GridView& v, const Scratch& s, 
     }
 }
 
-__device__ __forceinline__ void ad_combine_body(const Scratch& s, long long lo, long long hi,
-                                                long long stride) {
-    for (long long li = lo + threadIdx.x; li < hi; li += stride) {
-        const int i = (int)li;
-        s.mu_e[i] += s.raw[0][i];
-        s.beta[i] = s.raw[1][i];
-        s.K[i] += s.raw[2][i];
-#pragma unroll
-        for (int sp = 0; sp < NSP; ++sp) s.G[sp][i] = s.Wd[sp][i] + s.W[sp][i] * s.raw[3 + sp][i];
-    }
-}
-
-// (F, I) normal stresses and momentum fluxes at centres (Eqs. 5, 6, 9)
+// (F, I) normal stresses and momentum fluxes at centres (Eqs. 5, 6, 9). AD: the filtered artificial
+// diffusivities join the transport coefficients first: memory bounds both, and one pass instead of
+// two (13 fields of a cell read and written once less) takes a launch off the chain too: the
+// 32 x 16 right-hand side 166 -> 163 us with the single flux launch below, 515 x 131 411 -> 402.
+template <bool AD>
 __device__ __forceinline__ void stress_c_body(const Scratch& s, long long lo, long long hi,
                                               long long stride) {
     for (long long li = lo + threadIdx.x; li < hi; li += stride) {
         const int i = (int)li;
         const double ux = s.dudx[i], vy = s.dvdy[i];
         const double dv = ux + vy;
-        const double mu = s.mu_e[i], b = s.beta[i];
+        double mu = s.mu_e[i], b;
+        if constexpr (AD) {
+            mu += s.raw[0][i];
+            b = s.raw[1][i];
+            s.mu_e[i] = mu;
+            s.K[i] += s.raw[2][i];
+#pragma unroll
+            for (int sp = 0; sp < NSP; ++sp) s.G[sp][i] = s.Wd[sp][i] + s.W[sp][i] * s.raw[3 + sp][i];
+        } else {
+            b = s.beta[i];
+        }
         const double txx = mu * (2.0 * ux - 2.0 / 3.0 * dv) + b * dv;
         const double tyy = mu * (2.0 * vy - 2.0 / 3.0 * dv) + b * dv;
         s.tau_xx[i] = txx;
@@ -539,16 +541,17 @@ __device__ __forceinline__ void flux_point(const GasDev& gd, const Scales& sc, c
     FE[i] = m * Hf[i] + q - work;
 }
 
-// Index range: the x-faces, then the y-faces (dir < 0), or the faces of one direction.
+// Index range: the x-faces, then the y-faces, in one launch: the two families are independent and
+// a launch each left the chip idle between them (2048 x 256 step 5.46 -> 5.43 ms, 515 x 131
+// right-hand side 407 -> 402 us).
 template <bool SMK>
 __device__ __forceinline__ void flux_body(const GasDev& gd, const Scales& sc, const GridView& v,
-                                          const double* __restrict__ U, const Scratch& s, int dir,
+                                          const double* __restrict__ U, const Scratch& s,
                                           long long lo, long long hi, long long stride) {
     const int nxf = v.ny * (v.nx + 1);
     for (long long li = lo + threadIdx.x; li < hi; li += stride) {
         const int i = (int)li;
-        if (dir >= 0) flux_point<SMK>(gd, sc, v, U, s, dir, i);
-        else if (i < nxf) flux_point<SMK>(gd, sc, v, U, s, 0, i);
+        if (i < nxf) flux_point<SMK>(gd, sc, v, U, s, 0, i);
         else flux_point<SMK>(gd, sc, v, U, s, 1, i - nxf);
     }
 }

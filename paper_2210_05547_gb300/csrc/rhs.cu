@@ -406,12 +406,9 @@ __global__ void k_gauss(GridView v, Scratch s, int dir) {
     gauss_body(v, s, dir, GRID_RANGE((long long)AD_FIELDS * gauss_runs(v.nx, v.ny, dir)));
 }
 
-__global__ void k_ad_combine(GridView v, Scratch s) {
-    ad_combine_body(s, GRID_RANGE((long long)v.nx * v.ny));
-}
-
+template <bool AD>
 __global__ void k_stress_c(GridView v, Scratch s) {
-    stress_c_body(s, GRID_RANGE((long long)v.nx * v.ny));
+    stress_c_body<AD>(s, GRID_RANGE((long long)v.nx * v.ny));
 }
 
 __global__ void k_stress_cn(GridView v, Scratch s) {
@@ -419,9 +416,9 @@ __global__ void k_stress_cn(GridView v, Scratch s) {
 }
 
 template <bool SMK>
-__global__ void k_flux(GasDev g, Scales sc, GridView v, const double* __restrict__ U, Scratch s,
-                       int dir) {
-    flux_body<SMK>(g, sc, v, U, s, dir, GRID_RANGE(dir == 0 ? (long long)v.ny * (v.nx + 1) : (long long)(v.ny + 1) * v.nx));
+__global__ void k_flux(const __grid_constant__ GasDev g, Scales sc, GridView v, const double* __restrict__ U,
+                       Scratch s) {
+    flux_body<SMK>(g, sc, v, U, s, GRID_RANGE((long long)v.ny * (v.nx + 1) + (long long)(v.ny + 1) * v.nx));
 }
 
 __global__ void k_assemble(long long n, AssembleArgs a) { assemble_body(a, GRID_RANGE(n)); }
@@ -1022,10 +1019,11 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
         TIMED(KID_AD_RAW, (k_ad_raw<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, 0), 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S)));
         for (int dir = 0; dir < 2; ++dir)
             TIMED(KID_AD_GAUSS, (k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir)));
-        TIMED(KID_AD_COMBINE, (k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
-        HYP_CUDA(cudaGetLastError());
+        TIMED(KID_AD_COMBINE, (k_stress_c<true><<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
+    } else {
+        TIMED(KID_STRESS_C, (k_stress_c<false><<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
     }
-    TIMED(KID_STRESS_C, (k_stress_c<<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
+    HYP_CUDA(cudaGetLastError());
     // fork: viscosity to the corners, shear stress and its face interpolants beside the face phase
     HYP_CUDA(cudaEventRecord(G->fork[1], s));
     HYP_CUDA(cudaStreamWaitEvent(s2, G->fork[1], 0));
@@ -1043,11 +1041,9 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
     HYP_CUDA(e1);
     HYP_CUDA(cudaStreamWaitEvent(s, G->join[1], 0));
     if (v.sm) {
-        TIMED(KID_FLUX, (k_flux<true><<<blocks_for(d.size(NXF), 128), 128, 0, s>>>(g, sc, v, U, S, 0)));
-        TIMED(KID_FLUX, (k_flux<true><<<blocks_for(d.size(NYF), 128), 128, 0, s>>>(g, sc, v, U, S, 1)));
+        TIMED(KID_FLUX, (k_flux<true><<<blocks_for(d.size(NXF) + d.size(NYF), 128), 128, 0, s>>>(g, sc, v, U, S)));
     } else {
-        TIMED(KID_FLUX, (k_flux<false><<<blocks_for(d.size(NXF), 128), 128, 0, s>>>(g, sc, v, U, S, 0)));
-        TIMED(KID_FLUX, (k_flux<false><<<blocks_for(d.size(NYF), 128), 128, 0, s>>>(g, sc, v, U, S, 1)));
+        TIMED(KID_FLUX, (k_flux<false><<<blocks_for(d.size(NXF) + d.size(NYF), 128), 128, 0, s>>>(g, sc, v, U, S)));
     }
     TIMED(KID_LINES_DIV, e1 = launch_lines(G->jobs + G->ph_start[PH_DIV], G->ph_count[PH_DIV],
                                            G->ph_blocks[PH_DIV], U, s));
@@ -1371,21 +1367,20 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
         k_ad_raw<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, 0), 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S);
         for (int dir = 0; dir < 2; ++dir)
             k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir);
-        k_ad_combine<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
-        HYP_CUDA(cudaGetLastError());
+        k_stress_c<true><<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
+    } else {
+        k_stress_c<false><<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
     }
-    k_stress_c<<<blocks_for(nc, 256), 256, 0, s>>>(v, S);
+    HYP_CUDA(cudaGetLastError());
     HYP_CUDA(lines(PH_MU1, 1));
     HYP_CUDA(lines(PH_MU2, 1));
     k_stress_cn<<<blocks_for(d.size(NCN), 256), 256, 0, s>>>(v, S);
     HYP_CUDA(lines(PH_FACE, G->ph_count[PH_FACE]));
     HYP_CUDA(lines(PH_FACEB, G->ph_count[PH_FACEB]));
     if (v.sm) {
-        k_flux<true><<<blocks_for(d.size(NXF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S, 0);
-        k_flux<true><<<blocks_for(d.size(NYF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S, 1);
+        k_flux<true><<<blocks_for(d.size(NXF) + d.size(NYF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S);
     } else {
-        k_flux<false><<<blocks_for(d.size(NXF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S, 0);
-        k_flux<false><<<blocks_for(d.size(NYF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S, 1);
+        k_flux<false><<<blocks_for(d.size(NXF) + d.size(NYF), 128), 128, 0, s>>>(g, scales_of(g), v, U, S);
     }
     HYP_CUDA(lines(PH_DIV, G->ph_count[PH_DIV]));
     const AssembleArgs aa{S.DX, S.DY, S.SRC, G->sigma, G->Uref, G->mask, (double*)U, dUdt,

@@ -33,40 +33,28 @@ METRIC = "Mpts*RHS/s FP64"
 UNIT = "Mpts*RHS/s"
 STAGES = 3
 L2_FLUSH_BYTES = 256 << 20
-# FP64 operations per cell-centre point executed by k_closure (DADD + DMUL + 2 DFMA), from ncu's
-# thread instruction counts of a launch of an RK step after the first (1024 x 256 cells;
-# 680.8 DFMA, 124.8 DADD, 513.3 DMUL per point; profiles/k_closure_sbli.md).
-CLOSURE_FP64_FLOP_PER_POINT = 1999.7
-# The same counts as FP64 warp-lane instructions (DFMA + DADD + DMUL): a DADD or DMUL takes an FP64
-# issue slot like a DFMA but counts one flop, so the pipe's occupancy is the instruction rate
-# against 2 instructions per clock per SM. All instructions on the FP64 pipe (comparisons and
-# conversions included): 1460.5 per point.
-CLOSURE_FP64_INSTR_PER_POINT = 1318.9
-CLOSURE_FP64_PIPE_INSTR_PER_POINT = 1460.5
-# The closure's FP64 operation count when every exponential, logarithm, quotient and square root
-# is CUDA's own (the earlier form of this kernel): 3041 per point. Dividing it by the time of the
-# current kernel gives an effective rate, reported beside the measured-count roofline.
-CLOSURE_LIBM_FLOP_PER_POINT = 3041.0
-# DRAM bytes (read + write) per k_closure launch at 2048 x 256: 696 B per point measured at
-# 1024 x 256 (dram__bytes counters of the same launch) scaled by the point count.
-CLOSURE_DRAM_BYTES = 695.7 * 1024 * 256
-CLOSURE_DRAM_POINTS = 1024 * 256
-# FP64 operations (2 DFMA + DADD + DMUL) per cell centre and right-hand side over every kernel of
-# a step, from ncu's thread instruction counts of every launch of one step at 1024 x 256:
-# closure 1999.7, line operators 1104.9, pointwise kernels 781.3 (profiles/fp64_flops_sbli_1024x256.md;
-# the closure re-counted after its last change, the other kernels unchanged since their count).
-RHS_FP64_FLOP_PER_POINT = 3885.9
-# GB300 FP64 peak derived from the unit counts: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz.
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# hyp_thermo_eval (five-species air, FP64, every output): FP64 operations per state, 2 DFMA + DADD
-# + DMUL from ncu's thread instruction counts of one launch over 2e6 states of the sweep's
-# distribution (919.5 DFMA, 232.0 DADD, 585.6 DMUL per state; profiles/k_thermo_eval_sweep.md).
-THERMO_FP64_FLOP_PER_STATE = 2656.6
-THERMO_FP64_INSTR_PER_STATE = 1737.1
-# k_closure3 (the three-dimensional jet's closure, FP64): FP64 operations per cell from ncu's
-# thread instruction counts of the first launch after a warm-up step at 256 x 128 x 64 cells
-# (794.1 DFMA, 111.7 DADD, 511.5 DMUL per cell; profiles/k_closure3_jet.md).
-CLOSURE3_FP64_FLOP_PER_POINT = 2211.3
+# Most of the path runs on 64-bit integers, so rooflines are in warp instructions: executed (ncu's
+# smsp__inst_executed, as thread instructions per cell: 32 per warp instruction) against four per
+# clock and SM; the binary64 unit's instructions (sm__inst_executed_pipe_fp64) against its two lanes
+# per clock and SM beside them (profiles/instructions_per_case.md).
+ISSUE_PEAK_TINSTR = 152 * 4 * 32 * 2.07e9 / 1e12      # thread instructions
+FP64_PEAK_TINSTR = 152 * 2 * 2.07e9 / 1e12
+PEAK_SOURCE = "derived: 152 SMs x 4 warp instructions/clk x 32 x 2.07 GHz"
+# instructions per cell (state): (all, binary64 unit)
+CLOSURE_INSTR = (15496, 284.7)
+CLOSURE3_INSTR = (14698, 438.5)
+THERMO_INSTR = (19944, 417.1)
+RHS_INSTR = (50923, 676.7)
+
+
+def issue_roofline(instr, units_per_s):
+    """Roofline of a kernel that executes `instr` (all, binary64) per unit of work."""
+    ach = instr[0] * units_per_s / 1e12
+    return {"bound": "alu", "achieved": ach, "peak": ISSUE_PEAK_TINSTR,
+            "unit": "T thread instructions/s", "frac": ach / ISSUE_PEAK_TINSTR,
+            "instr_per_point": instr[0], "fp64_instr_per_point": instr[1],
+            "fp64_pipe_frac": instr[1] * units_per_s / 1e12 / FP64_PEAK_TINSTR,
+            "peak_source": PEAK_SOURCE}
 
 
 def parse():
@@ -387,13 +375,7 @@ def thermo_sweep(A, gas, dev, n, seed, reps=2, precision=0):
     bad = int((status != 0).sum())
     roof = None
     if precision == 0 and ns == 5:
-        ach = THERMO_FP64_FLOP_PER_STATE * n / (ms / 1e3) / 1e12
-        roof = {"kernel": "k_thermo_eval", "bound": "alu", "achieved": ach,
-                "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": ach / FP64_PEAK_TFLOPS,
-                "algorithmic_flop_per_state": THERMO_FP64_FLOP_PER_STATE,
-                "fp64_pipe_frac": THERMO_FP64_INSTR_PER_STATE * n / (ms / 1e3)
-                                  / (FP64_PEAK_TFLOPS * 1e12 / 2.0),
-                "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2.07 GHz"}
+        roof = {"kernel": "k_thermo_eval", **issue_roofline(THERMO_INSTR, n / (ms / 1e3))}
     return {"value": n / (ms / 1e3) / 1e6, "unit": "Mstates/s", "states": n, "ms_per_sweep": ms,
             "roofline": roof,
             "bytes_per_state": 8 * (2 + ns) + 8 * (4 + 2 * ns) + 1,
@@ -567,12 +549,7 @@ def jet3d_bench(A, I, dev, rank, world, barrier, flush, steps=2, warmup=1, size=
                 avg_s = cms / ccount / 1e3
                 roof = {"kernel": "k_closure3", "launches": ccount, "avg_launch_ms": avg_s * 1e3,
                         "share_of_step": cms / max(sum(a.elapsed_time(b) for a, b in ev), 1e-30),
-                        "bound": "alu", "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                        "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2.07 GHz"}
-                if CLOSURE3_FP64_FLOP_PER_POINT > 0:
-                    ach = CLOSURE3_FP64_FLOP_PER_POINT * out["cells"] / avg_s / 1e12
-                    roof.update(achieved=ach, frac=ach / FP64_PEAK_TFLOPS,
-                                algorithmic_flop_per_point=CLOSURE3_FP64_FLOP_PER_POINT)
+                        **issue_roofline(CLOSURE3_INSTR, out["cells"] / avg_s)}
                 out["roofline"] = roof
         del step, graph, st, U, dQ
         torch.cuda.empty_cache()
@@ -701,34 +678,20 @@ def ours_arm(args, rank, world, local_rank):
                "unit": UNIT, "h2d_bytes_per_step": n * 8, "d2h_bytes_per_step": n * 8}
 
     # ---------------- roofline of the dominant kernel ----------------
-    # k_closure has the largest share of the serialised ncu launch list of the bench. The
-    # event time of a second-stream line phase that runs beside it includes the time it waits for
-    # the FP64 pipe the closure holds, so the ranking is not taken from the live totals.
+    # k_closure is the largest launch of the serialised launch list (the nine line phases together
+    # take a little more). The event time of a second-stream line phase that runs beside it includes
+    # the time it waits for issue slots, so the ranking is not taken from the live totals.
     name = "k_closure" if "k_closure" in prof else max(prof.items(), key=lambda kv: kv[1][0])[0]
     kms, kcount = prof[name]
     avg_s = kms / max(kcount, 1) / 1e3
     roof = {"kernel": name, "launches": kcount, "avg_launch_ms": avg_s * 1e3,
             "share_of_step": kms / max(dev_ms, 1e-30)}
-    if name == "k_closure" and CLOSURE_FP64_FLOP_PER_POINT > 0:
-        ach = CLOSURE_FP64_FLOP_PER_POINT * points / avg_s / 1e12
-        roof.update(bound="alu", achieved=ach, peak=FP64_PEAK_TFLOPS, unit="TFLOP/s",
-                    frac=ach / FP64_PEAK_TFLOPS,
-                    traffic=(CLOSURE_DRAM_BYTES * points / CLOSURE_DRAM_POINTS
-                             if CLOSURE_DRAM_BYTES else None),
-                    algorithmic_flop_per_point=CLOSURE_FP64_FLOP_PER_POINT,
-                    peak_source="derived: 152 SMs x 2 DFMA/clk x 2.07 GHz (a DFMA probe "
-                                "measured 1.20 TFLOP/s)",
-                    fp64_instr_per_point=CLOSURE_FP64_INSTR_PER_POINT,
-                    fp64_pipe_frac=(CLOSURE_FP64_PIPE_INSTR_PER_POINT * points / avg_s)
-                                   / (FP64_PEAK_TFLOPS * 1e12 / 2.0),
-                    effective_frac=CLOSURE_LIBM_FLOP_PER_POINT * points / avg_s / 1e12
-                                   / FP64_PEAK_TFLOPS,
-                    effective_note="the FP64 operation count of the same closure with CUDA's "
-                                   "exp, division and reciprocal (3041 per point) over this "
-                                   "kernel's time")
+    if name == "k_closure":
+        roof.update(issue_roofline(CLOSURE_INSTR, points / avg_s), traffic=None)
     else:
-        roof.update(bound="alu", achieved=None, peak=FP64_PEAK_TFLOPS, unit="TFLOP/s", frac=None,
-                    traffic=None, note="per-point FP64 count not yet measured for this kernel")
+        roof.update(bound="alu", achieved=None, peak=ISSUE_PEAK_TINSTR,
+                    unit="T thread instructions/s", frac=None, traffic=None,
+                    note="per-point instruction count not measured for this kernel")
 
     # ---------------- model variants on the same workload (FP64, same steps) ----------------
     def variant(cfg_v):
@@ -825,10 +788,7 @@ def ours_arm(args, rank, world, local_rank):
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
                 "data": "synthetic", "config": workload_config(cfg, world), "e2e": e2e,
                 "gpu_launches": launches, "roofline": roof, "cpu_baseline": cpu, "clocks": clk,
-                "whole_rhs": {"bound": "alu", "fp64_flop_per_point": RHS_FP64_FLOP_PER_POINT,
-                              "achieved": value / world * RHS_FP64_FLOP_PER_POINT / 1e6,
-                              "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s (per GPU)",
-                              "frac": value / world * RHS_FP64_FLOP_PER_POINT / 1e6 / FP64_PEAK_TFLOPS},
+                "whole_rhs": issue_roofline(RHS_INSTR, value / world * 1e6),
                 "wall_s_timed": t_wall, "status_flags": status, "mixed": mixed,
                 "serving": serving, "serving_fp64": serving_fp64,
                 "serving_plain_fp64": serving_plain, "stefan_maxwell": smd,

@@ -17,8 +17,9 @@
  * - Ownership: the caller owns every field buffer it passes (state, right-hand side, the
  *   thermo_eval inputs and outputs). The library owns the opaque handles and everything inside
  *   them (gas tables, metrics, sponge, reference state, scratch), and frees them in *_free.
- * - Floating point: FP64 throughout with precision HYP_FP64; HYP_MIXED moves the parts listed at
- *   enum hyp_precision to binary32. No call falls back to the CPU: every arithmetic step of
+ * - Floating point: inputs and results are binary64. With precision HYP_FP64 every step is in
+ *   binary64 or on 64-bit integers that carry at least its 53 bits; HYP_MIXED moves the parts
+ *   listed at enum hyp_precision to binary32. No call falls back to the CPU: every arithmetic step of
  *   rhs / rk_stage / thermo_eval runs in CUDA kernels.
  * - A grid handle carries scratch memory: calls that use the same grid (rhs, rk_stage) must not
  *   overlap on the device; serialise them on one stream.
@@ -61,18 +62,11 @@ enum hyp_gas_kind {
                             hyp_lte_eval) */
 };
 
-/* HYP_FP64: every step in binary64. HYP_MIXED: in binary32 the transport and diffusion
- * coefficients (Blottner, Eucken, Wilke, Chapman-Enskog; Sec. 2.2.1, Eq. 19), the forward-rate
- * exponentials (Eq. 13), the species heat capacities and the weakly populated electronic levels
- * (theta / T >= 9) of the species thermodynamics (Sec. 2.2.1; in the right-hand side, whose
- * neighbouring cells share a choice per level, not in hyp_thermo_eval), the Gaussian filter of
- * the artificial diffusivities (Sec. 3.3), and the interior rows of the compact
- * interpolations and derivatives that feed only the diffusive fluxes (Sec. 3.1); in double-word
- * binary32 (each value a pair of binary32 words) the interior rows of the other compact operators;
- * in binary64 the Newton iteration for the temperature, the vibrational factors and populated
- * electronic levels that set the species energies, equilibrium constants and backward rates,
- * every closure row of the operators, every divergence, the fluxes themselves and the stage
- * update. */
+/* HYP_FP64: every step in binary64 or on 64-bit integers that carry at least its 53 bits (the
+ * species thermodynamics, kinetics, compact operators, filters and fourth differences, in a common
+ * scale; states and lines outside their range take binary64). HYP_MIXED: the transport and
+ * diffusion coefficients (Blottner, Eucken, Wilke, Chapman-Enskog; Sec. 2.2.1, Eq. 19) in
+ * binary32, all else as HYP_FP64. */
 enum hyp_precision { HYP_FP64 = 0, HYP_MIXED = 1 };
 
 enum hyp_error {
@@ -345,9 +339,8 @@ void hyp_server_free(hyp_server* sv);
  * (binary64): DEVICE outputs, each nullable. */
 int hyp_round_f32(int64_t n, const double* x, float* y, double* back, void* stream);
 
-/* The binary64 exponential, quotient, reciprocal and logarithm the FP64 closure uses
- * (diagnostics; no counterpart in the paper): exp and log by Tang's table-driven methods, a / b
- * and 1 / b from a binary32 reciprocal refined in binary64, each within 2 ulp; arguments outside
+/* The binary64 exponential, quotient, reciprocal and logarithm of the closure's general form
+ * (diagnostics; no counterpart in the paper), on 64-bit integers, each within 2 ulp; arguments outside
  * their fast ranges (|a| >= 512 for exp, |b| outside [2^-120, 2^120] for the quotients, a outside
  * [2, 2^1000) for log) go through CUDA's exp, division and log. fn 0: out[i] = exp(a[i]); fn 1:
  * out[i] = a[i] / b[i]; fn 2: out[i] = 1 / b[i]; fn 3: out[i] = log(a[i]). a, b (the one a
@@ -391,7 +384,7 @@ int hyp_lte_eval(const hyp_gas* gas, int64_t n, const double* rho, const double*
  * cudaMalloc behind their back. It computes the same right-hand side as hyp_rhs for the same gas,
  * grid and U, within rounding (the Newton inversion starts from 1000 K instead of the grid's
  * previous temperatures). Arguments as for hyp_rhs, always FP64; two-dimensional grids only.
- * - Scratch: every per-call scratch field, the line-sweep storage and the launch plan live in one
+ * - Scratch: every per-call scratch field and the launch plan live in one
  *   file-scope device array of 12 MiB (1,572,864 doubles) that every GPU loading the library holds
  *   until exit. Grids needing more (a few thousand cells, e.g. up to 64 x 64) are rejected with
  *   HYP_ERR_ARG and the required size in hyp_last_error(). The grid's own scratch and predictor

@@ -17,15 +17,15 @@
 //     q_r = (1 + rho^2) rhs_r - rho q_{r-1},     y_r = q_r - rho y_{r+1}
 // with the same rho (1/3, 0.148) on every row. A thread runs both from zero; what enters from its
 // neighbours follows from their own end values, q_in = e_{-1} + rho^8 e_{-2} + ... (five terms,
-// rho^40 < 2^-63), likewise y_in, and their effect on row k, a_k q_in + b_k y_in, is added. The row before the first interior row is an
-// explicit closure row, as is the row after the last: the latter starts the backward recurrence,
-// the former fixes q's unknown start Q, whose effect h_k Q is added to the first rows.
-// Periodic lines wrap the exchange around (or, when 16 does not divide the period, extend the line
-// by three segments each way), lines of more than LINE_THREADS segments are cut into chunks with
-// such margins.
+// rho^40 < 2^-63), likewise y_in, and their effect on row k, a_k q_in + b_k y_in, is added. The row
+// before the first interior row is an explicit closure row, as is the row after the last: the
+// latter starts the backward recurrence, the former fixes q's unknown start Q, whose effect h_k Q
+// is added to the first rows. Periodic lines wrap the exchange around (or, when 8 does not divide
+// the period, extend the line by LINE_TAIL rows each way); lines of more than LINE_THREADS threads
+// are cut into chunks with such margins.
 //
-// Inputs and, for lines along x (unit stride), results pass through shared memory, 17 words per
-// thread of 16 so that neither the threads' rows nor the coalesced copies meet bank conflicts;
+// Inputs and, for lines along x (unit stride), results pass through shared memory, 9 words per
+// thread of 8 so that neither the threads' rows nor the coalesced copies meet bank conflicts;
 // neighbouring threads hold neighbouring lines, which keeps the few threads with closure rows in
 // one or two warps.
 //
@@ -33,8 +33,8 @@
 // block), so that such values spread as far as a binary64 solve lets them.
 //
 // Measured (GB300): the 50 operators of the face phase at 1024 x 256 take 190 us (the binary64
-// sweeps 234, the binary32 and double-word ones 201), a phase of one or two operators 19-21 us (38-46); the
-// step of the 2048 x 256 shock case 6.69 -> 5.96 ms, of the 256 x 64 boundary layer 0.85 -> 0.57,
+// sweeps 234, those in pairs of binary32 words 201), a phase of one or two operators 19-21 us
+// (38-46); the step of the 2048 x 256 shock case 6.69 -> 5.96 ms, of the 256 x 64 boundary layer 0.85 -> 0.57,
 // the 256 x 128 x 64 jet's right-hand side 12.2 -> 10.5. About 280 integer instructions a row
 // warp at 2.2 per clock and SM bound it; eight rows a thread (four blocks of 288 threads per SM)
 // against sixteen (three): 5.96 against 6.5 ms. Converting the results to binary64 on the binary64
@@ -104,7 +104,7 @@ struct Shared {
     unsigned top[LINE_MAX_LINES];                // largest |input|, high word
 };
 
-// The thread's place: rows r0 .. r0 + 15 of a line, segment `seg` of `nseg`; the line's next
+// The thread's place: rows r0 .. r0 + LSEG - 1 of a line, segment `seg` of `nseg`; the line's next
 // segment is `nl` threads on.
 struct Place {
     int r0, seg, nseg, nl, line, lo, hi;

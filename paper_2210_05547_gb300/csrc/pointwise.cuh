@@ -260,9 +260,9 @@ __device__ __forceinline__ double d4y(const double* f, int j, int i, int nx, int
 // Raw artificial diffusivities: a factor times |d4x wx + d4y wy|. Fourteen binary64 operations per
 // point and field bound the plain form (110 us at 2048 x 256); here a thread takes four neighbours
 // along x of one field, the fourth differences (weights 1, -4, 6, exact) on integers in units of
-// 2^-58 of the largest of their 24 inputs, and two products and a sum remain binary64: 73 us. (The same in three dimensions, forty inputs a run, was
-// slower than the plain form there: jet right-hand side 9.77 against 9.61 ms.) Runs at
-// the ends of a row and inputs that are not finite or huge take the plain form.
+// 2^-58 of the largest of their 24 inputs, and two products and a sum remain binary64: 73 us. (The
+// same in three dimensions, forty inputs a run, was slower than the plain form there: jet
+// right-hand side 9.77 against 9.61 ms.) Runs at the ends of a row and inputs that are not finite or huge take the plain form.
 constexpr int RUN = 4;                                   // outputs per thread, here and in the filters
 
 // Runs of four per field along dir.
@@ -361,8 +361,8 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
 // Gaussian filter of the raw diffusivities along x (dir 0) or y (dir 1); indices clamp. Nine
 // binary64 operations a point on a unit that takes 19 cycles each bound the plain form (80 us a
 // pass at 2048 x 256). Here a thread filters four neighbours on 62-bit integers scaled by the
-// largest of their twelve inputs, which share the conversions: 36 us (binary32 in the mixed path before: 37). Inputs that are not finite or
-// huge take the plain form.
+// largest of their twelve inputs, which share the conversions: 36 us
+// (binary32 in the mixed path before: 37). Inputs that are not finite or huge take the plain form.
 // the weights c_gauss in units of 2^-64, as the words (h, l) of mul_const
 static __constant__ int c_gauss_h[5] = {1476809260, 1024362956, 330904695, 49378868, 4432499};
 static __constant__ int c_gauss_l[5] = {1060485752, 721130311, -710525454, -721130311, 180282578};
@@ -425,7 +425,7 @@ __device__ __forceinline__ void gauss_body(const GridView& v, const Scratch& s, 
 
 // (F, I) normal stresses and momentum fluxes at centres (Eqs. 5, 6, 9). AD: the filtered artificial
 // diffusivities join the transport coefficients first: memory bounds both, and one pass instead of
-// two (13 fields of a cell read and written once less) takes a launch off the chain too: the
+// two (beta is no longer stored, beta and mu not read again) takes a launch off the chain too: the
 // 32 x 16 right-hand side 166 -> 163 us with the single flux launch below, 515 x 131 411 -> 402.
 template <bool AD>
 __device__ __forceinline__ void stress_c_body(const Scratch& s, long long lo, long long hi,

@@ -1263,9 +1263,9 @@ extern "C" int hyp_grid_profile_read(const hyp_grid* grid, int n, double* ms, in
 // hosts) that own all device memory through their own allocator and do not let a library call
 // cudaMalloc behind their back. hyp_rhs never allocates either, but it keeps its scratch inside
 // the grid handle, which the grid allocated when it was built; this variant instead takes every
-// scratch field, the line-sweep storage and its launch plan from the file-scope array below, so a
-// grid's scratch is not touched. The grid's read-only data (metrics, reference state, sponge,
-// operators) are used as is, and the per-point status bits go to the grid's status word.
+// scratch field and its launch plan from the file-scope array below, so a grid's scratch is not
+// touched. The grid's read-only data (metrics, reference state, sponge, operators) are used as is,
+// and the per-point status bits go to the grid's status word.
 // ---------------------------------------------------------------------------------------------
 
 #define HYP_NOALLOC_DOUBLES (3LL << 19)   // 1,572,864 doubles = 12 MiB per GPU

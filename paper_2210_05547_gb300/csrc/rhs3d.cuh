@@ -13,8 +13,8 @@
 // at centres and on the three edge families, the three-dimensional strain and vorticity in the
 // artificial-diffusivity sensors (fourth differences and Gaussian filter periodic in z), stresses
 // at centres and edges, species and energy fluxes on the three face families, divergences in
-// three directions. Lines along x and y run through the segmented line kernel of the
-// two-dimensional path (lines.cu; lines along y grouped by z-plane); lines along z are periodic
+// three directions. Lines along x and y run through the line kernel of the two-dimensional
+// path (lines.cu; lines along y grouped by z-plane); lines along z are periodic
 // (every row interior) and go through it too. Each phase is one launch; the velocity-gradient and
 // artificial-diffusivity phases run on a second stream beside the closure, and the viscosity
 // phase, the stresses and their face values there beside the other face values.

@@ -649,7 +649,7 @@ def ours_arm(args, rank, world, local_rank):
         del R64, R32
         mixed = {"value": job_rate(world, points, args.steps, m_ms),
                  "unit": UNIT, "ms_per_step": m_ms / args.steps,
-                 "dtype": "f64 with f32 transport and diffusion",
+                 "dtype": "f64 with f32 transport, diffusion and forward-rate exponentials",
                  "rhs_err_vs_fp64_path": errs, "max_rhs_err": max(errs.values()),
                  "err_bound": "1e-6 of max|R| per field against the FP64 oracle "
                               "(tests/test_gpu_mixed.py); wall heat flux and skin friction "

@@ -65,8 +65,8 @@ enum hyp_gas_kind {
 /* HYP_FP64: every step in binary64 or on 64-bit integers that carry at least its 53 bits (the
  * species thermodynamics, kinetics, compact operators, filters and fourth differences, in a common
  * scale; states and lines outside their range take binary64). HYP_MIXED: the transport and
- * diffusion coefficients (Blottner, Eucken, Wilke, Chapman-Enskog; Sec. 2.2.1, Eq. 19) in
- * binary32, all else as HYP_FP64. */
+ * diffusion coefficients (Blottner, Eucken, Wilke, Chapman-Enskog; Sec. 2.2.1, Eq. 19) and the
+ * forward-rate exponentials (Eq. 13) in binary32, all else as HYP_FP64. */
 enum hyp_precision { HYP_FP64 = 0, HYP_MIXED = 1 };
 
 enum hyp_error {

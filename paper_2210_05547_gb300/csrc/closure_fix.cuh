@@ -185,7 +185,9 @@ FX bool fix_signed62(double x, i64& out) {
     return ex <= 0;
 }
 
-// e^(n ln T - theta / T), theta given by sign and xf; zero for theta / T > 900.
+// e^(n ln T - theta / T), theta given by sign and xf; zero for theta / T > 900. F32: in binary32
+// (the exponent rounded to binary32, a subnormal result zero), above binary32's range in 64 bits.
+template <bool F32>
 FX xf rate_exp(i64 n59, i64 L58, int neg, u64 tm, int te, xf iT) {
     const u64 p = mulhi64(tm, iT.m);             // theta / T in units of 2^-62 2^(te + ie)
     const int d = 9 - te - iT.e;                 // to units of 2^-53
@@ -194,11 +196,18 @@ FX xf rate_exp(i64 n59, i64 L58, int neg, u64 tm, int te, xf iT) {
     else t53 = ~(u64)0;
     if (t53 > ((u64)900 << 53)) return xf{0, 0};
     const i64 a = mulhi64su(n59, (u64)L58) + (neg ? (i64)t53 : -(i64)t53);
+    if (F32 && a < ((i64)88 << 53)) {
+        const u32 u = bits_of_float(expf((float)a * (1.0f / 9007199254740992.0f)));
+        const int ex = (int)(u >> 23);
+        return ex == 0 ? xf{0, 0} : xf{(u64)((u & 0x7fffffu) | 0x800000u) << 40, ex - 127};
+    }
     return exp_fixed<53>(a);
 }
 
 // Production rates (Eqs. 14, 15). With z_s = conc_s / r_s (r_s the molar partition function per
-// unit volume): R = (sum_r C_r [M_r]) prod r^rf (E_f prod z^rf - E_b prod z^rb).
+// unit volume): R = (sum_r C_r [M_r]) prod r^rf (E_f prod z^rf - E_b prod z^rb). MIXED: E_f in
+// binary32.
+template <bool MIXED>
 FX void kinetics_fix(const GasDev& g, double T, i64 L58, xf iT, const FixState& s,
                      const double* conc, double* wdot) {
     const xf t15 = exp_fixed<58>(L58 + (L58 >> 1));          // T^(3/2): below e^17.3
@@ -218,8 +227,8 @@ FX void kinetics_fix(const GasDev& g, double T, i64 L58, xf iT, const FixState& 
     }
     for (int k = 0; k < g.ngroup; ++k) {
         const xf one{0x8000000000000000ull, 0};
-        xf f = rate_exp(g.fix.n59[k], L58, g.fix.sgn[k] & 1, g.fix.ta_m[k], g.fix.ta_e[k], iT);
-        xf b = rate_exp(g.fix.n59[k], L58, g.fix.sgn[k] >> 1, g.fix.tb_m[k], g.fix.tb_e[k], iT);
+        xf f = rate_exp<MIXED>(g.fix.n59[k], L58, g.fix.sgn[k] & 1, g.fix.ta_m[k], g.fix.ta_e[k], iT);
+        xf b = rate_exp<false>(g.fix.n59[k], L58, g.fix.sgn[k] >> 1, g.fix.tb_m[k], g.fix.tb_e[k], iT);
         xf rr = one;
         unsigned nf = 0, nb = 0;
 #pragma unroll

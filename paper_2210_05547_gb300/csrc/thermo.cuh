@@ -431,7 +431,9 @@ __host__ __device__ __forceinline__ void transport_f64(const GasDev& g, double T
     }
 }
 
-// Full closure (SI) in binary64. reactions: evaluate w_s; diffusion: evaluate D_s.
+// Full closure (SI) in binary64. reactions: evaluate w_s; diffusion: evaluate D_s. MIXED (device
+// only): the forward-rate exponentials, transport and diffusion in binary32.
+template <bool MIXED = false>
 __host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho, double e, const double* Y,
                                            double T0, bool reactions, bool diffusion,
                                            ClosureOut& o) {
@@ -500,7 +502,12 @@ __host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho,
             for (int rx = g.gstart[k]; rx < g.gstart[k + 1]; ++rx)
                 w += g.C[rx] * (g.spec[rx] >= 0 ? conc[g.spec[rx]] : 1.0);
             const double base = g.g_n[k] * lnT;
-            const double Ef = cl_exp(base - g.g_Ta[k] * invT);
+            double Ef;
+#ifdef __CUDA_ARCH__
+            if (MIXED) Ef = f64_of(expf(f32_of(base - g.g_Ta[k] * invT)));
+            else
+#endif
+                Ef = cl_exp(base - g.g_Ta[k] * invT);
             const double Eb = cl_exp(base - (g.g_Ta[k] - g.g_theta_d[k]) * invT) * cl_div(den, num);
             const double Rg = w * (Ef * fwd - Eb * bwd);
 #pragma unroll
@@ -511,7 +518,13 @@ __host__ __device__ __forceinline__ void closure_si(const GasDev& g, double rho,
         for (int i = 0; i < NSP; ++i) o.wdot[i] = g.M[i] * molar[i];
     }
 
-    transport_f64(g, T, lnT, p, s, diffusion, o);
+    if constexpr (MIXED) {
+#ifdef __CUDA_ARCH__
+        transport_f32(g, T, lnT, p, s.cv, diffusion, o);
+#endif
+    } else {
+        transport_f64(g, T, lnT, p, s, diffusion, o);
+    }
 }
 
 }  // namespace hyp
@@ -531,14 +544,15 @@ constexpr int SWEEP_MIN_BLOCKS = 4;
 
 #ifdef __CUDACC__
 // The binary64 closure out of line: the states and gases that closure_fix.cuh does not take.
+template <bool MIXED>
 static __device__ __noinline__ void closure_general(const GasDev& g, double rho, double e, const double* Y,
                                              double T0, bool reactions, bool diffusion,
                                              ClosureOut* o) {
-    closure_si(g, rho, e, Y, T0, reactions, diffusion, *o);
+    closure_si<MIXED>(g, rho, e, Y, T0, reactions, diffusion, *o);
 }
 
-// The closure on integers; false (o unspecified) for states outside its range. MIXED: transport
-// and diffusion coefficients in binary32.
+// The closure on integers; false (o unspecified) for states outside its range. MIXED: the
+// forward-rate exponentials, transport and diffusion coefficients in binary32.
 template <bool MIXED>
 __device__ __forceinline__ bool closure_fix(const GasDev& g, double rho, double e, const double* Y,
                                             double T0, bool reactions, bool diffusion,
@@ -585,7 +599,7 @@ __device__ __forceinline__ bool closure_fix(const GasDev& g, double rho, double 
         double conc[NSP];
 #pragma unroll
         for (int i = 0; i < NSP; ++i) conc[i] = rho * ymol[i];
-        kinetics_fix(g, T, L58, xf_rcp(xf_of(T)), s, conc, o.wdot);
+        kinetics_fix<MIXED>(g, T, L58, xf_rcp(xf_of(T)), s, conc, o.wdot);
     } else {
 #pragma unroll
         for (int i = 0; i < NSP; ++i) o.wdot[i] = 0.0;
@@ -610,7 +624,7 @@ __device__ __forceinline__ void closure_si_p(const GasDev& g, double rho, double
     double y[NSP];
 #pragma unroll
     for (int i = 0; i < NSP; ++i) y[i] = Y[i];
-    closure_general(g, rho, e, y, T0, reactions, diffusion, &c);
+    closure_general<MIXED>(g, rho, e, y, T0, reactions, diffusion, &c);
     o = c;
 }
 #endif

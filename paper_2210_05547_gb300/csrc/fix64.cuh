@@ -84,6 +84,14 @@ FX int clz64(u64 x) {       // x != 0
 #endif
 }
 
+FX int clz32(u32 x) {       // x != 0
+#ifdef __CUDA_ARCH__
+    return __clz((int)x);
+#else
+    return __builtin_clz(x);
+#endif
+}
+
 FX u32 mulhi32(u32 a, u32 b) {
 #ifdef __CUDA_ARCH__
     return __umulhi(a, b);
@@ -320,56 +328,105 @@ FX double f64_of_signed(i64 v, int q) {
 
 // ---- fixed-point numbers of a common scale (line solver, filters): values below 2^E in magnitude ----
 
-#ifdef __CUDACC__
-// m >> s, zero for s >= 64.
-__device__ __forceinline__ u64 shift_down(u64 m, int s) {
+// m >> s, zero for s outside 0..63.
+FX u64 shift_down(u64 m, int s) {
+#ifdef __CUDA_ARCH__
     u64 v;
     asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // PTX clamps the shift amount
     return v;
+#else
+    return (unsigned)s < 64u ? m >> s : 0;
+#endif
 }
 
-__device__ __forceinline__ unsigned magnitude(double x) {    // high word of |x|
-    return (unsigned)__double2hiint(x) & 0x7fffffffu;
-}
+FX int high_word(double x) { return (int)(bits_of(x) >> 32); }
+FX unsigned magnitude(double x) { return (unsigned)high_word(x) & 0x7fffffffu; }   // of |x|
+FX unsigned larger(unsigned a, unsigned b) { return a > b ? a : b; }
 
 // Values whose largest high word is `top`: too large (or not finite) for a common scale, or its E.
-__device__ __forceinline__ bool scale_wild(unsigned top) { return top >= (unsigned)(1023 + 899) << 20; }
-__device__ __forceinline__ int scale_of(unsigned top) { return max((int)(top >> 20) - 1022, -960); }
+FX bool scale_wild(unsigned top) { return top >= (unsigned)(1023 + 899) << 20; }
+FX int scale_of(unsigned top) {
+    const int E = (int)(top >> 20) - 1022;
+    return E > -960 ? E : -960;
+}
+
+// Whether values whose largest high word is `top` are zero or have a scale of their own (E above its
+// floor of -960, below which units of 2^(E - 62) would leave binary64's normal range).
+FX bool scale_fits(unsigned top) {
+    return top == 0u || (!scale_wild(top) && top >= (unsigned)(1023 - 960) << 20);
+}
 
 // x in units of 2^(E - q), truncated towards zero.
-__device__ __forceinline__ i64 to_scale(double x, int E, int q) {
-    const int hi = __double2hiint(x);
-    const u64 m = ((u64)__double_as_longlong(x) << 11) | 0x8000000000000000ull;
+FX i64 to_scale(double x, int E, int q) {
+    const int hi = high_word(x);
+    const u64 m = (bits_of(x) << 11) | 0x8000000000000000ull;
     const i64 v = (i64)shift_down(m, 63 - q + E + 1023 - ((hi >> 20) & 0x7ff));
     const i64 s = hi >> 31;
     return (v ^ s) - s;
 }
 
 // The binary64 nearest to m 2^(E - q) for m < 2^33, its sign bit set by `sign`.
-__device__ __noinline__ inline double small_from_scale(u64 m, int E, int q, unsigned sign) {
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+static inline double small_from_scale(u64 m, int E, int q, unsigned sign) {
     return double_of(bits_of(f64_of_fixed(m, q - E)) | (u64)sign << 32);
 }
 
 // The binary64 nearest to y 2^(E - q), |y| < 2^63, its sign flipped by `sign` (0 or the sign bit).
-__device__ __forceinline__ double from_scale(i64 y, int E, int q, unsigned sign = 0) {
+FX double from_scale(i64 y, int E, int q, unsigned sign = 0) {
     const int s = (int)(y >> 63);
     const u64 m = (u64)((y ^ (i64)s) - (i64)s);
     const u32 h = (u32)(m >> 32);
-    const unsigned sg = (unsigned)(s & 0x80000000) ^ sign;
+    const unsigned sg = ((unsigned)s & 0x80000000u) ^ sign;
     if (h < 2u) return small_from_scale(m, E, q, sg);
-    const int z = __clz(h) - 1;                          // leading one to bit 62
+    const int z = clz32(h) - 1;                          // leading one to bit 62
     const u64 v = ((m << z) + 0x200) >> 10;              // [2^52, 2^53]
     return double_of((v + ((u64)(u32)(E + 62 - q - z + 1022) << 52)) | (u64)sg << 32);
 }
 
 // a c 2^-64 for a constant c = h 2^32 + l (h >= 0), |a| h and |a| l small enough that the sum of
 // cross products stays below 2^63.
-__device__ __forceinline__ i64 mul_const(i64 a, int h, int l) {
+FX i64 mul_const(i64 a, int h, int l) {
     const int ah = (int)(a >> 32);
     const i64 x = (i64)ah * l + (i64)((u64)(u32)a * (u32)h);
     return (i64)ah * h + (x >> 32);
 }
-#endif
+
+constexpr int RUN = 4;                                   // outputs per thread of the filters and differences
+
+// Tenth differences over 1024 (weights 252, -210, 120, -45, 10, -1) of the four windows of eleven in
+// x, in 72 bits (high and low words apart) and so within 2 units of 2^-62 of the largest input; then
+// rounded to binary64. False where that is not better than binary64: inputs that are not finite, huge
+// or tiny, or a window whose inputs may all be below 2^-7 of the largest.
+FX bool tenth_run(const double (&x)[RUN + 10], double (&acc)[RUN]) {
+    unsigned core = 0, ends = 0;                         // core: in every window
+    for (int k = 0; k < RUN + 10; ++k) {
+        if (k >= RUN - 1 && k < 11) core = larger(core, magnitude(x[k]));
+        else ends = larger(ends, magnitude(x[k]));
+    }
+    const unsigned top = larger(core, ends);
+    if (!scale_fits(top) || (core >> 20) + 6 < top >> 20) return false;
+    const int E = scale_of(top);
+    i64 v[RUN + 10];
+#pragma unroll
+    for (int k = 0; k < RUN + 10; ++k) v[k] = to_scale(x[k], E, 62);
+#pragma unroll
+    for (int o = 0; o < RUN; ++o) {
+        const i64 s[6] = {v[o + 5], v[o + 4] + v[o + 6], v[o + 3] + v[o + 7], v[o + 2] + v[o + 8],
+                          v[o + 1] + v[o + 9], v[o] + v[o + 10]};
+        const u32 w[6] = {252, 210, 120, 45, 10, 1};
+        i64 h = 0;
+        u64 even = 0, odd = 0;                           // low words' sums
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            h += (i64)(int)(s[k] >> 32) * (k & 1 ? -(int)w[k] : (int)w[k]);
+            (k & 1 ? odd : even) += (u64)(u32)s[k] * w[k];
+        }
+        acc[o] = from_scale((h << 22) + ((i64)(even - odd) >> 10), E, 62);
+    }
+    return true;
+}
 
 // 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of
 // the same range (positive under the roots): one rounding, within 0.51 ulp.

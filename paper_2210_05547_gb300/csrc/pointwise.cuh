@@ -263,8 +263,6 @@ __device__ __forceinline__ double d4y(const double* f, int j, int i, int nx, int
 // 2^-58 of the largest of their 24 inputs, and two products and a sum remain binary64: 73 us. (The
 // same in three dimensions, forty inputs a run, was slower than the plain form there: jet
 // right-hand side 9.77 against 9.61 ms.) Runs at the ends of a row and inputs that are not finite or huge take the plain form.
-constexpr int RUN = 4;                                   // outputs per thread, here and in the filters
-
 // Runs of four per field along dir.
 __host__ __device__ __forceinline__ int gauss_runs(int nx, int ny, int dir) {
     return dir == 0 ? ny * ((nx + RUN - 1) / RUN) : (ny + RUN - 1) / RUN * nx;
@@ -612,9 +610,9 @@ __host__ __device__ __forceinline__ long long filter_runs(int nx, int ny, int di
 
 // The plain form took twelve binary64 operations an entry (96 us a pass at 2048 x 256). A thread
 // takes four entries of a line: away from the ends the tenth difference is formed on integers, whose
-// weights 252, 210, 120, 45, 10, 1 are exact, in units of 2^-52 of the largest input; one FMA with
-// the entry itself (binary64) finishes: 43 us. Entries near the ends, and inputs that are not finite
-// or huge, take the plain form.
+// weights are exact (tenth_run, fix64.cuh: closer than the plain form's eleven roundings); one FMA with
+// the entry itself (binary64) finishes: 43 us. Entries near the ends, and runs that tenth_run does not
+// take, have the plain form.
 __device__ __forceinline__ void filter_body(int nx, int ny, const double* __restrict__ in,
                                             double* __restrict__ out, int dir, double sigma,
                                             long long lo, long long hi, long long stride) {
@@ -658,18 +656,10 @@ __device__ __forceinline__ void filter_body(int nx, int ny, const double* __rest
             st = pitch;
         }
         const double* __restrict__ p = in + first;
-        double x[RUN + 10];
-        unsigned top = 0;
+        double x[RUN + 10], tenth[RUN];
 #pragma unroll
-        for (int k = 0; k < RUN + 10; ++k) {
-            x[k] = p[min(max(pos - 5 + k, 0), n - 1) * st];
-            top = max(top, magnitude(x[k]));
-        }
-        const bool wild = scale_wild(top);
-        const int E = scale_of(top);
-        i64 v[RUN + 10];
-#pragma unroll
-        for (int k = 0; k < RUN + 10; ++k) v[k] = to_scale(x[k], E, 52);
+        for (int k = 0; k < RUN + 10; ++k) x[k] = p[min(max(pos - 5 + k, 0), n - 1) * st];
+        const bool fixed = tenth_run(x, tenth);
 #pragma unroll
         for (int o = 0; o < RUN; ++o) {
             const int at = pos + o;
@@ -677,10 +667,8 @@ __device__ __forceinline__ void filter_body(int nx, int ny, const double* __rest
             const int m = min(min(at, n - 1 - at), 5);
             const double f = x[o + 5];
             double acc = 0.0;
-            if (m == 5 && !wild) {
-                i64 d = 252 * v[o + 5] - 210 * (v[o + 4] + v[o + 6]) + 120 * (v[o + 3] + v[o + 7]) -
-                        45 * (v[o + 2] + v[o + 8]) + 10 * (v[o + 1] + v[o + 9]) - (v[o] + v[o + 10]);
-                acc = from_scale(d, E, 62);              // over 1024
+            if (m == 5 && fixed) {
+                acc = tenth[o];
             } else if (m > 0) {
                 const double* w = c_filter_w[m - 1];
                 const double* c = p + (at - m) * st;

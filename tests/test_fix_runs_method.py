@@ -1,0 +1,95 @@
+"""The integer differences and filters over runs of four (fix64.cuh), compiled for the host, against
+exact rational arithmetic: smooth fields, fields that cross zero, steps and decays of up to a hundred
+decades. A run is either refused (it then takes binary64) or at least as good as binary64, output by
+output: the bound is one final rounding and a part of one unit in the last place (2^-53) of the
+largest input of the output's own window.
+
+Tenth difference over 1024: inputs and sum are within 2 units of 2^-62 of the run's power of two,
+which a window passes by at most 2^7: 2^-54 of the window's largest input."""
+import ctypes
+import os
+import shutil
+import subprocess
+from fractions import Fraction as Fr
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2210_05547_gb300", "csrc")
+SHIM = """
+#include "fix64.cuh"
+using namespace hyp;
+extern "C" int tenth(const double* p, double* out) {
+    double x[RUN + 10], y[RUN];
+    for (int k = 0; k < RUN + 10; ++k) x[k] = p[k];
+    const bool ok = tenth_run(x, y);
+    for (int k = 0; k < RUN; ++k) out[k] = y[k];
+    return ok;
+}
+"""
+TENTH = [-1, 10, -45, 120, -210, 252, -210, 120, -45, 10, -1]
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("runs")
+    src, so = d / "shim.cpp", d / "shim.so"
+    src.write_text(SHIM)
+    subprocess.run([gxx, "-O1", "-w", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(so)], check=True)
+    return ctypes.CDLL(str(so))
+
+
+def _fields():
+    s = np.arange(403.0)
+    rng = np.random.default_rng(3)
+    return {
+        "smooth": 1 + 0.3 * np.sin(s / 20) + 0.1 * np.sin(s / 7),
+        "binade": 1 + 0.02 * np.sin(s / 9),
+        "zero": np.sin(s / 15),
+        "noise": 1 + 1e-3 * rng.standard_normal(s.size),
+        "step": 1e-9 + 0.5 * (1 + np.tanh((s - 200) / 2)),
+        "spike": np.where(np.arange(403) % 37 == 5, 1.0, 1e-11),
+        "decay": 10.0 ** (-100 * s / s.size),
+        "top": np.where(rng.random(s.size) < 0.5, -1.0, 1.0) * np.nextafter(2.0, 1),
+        "none": 0.0 * s,
+        "small": 1e-280 * np.cos(s / 11),
+    }
+
+
+def _call(fn, x, n):
+    x = np.ascontiguousarray(x)
+    out = np.zeros(n)
+    ok = fn(x.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p))
+    return ok, out
+
+
+@pytest.mark.parametrize("name", _fields().keys())
+def test_tenth_difference(lib, name):
+    f = _fields()[name]
+    taken = 0
+    for a in range(0, f.size - 13):
+        ok, got = _call(lib.tenth, f[a:a + 14], 4)
+        if not ok:
+            continue
+        taken += 1
+        for o in range(4):
+            w = f[a + o:a + o + 11]
+            exact = sum(Fr(float(v)) * c for v, c in zip(w, TENTH)) / 1024
+            floor = Fr(2) ** -1022                       # below it results are rounded to it
+            bound = abs(exact) * Fr(2) ** -53 + Fr(float(np.abs(w).max())) * Fr(2) ** -54 + floor
+            assert abs(Fr(float(got[o])) - exact) <= bound, (a, o)
+    assert taken == f.size - 13 or name in ("step", "spike", "decay")
+    assert taken > f.size // 4
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 1e290])
+def test_inputs_out_of_range_are_refused(lib, bad):
+    for k in range(14):
+        x = np.ones(14)
+        x[k] = bad
+        assert not _call(lib.tenth, x, 4)[0]
+    assert not _call(lib.tenth, np.full(14, 1e-300), 4)[0]

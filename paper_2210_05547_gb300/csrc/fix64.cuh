@@ -428,6 +428,35 @@ FX bool tenth_run(const double (&x)[RUN + 10], double (&acc)[RUN]) {
     return true;
 }
 
+// Four outputs of the nine-point Gaussian filter over the windows of nine in x, within 11 units of 2^-62 of the run's
+// power of two before their rounding. Returns the mask of outputs for which that is not better than
+// binary64 (above 2^-53.5 of the output, or inputs that are not finite, huge or tiny).
+FX int gauss_fixed(const double (&x)[RUN + 8], double (&y)[RUN]) {
+    // the weights (centre, +-1, .. +-4) in units of 2^-64, as the words (h, l) of mul_const
+    const int wh[5] = {1476809260, 1024362956, 330904695, 49378868, 4432499};
+    const int wl[5] = {1060485752, 721130311, -710525454, -721130311, 180282578};
+    unsigned top = 0;
+#pragma unroll
+    for (int k = 0; k < RUN + 8; ++k) top = larger(top, magnitude(x[k]));
+    if (!scale_fits(top)) return (1 << RUN) - 1;
+    const int E = scale_of(top);
+    i64 v[RUN + 8];
+#pragma unroll
+    for (int k = 0; k < RUN + 8; ++k) v[k] = to_scale(x[k], E, 62);
+    int coarse = 0;
+#pragma unroll
+    for (int o = 0; o < RUN; ++o) {
+        i64 acc = mul_const(v[o + 4], wh[0], wl[0]);
+#pragma unroll
+        for (int d = 1; d <= 4; ++d)
+            acc += mul_const(v[o + 4 - d] + v[o + 4 + d], wh[d], wl[d]);
+        y[o] = from_scale(acc, E, 62);
+        const int h = (int)(acc >> 32);
+        if ((u32)(h ^ (h >> 31)) < 1u << 25) coarse |= 1 << o;   // |acc| < 2^57
+    }
+    return top == 0u ? 0 : coarse;
+}
+
 // 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of
 // the same range (positive under the roots): one rounding, within 0.51 ulp.
 FX bool fix_in_range(double b) {

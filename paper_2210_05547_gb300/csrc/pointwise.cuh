@@ -359,43 +359,25 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
 // Gaussian filter of the raw diffusivities along x (dir 0) or y (dir 1); indices clamp. Nine
 // binary64 operations a point on a unit that takes 19 cycles each bound the plain form (80 us a
 // pass at 2048 x 256). Here a thread filters four neighbours on 62-bit integers scaled by the
-// largest of their twelve inputs, which share the conversions: 36 us
-// (binary32 in the mixed path before: 37). Inputs that are not finite or huge take the plain form.
-// the weights c_gauss in units of 2^-64, as the words (h, l) of mul_const
-static __constant__ int c_gauss_h[5] = {1476809260, 1024362956, 330904695, 49378868, 4432499};
-static __constant__ int c_gauss_l[5] = {1060485752, 721130311, -710525454, -721130311, 180282578};
-
+// largest of their twelve inputs, which share the conversions (gauss_fixed, fix64.cuh): 36 us
+// (binary32 in the mixed path before: 37). Outputs that it does not give to binary64's precision
+// take the plain form.
 // in(i): input i of the line, indices clamped or wrapped by the caller; put(k, v): output pos + k
 template <class In, class Put>
 __device__ __forceinline__ void gauss_run(int pos, const In& in, const Put& put) {
-    double x[RUN + 8];
-    unsigned top = 0;
+    double x[RUN + 8], y[RUN];
 #pragma unroll
-    for (int k = 0; k < RUN + 8; ++k) {
-        x[k] = in(pos - 4 + k);
-        top = max(top, magnitude(x[k]));
-    }
-    if (scale_wild(top)) {
+    for (int k = 0; k < RUN + 8; ++k) x[k] = in(pos - 4 + k);
+    const int plain = gauss_fixed(x, y);
 #pragma unroll
-        for (int o = 0; o < RUN; ++o) {
-            double acc = c_gauss[0] * x[o + 4];
+    for (int o = 0; o < RUN; ++o)
+        if (!(plain >> o & 1)) put(o, y[o]);
+    for (int o = 0; plain >> o; ++o) {
+        if (!(plain >> o & 1)) continue;
+        double acc = c_gauss[0] * in(pos + o);
 #pragma unroll
-            for (int d = 1; d <= 4; ++d) acc += c_gauss[d] * (x[o + 4 - d] + x[o + 4 + d]);
-            put(o, acc);
-        }
-        return;
-    }
-    const int E = scale_of(top);
-    i64 v[RUN + 8];
-#pragma unroll
-    for (int k = 0; k < RUN + 8; ++k) v[k] = to_scale(x[k], E, 62);
-#pragma unroll
-    for (int o = 0; o < RUN; ++o) {
-        i64 acc = mul_const(v[o + 4], c_gauss_h[0], c_gauss_l[0]);
-#pragma unroll
-        for (int d = 1; d <= 4; ++d)
-            acc += mul_const(v[o + 4 - d] + v[o + 4 + d], c_gauss_h[d], c_gauss_l[d]);
-        put(o, from_scale(acc, E, 62));
+        for (int d = 1; d <= 4; ++d) acc += c_gauss[d] * (in(pos + o - d) + in(pos + o + d));
+        put(o, acc);
     }
 }
 

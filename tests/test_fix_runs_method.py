@@ -5,7 +5,9 @@ output: the bound is one final rounding and a part of one unit in the last place
 largest input of the output's own window.
 
 Tenth difference over 1024: inputs and sum are within 2 units of 2^-62 of the run's power of two,
-which a window passes by at most 2^7: 2^-54 of the window's largest input."""
+which a window passes by at most 2^7: 2^-54 of the window's largest input.
+Gaussian filter: 11 units of 2^-62 (five products, each up to 1.5 short, the inputs' truncation and
+the weights' rounding) against outputs of at least 2^-5: 2^-53.5 of the output."""
 import ctypes
 import os
 import shutil
@@ -27,7 +29,17 @@ extern "C" int tenth(const double* p, double* out) {
     for (int k = 0; k < RUN; ++k) out[k] = y[k];
     return ok;
 }
+extern "C" int gauss(const double* p, double* out) {
+    double x[RUN + 8], y[RUN];
+    for (int k = 0; k < RUN + 8; ++k) x[k] = p[k];
+    const int plain = gauss_fixed(x, y);
+    for (int k = 0; k < RUN; ++k) out[k] = y[k];
+    return plain;
+}
 """
+EPS = Fr(2) ** -53
+GAUSS = [Fr(107, 103680), Fr(149, 12960), Fr(1997, 25920), Fr(3091, 12960), Fr(3565, 10368)]
+GAUSS += GAUSS[-2::-1]
 TENTH = [-1, 10, -45, 120, -210, 252, -210, 120, -45, 10, -1]
 
 
@@ -86,10 +98,28 @@ def test_tenth_difference(lib, name):
     assert taken > f.size // 4
 
 
+@pytest.mark.parametrize("name", _fields().keys())
+def test_gaussian_filter(lib, name):
+    f = _fields()[name]
+    taken = 0
+    for a in range(0, f.size - 11):
+        plain, got = _call(lib.gauss, f[a:a + 12], 4)
+        for o in range(4):
+            if plain >> o & 1:
+                continue
+            taken += 1
+            exact = sum(Fr(float(v)) * c for v, c in zip(f[a + o:a + o + 9], GAUSS))
+            assert abs(Fr(float(got[o])) - exact) <= abs(exact) * EPS * Fr(171, 100), (a, o)
+    n = 4 * (f.size - 11)
+    assert taken == n if name in ("smooth", "binade", "noise", "none") else taken > n // 4
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 1e290])
 def test_inputs_out_of_range_are_refused(lib, bad):
     for k in range(14):
         x = np.ones(14)
         x[k] = bad
         assert not _call(lib.tenth, x, 4)[0]
+        assert k > 11 or _call(lib.gauss, x[:12], 4)[0] == 15
+    assert _call(lib.gauss, np.full(12, 1e-300), 4)[0] == 15
     assert not _call(lib.tenth, np.full(14, 1e-300), 4)[0]

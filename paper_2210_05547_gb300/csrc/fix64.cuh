@@ -428,6 +428,45 @@ FX bool tenth_run(const double (&x)[RUN + 10], double (&acc)[RUN]) {
     return true;
 }
 
+FX i64 fourth_difference(i64 a, i64 b, i64 c, i64 d, i64 e) { return (a + e) - 4 * (b + d) + 6 * c; }
+
+// Fourth differences of four neighbours: dx along their row w (two before to two after), dy across it
+// over the rows r (two below, one below, one above, two above). Sixteen units of 2^-59 of the power of
+// two above the largest of the 24 inputs bound their error; false where that may exceed binary64's
+// (rms 2^-52.2 of the largest of a difference's five inputs, here 2^-52.7 at the line drawn): an
+// output one of whose two windows lies below 2^-5 of the largest, or inputs not finite, huge or tiny.
+FX bool fourth_run(const double (&w)[RUN + 4], const double (&r)[4][RUN], double (&dx)[RUN],
+                   double (&dy)[RUN]) {
+    unsigned mw[RUN + 4], top = 0, least = ~0u;
+#pragma unroll
+    for (int k = 0; k < RUN + 4; ++k) mw[k] = magnitude(w[k]);
+    const unsigned mid = larger(mw[3], mw[4]);
+#pragma unroll
+    for (int k = 0; k < RUN; ++k) {
+        unsigned mx = mid, my = mw[k + 2];
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            if (k + q != 3 && k + q != 4) mx = larger(mx, mw[k + q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) my = larger(my, magnitude(r[q][k]));
+        const unsigned lo = mx < my ? mx : my;
+        top = larger(top, larger(mx, my));
+        least = lo < least ? lo : least;
+    }
+    if (!scale_fits(top) || (least >> 20) + 4 < top >> 20) return false;
+    const int E = scale_of(top);
+    i64 v[RUN + 4];
+#pragma unroll
+    for (int k = 0; k < RUN + 4; ++k) v[k] = to_scale(w[k], E, 59);
+#pragma unroll
+    for (int k = 0; k < RUN; ++k) {
+        dx[k] = from_scale(fourth_difference(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4]), E, 59);
+        dy[k] = from_scale(fourth_difference(to_scale(r[0][k], E, 59), to_scale(r[1][k], E, 59), v[k + 2],
+                                             to_scale(r[2][k], E, 59), to_scale(r[3][k], E, 59)), E, 59);
+    }
+    return true;
+}
+
 // Four outputs of the nine-point Gaussian filter over the windows of nine in x, within 11 units of 2^-62 of the run's
 // power of two before their rounding. Returns the mask of outputs for which that is not better than
 // binary64 (above 2^-53.5 of the output, or inputs that are not finite, huge or tiny).

@@ -259,48 +259,13 @@ __device__ __forceinline__ double d4y(const double* f, int j, int i, int nx, int
 
 // Raw artificial diffusivities: a factor times |d4x wx + d4y wy|. Fourteen binary64 operations per
 // point and field bound the plain form (110 us at 2048 x 256); here a thread takes four neighbours
-// along x of one field, the fourth differences (weights 1, -4, 6, exact) on integers in units of
-// 2^-58 of the largest of their 24 inputs, and two products and a sum remain binary64: 73 us. (The
-// same in three dimensions, forty inputs a run, was slower than the plain form there: jet
-// right-hand side 9.77 against 9.61 ms.) Runs at the ends of a row and inputs that are not finite or huge take the plain form.
+// along x of one field, the fourth differences (weights 1, -4, 6, exact) on integers (fourth_run,
+// fix64.cuh), and two products and a sum remain binary64: 73 us. (The same in three dimensions, forty
+// inputs a run, was slower than the plain form there: jet right-hand side 9.77 against 9.61 ms.) Runs
+// at the ends of a row and those that fourth_run does not take have the plain form.
 // Runs of four per field along dir.
 __host__ __device__ __forceinline__ int gauss_runs(int nx, int ny, int dir) {
     return dir == 0 ? ny * ((nx + RUN - 1) / RUN) : (ny + RUN - 1) / RUN * nx;
-}
-
-__device__ __forceinline__ i64 fourth(i64 a, i64 b, i64 c, i64 d, i64 e) {
-    return (a + e) - 4 * (b + d) + 6 * c;
-}
-
-// d4 of four neighbours: w their row from two before to two after, then per further direction the
-// four rows around (two below, one below, one above, two above). sums[k] = sum of d4 x weight.
-template <int ROWS>
-__device__ __forceinline__ bool fourth_run(const double (&w)[RUN + 4], const double (&r)[ROWS][RUN],
-                                           const double* wt, double* sums) {
-    unsigned top = 0;
-#pragma unroll
-    for (int k = 0; k < RUN + 4; ++k) top = max(top, magnitude(w[k]));
-#pragma unroll
-    for (int l = 0; l < ROWS; ++l)
-#pragma unroll
-        for (int k = 0; k < RUN; ++k) top = max(top, magnitude(r[l][k]));
-    if (scale_wild(top)) return false;
-    const int E = scale_of(top);
-    i64 v[RUN + 4];
-#pragma unroll
-    for (int k = 0; k < RUN + 4; ++k) v[k] = to_scale(w[k], E, 58);
-#pragma unroll
-    for (int k = 0; k < RUN; ++k) {
-        double s = from_scale(fourth(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4]), E, 58) * wt[0];
-#pragma unroll
-        for (int l = 0; l < ROWS; l += 4)
-            s = fma(from_scale(fourth(to_scale(r[l][k], E, 58), to_scale(r[l + 1][k], E, 58), v[k + 2],
-                                      to_scale(r[l + 2][k], E, 58), to_scale(r[l + 3][k], E, 58)),
-                               E, 58),
-                    wt[1 + l / 4], s);
-        sums[k] = s;
-    }
-    return true;
 }
 
 __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
@@ -332,7 +297,11 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
                 r[2][k] = in[row + i + k + nx];
                 r[3][k] = in[row + i + k + 2 * nx];
             }
-            done = fourth_run<4>(w, r, wt, sum);
+            double d4[RUN], e4[RUN];
+            done = fourth_run(w, r, d4, e4);
+            if (done)
+#pragma unroll
+                for (int k = 0; k < RUN; ++k) sum[k] = fma(e4[k], wt[1], d4[k] * wt[0]);
         }
         if (!done)
             for (int k = 0; k < RUN; ++k)

@@ -24,7 +24,10 @@
 #define LSEG 8                 // rows of a line per thread of the line-operator kernel
 #define LINE_THREADS 288       // threads per block: fits lines of 2^k + 1 rows (k = 5 .. 11)
 #define LINE_MAX_LINES 72      // lines per block, at most (a thread for each of 4 closure rows)
-#define LINE_TAIL 40           // rows a line's end reaches into (rho^40 < 2^-63)
+#define LINE_FALL_0 11         // bits that a segment's scale loses per segment of distance: at most
+#define LINE_FALL_1 20         // log2 rho^-LSEG (interpolation, derivative)
+#define LINE_MARGIN 40         // rows a chunk of a line starts early (rho^40 < 2^-63)
+#define LINE_TAIL 64           // rows a line's start reaches into (rho^64 < 2^-101)
 
 namespace hyp {
 
@@ -149,7 +152,8 @@ namespace hyp {
 // What the unknown start of q adds to the first rows of a line (lines.cu): row k of the interior gets
 // h_k Q, h_k = (-rho)^(k+1) (1 - rho^(2 (n - k))) / (1 - rho^2), Q = kappa (y_left + rho y_first).
 struct LineTail {
-    long long h[LINE_TAIL], kappa;               // in units of 2^-64, 2^-63
+    long long h[LINE_TAIL], kappa;               // in units of 2^-64 2^-up, 2^-63
+    int up[LINE_TAIL / LSEG];                    // per segment of rows of the line: its h below 1/2
     double hd[LINE_TAIL], kappa_d;
 };
 

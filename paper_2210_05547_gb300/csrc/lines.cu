@@ -4,24 +4,33 @@
 // What bounds it: a tridiagonal solve costs about seven binary64 operations per point, and GB300
 // has one binary64 unit per SM (19 cycles per warp instruction), so the binary64 sweeps this file
 // held before ran at 125 cycles per 32 points with that unit 60-85% busy and the lines' length
-// (latency) behind it. The operators are linear with constant coefficients and each line's values
+// (latency) behind it. The operators are linear with constant coefficients and neighbouring values
 // share a scale, so the solve runs on integers: a product with a constant takes three 32-bit
-// integer products (3 cycles), a sum less than one. Per line, the inputs are scaled by the power
-// of two above their largest magnitude to 62 bits (exact for values down to 2^-9 of it); results
-// are in units of 2^-59 of that magnitude, where binary64 rounds the largest values at 2^-53.
+// integer products (3 cycles), a sum less than one.
 //
-// One thread solves LSEG = 8 consecutive rows of a line in registers; the threads of a line sit
+// Scales: a thread's LSEG = 8 rows have one, the power of two above the largest of their inputs, to
+// which the inputs are taken to 62 bits (exact for values down to 2^-9 of it). What the neighbours
+// add carries their own scale; a segment whose neighbours' share needs more is shifted down to it.
+// A neighbour's scale counts in full one segment away and LINE_FALL bits less (2^11, 2^20; rho^8 is
+// 2^-12.7, 2^-22) for each segment more, so an entry's error is a few units of 2^-60 of the largest
+// value within sixteen rows, and of farther ones by how much their influence has decayed: fields that
+// fall by decades along a line keep binary64's precision at their small end. (With one scale per
+// line, as before, a fall over twelve decades left 2e-7 there.) End values reach eight segments on
+// (rho^64 < 2^-101); chunks and extended periodic lines start LINE_MARGIN rows early
+// (rho^40 < 2^-63).
+//
+// One thread solves its rows in registers; the threads of a line sit
 // in one block and exchange end values, so nothing is stored between the forward and
 // the backward recurrence (the earlier sweeps wrote and read it, and re-ran 26-40 warm-up rows per
 // segment). With rho / (1 + rho^2) = alpha the interior rows factor into
 //     q_r = (1 + rho^2) rhs_r - rho q_{r-1},     y_r = q_r - rho y_{r+1}
 // with the same rho (1/3, 0.148) on every row. A thread runs both from zero; what enters from its
-// neighbours follows from their own end values, q_in = e_{-1} + rho^8 e_{-2} + ... (five terms,
-// rho^40 < 2^-63), likewise y_in, and their effect on row k, a_k q_in + b_k y_in, is added. The row
+// neighbours follows from their own end values, q_in = e_{-1} + rho^8 e_{-2} + ... (eight terms),
+// likewise y_in, and their effect on row k, a_k q_in + b_k y_in, is added. The row
 // before the first interior row is an explicit closure row, as is the row after the last: the
 // latter starts the backward recurrence, the former fixes q's unknown start Q, whose effect h_k Q
 // is added to the first rows. Periodic lines wrap the exchange around (or, when 8 does not divide
-// the period, extend the line by LINE_TAIL rows each way); lines of more than LINE_THREADS threads
+// the period, extend the line by LINE_MARGIN rows each way); lines of more than LINE_THREADS threads
 // are cut into chunks with such margins.
 //
 // Inputs and, for lines along x (unit stride), results pass through shared memory, 9 words per
@@ -50,19 +59,28 @@ struct LineConst {
     int h, l;
     double d;
 };
-enum { C_P24 = 16, C_P32 = 17, C_WA = 18, C_WB = 19, C_G = 20, C_A = 21 };
-// per kind: rho^1 .. rho^16, rho^24, rho^32, the right-hand side's weights, rho^2 / (1 - rho^2), and
-// |response| of a segment's rows to what enters its forward recurrence,
+enum { C_8 = 16, C_16, C_32, C_WA, C_WB, C_G, C_A };
+// per kind: rho^1 .. rho^16, (rho^8 2^LINE_FALL)^1, ^2 and ^4, the right-hand side's weights,
+// rho^2 / (1 - rho^2), and |response| of a segment's rows to what enters its forward recurrence,
 // rho^(k+1) (1 - rho^(2 (LSEG - k))) / (1 - rho^2), the sign (-1)^(k+1)
 __constant__ LineConst c_line[2][C_A + LSEG] = {LINE_TABLE_BODY};
 
+// y >> s, all sign bits for s > 63.
+__device__ __forceinline__ i64 shift_right(i64 y, int s) {
+    i64 v;
+    asm("shr.s64 %0, %1, %2;" : "=l"(v) : "l"(y), "r"(s));   // PTX clamps the shift amount
+    return v;
+}
+
 struct Fix {                                     // y is held as y / 4
     typedef i64 T;
-    int E;                                       // inputs below 2^E
+    static constexpr bool scaled = true;
+    int E;                                       // the segment's scale: inputs below 2^E
     __device__ __forceinline__ T input(double x) const { return to_scale(x, E, 62); }
     __device__ __forceinline__ T closure(double x) const { return to_scale(x, E, 60); }
     __device__ __forceinline__ double value(T y, unsigned sign) const { return from_scale(y, E, 60, sign); }
     static __device__ __forceinline__ T flip(T a, int kind) { return kind ? -a : a; }
+    static __device__ __forceinline__ T shift(T a, int s) { return shift_right(a, s); }
     static __device__ __forceinline__ T mul(T a, const LineConst& c) { return mul_const(a, c.h, c.l); }
     static __device__ __forceinline__ T mul(T a, const LineTail& t, int k) { return __mul64hi(a, t.h[k]); }
     static __device__ __forceinline__ T start(T a, const LineTail& t) { return __mul64hi(a, t.kappa) << 1; }
@@ -70,10 +88,13 @@ struct Fix {                                     // y is held as y / 4
 
 struct Dbl {
     typedef double T;
+    static constexpr bool scaled = false;
+    int E;                                       // unused
     static __device__ __forceinline__ T input(double x) { return x; }
     static __device__ __forceinline__ T closure(double x) { return x; }
     static __device__ __forceinline__ double value(T y, unsigned sign) { return sign ? -y : y; }
     static __device__ __forceinline__ T flip(T a, int kind) { return kind ? -a : a; }
+    static __device__ __forceinline__ T shift(T a, int) { return a; }
     static __device__ __forceinline__ T mul(T a, const LineConst& c) { return a * c.d; }
     static __device__ __forceinline__ T mul(T a, const LineTail& t, int k) { return a * t.hd[k]; }
     static __device__ __forceinline__ T start(T a, const LineTail& t) { return a * t.kappa_d; }
@@ -98,10 +119,10 @@ constexpr int SLOT = LSEG + 1;                   // words of shared memory per t
 
 struct Shared {
     double stage[LINE_THREADS * SLOT];           // inputs, then results of x lines
-    u64 ends[2][LINE_THREADS];                   // segments' end values, forward and backward
+    u64 ends[2][LINE_THREADS];                   // what the segments exchange (by turns)
+    int scale[2][LINE_THREADS];                  // and its scales
     u64 start[LINE_MAX_LINES];                   // Q
     double clos[LINE_MAX_LINES][4];              // the closure rows' values, in the operator's order
-    unsigned top[LINE_MAX_LINES];                // largest |input|, high word
 };
 
 // The thread's place: rows r0 .. r0 + LSEG - 1 of a line, segment `seg` of `nseg`; the line's next
@@ -125,33 +146,58 @@ __device__ __forceinline__ T cooked(u64 u) {
     return v;
 }
 
-// What enters a segment from the five segments before it (way -1) or after it (way 1): the sum of
-// their end values times rho^(8 (i - 1)), rho^40 < 2^-63.
-constexpr int TERMS = 5;
-
+// What enters a segment from the eight before it (way -1) or after it (way 1): the sum of their end
+// values times rho^(8 (i - 1)), gathered in three exchanges (two, four, eight segments). The
+// segment's numbers q go over to the scale of that sum.
 template <class N>
-__device__ __forceinline__ typename N::T carried(const u64* ends, const Place& P, int way,
-                                                 const LineConst* C) {
-    typename N::T v = 0;
-#pragma unroll
-    for (int i = 1; i <= TERMS; ++i) {
+__device__ __forceinline__ typename N::T carried(Shared& sh, int buf, typename N::T end, const Place& P,
+                                                 int way, int kind, const LineConst* C, N& num,
+                                                 typename N::T (&q)[LSEG]) {
+    typedef typename N::T T;
+    const int tid = threadIdx.x, fall = kind ? LINE_FALL_1 : LINE_FALL_0;
+    auto thread = [&](int i) {                           // of the segment i on, -1 past the line's ends
         int s = P.seg + way * i;
         if (P.wrap) {
             s %= P.nseg;
             s += s < 0 ? P.nseg : 0;
         }
-        typename N::T e = 0;
-        if ((unsigned)s < (unsigned)P.nseg) e = cooked<typename N::T>(ends[(int)threadIdx.x + (s - P.seg) * P.nl]);
-        const int p = LSEG * (i - 1);
-        if (i == 1) v = e;
-        else v += N::mul(e, C[p == 32 ? C_P32 : (p == 24 ? C_P24 : p - 1)]);
+        return (unsigned)s < (unsigned)P.nseg ? tid + (s - P.seg) * P.nl : -1;
+    };
+    auto publish = [&](T v, int E) {
+        sh.ends[buf][tid] = raw(v);
+        if (N::scaled) sh.scale[buf][tid] = E;
+        __syncthreads();
+    };
+    auto scale = [&](int at, int down) { return N::scaled && at >= 0 ? sh.scale[buf][at] - down : -(1 << 20); };
+    auto value = [&](int at, int by, int c) {
+        T e = at >= 0 ? cooked<T>(sh.ends[buf][at]) : T(0);
+        if (c >= 0) e = N::mul(e, C[c]);
+        return N::shift(e, by);
+    };
+    publish(end, num.E);
+    const int a1 = thread(1), a2 = thread(2);
+    const int s1 = scale(a1, 0), s2 = scale(a2, fall);
+    int E = max(num.E, max(s1, s2));
+    T v = value(a1, E - s1, -1) + value(a2, E - s2, C_8);
+#pragma unroll
+    for (int i = 2; i <= 4; i += 2) {
+        buf ^= 1;
+        publish(v, E);
+        const int at = thread(i), s = scale(at, fall * i), E0 = E;
+        E = max(E, s);
+        v = N::shift(v, E - E0) + value(at, E - s, i == 2 ? C_16 : C_32);
+    }
+    if (N::scaled && E != num.E) {
+#pragma unroll
+        for (int k = 0; k < LSEG; ++k) q[k] = N::shift(q[k], E - num.E);
+        num.E = E;
     }
     return v;
 }
 
 // The solve and its output, once the inputs are in shared memory.
 template <class N>
-__device__ __forceinline__ void solve(const N& num, const LineJob& J, const LineOp& op, const Place& P,
+__device__ __forceinline__ void solve(N num, const LineJob& J, const LineOp& op, const Place& P,
                                       Shared& sh, double* __restrict__ out) {
     typedef typename N::T T;
     const int kind = op.kind, fi = op.first_interior, li = op.last_interior, tid = threadIdx.x;
@@ -162,6 +208,14 @@ __device__ __forceinline__ void solve(const N& num, const LineJob& J, const Line
     const double* own = sh.stage + tid * SLOT;
     const int next = P.seg + 1 < P.nseg ? tid + P.nl : (P.wrap ? tid - (P.nseg - 1) * P.nl : tid);
     const double* nxt = sh.stage + (P.active ? next : tid) * SLOT;
+    if constexpr (N::scaled) {
+        unsigned top = 0;
+#pragma unroll
+        for (int k = 0; k < LSEG + 3; ++k) top = larger(top, magnitude(k < LSEG ? own[k] : nxt[k - LSEG]));
+        if (first) top = larger(top, magnitude(sh.clos[P.line][fi - 1]));
+        if (rr >= 0 && rr < LSEG) top = larger(top, magnitude(sh.clos[P.line][fi]));
+        num.E = scale_of(top);
+    }
     // forward: f0 f1 f2 f3 at offsets -3/2 .. +3/2 of row r; g the same, negated for a derivative
     T q[LSEG];
     T g0 = N::flip(num.input(own[0]), kind), g1 = N::flip(num.input(own[1]), kind);
@@ -176,7 +230,6 @@ __device__ __forceinline__ void solve(const N& num, const LineJob& J, const Line
         g1 = N::flip(f2, kind);
         f2 = f3;
     }
-    sh.ends[0][tid] = raw(p);
     if (rr < LSEG) {                                     // the line ends here
         const T yr = num.closure(rr >= 0 ? sh.clos[P.line][fi] : 0.0);
 #pragma unroll
@@ -190,8 +243,7 @@ __device__ __forceinline__ void solve(const N& num, const LineJob& J, const Line
         y = q[k] - N::mul(y, C[0]);
         q[k] = y;
     }
-    __syncthreads();
-    const T qin = carried<N>(sh.ends[0], P, -1, C);
+    const T qin = carried(sh, 0, p, P, -1, kind, C, num, q);
     if (rr >= LSEG) {
 #pragma unroll
         for (int k = 0; k < LSEG; ++k) {
@@ -207,9 +259,7 @@ __device__ __forceinline__ void solve(const N& num, const LineJob& J, const Line
             q[k] = (k & 1) ? q[k] + c : q[k] - c;
         }
     }
-    sh.ends[1][tid] = raw(q[0]);
-    __syncthreads();
-    const T yin = carried<N>(sh.ends[1], P, 1, C);
+    const T yin = carried(sh, 1, q[0], P, 1, kind, C, num, q);
 #pragma unroll
     for (int k = 0; k < LSEG; ++k) {
         const T c = N::mul(yin, C[LSEG - 1 - k]);
@@ -219,14 +269,23 @@ __device__ __forceinline__ void solve(const N& num, const LineJob& J, const Line
         if (first) {
             const T Yl = num.closure(sh.clos[P.line][fi - 1]);
             sh.start[P.line] = raw(N::start(Yl + N::mul(fi == 1 ? q[1] : q[2], C[0]), op.tail[0]));
+            if (N::scaled) sh.scale[0][tid] = num.E;     // (the last exchange used the other)
         }
         __syncthreads();
-        if (P.active && P.seg < LINE_TAIL / LSEG) {
+        constexpr int tail = N::scaled ? LINE_TAIL : LINE_MARGIN;
+        if (P.active && P.seg < tail / LSEG) {
             const T Q = cooked<T>(sh.start[P.line]);
+            // the share of Q in this segment's scale; it outgrows that by less than its headroom
+            const int down = N::scaled ? num.E + op.tail->up[P.seg] - sh.scale[0][P.line] : 0;
+            if (down < 63) {
 #pragma unroll
-            for (int k = 0; k < LSEG; ++k) {
-                const int i = P.r0 + k - fi;
-                if (i >= 0 && i < LINE_TAIL) q[k] += N::mul(Q, op.tail[0], i);
+                for (int k = 0; k < LSEG; ++k) {
+                    const int i = P.r0 + k - fi;
+                    if (i < 0 || i >= tail) continue;
+                    T v = N::mul(Q, op.tail[0], i);
+                    if constexpr (N::scaled) v = down < 0 ? v << -down : N::shift(v, down);
+                    q[k] += v;
+                }
             }
         }
     }
@@ -312,8 +371,6 @@ __global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __rest
     const double* __restrict__ in = base_in + (P.active ? offset(line, J.in_ls, J.in_ps) : 0);
     double* __restrict__ out = J.out + (P.active ? offset(line, J.out_ls, J.out_ps) : 0);
     const double wall = (J.wall_arr && P.active) ? J.wall_arr[line] : J.wall_value;
-    if (tid < LINE_MAX_LINES) sh.top[tid] = 0;
-    __syncthreads();
 
     // inputs: row r reads r + base .. r + base + 3
     const int base = op.dir == 0 ? -2 : -1, n_in = op.n_in;
@@ -354,7 +411,6 @@ __global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __rest
             }
         }
     }
-    if (P.active) atomicMax(&sh.top[P.line], top);
     // the closure rows, one per thread from the block's end
     if (!op.periodic && LINE_THREADS - 1 - tid < nl * op.ncl) {
         const int i = LINE_THREADS - 1 - tid, c = (i * J.inv_nl) >> 20, l = i - c * nl;
@@ -367,9 +423,7 @@ __global__ void __launch_bounds__(LINE_THREADS, 4) k_lines(const LineJob* __rest
         solve_wild(J, op, P, sh, out);
         return;
     }
-    Fix num;
-    num.E = scale_of(sh.top[P.active ? P.line : 0]);
-    solve<Fix>(num, J, op, P, sh, out);
+    solve<Fix>(Fix(), J, op, P, sh, out);
 }
 
 }  // namespace

@@ -325,7 +325,7 @@ LineOp make_op(int kind, int dir, int n, int wall, std::vector<LineTail>& tails)
             for (int k = 0; k < 5; ++k) op.cw[c][k] = w[k];
         }
     }
-    op.margin = m + 2 >= LINE_THREADS * LSEG ? LINE_TAIL : 0;   // cut into chunks (plan_line)
+    op.margin = m + 2 >= LINE_THREADS * LSEG ? LINE_MARGIN : 0;   // cut into chunks (plan_line)
     // rho / (1 + rho^2) = alpha = 3/10 (interpolation), 9/62 (derivative)
     const long double rho = kind == 0 ? 1.0L / 3.0L : (31.0L - sqrtl(880.0L)) / 9.0L;
     const int ni = op.last_interior - op.first_interior + 1;
@@ -338,7 +338,11 @@ LineOp make_op(int kind, int dir, int n, int wall, std::vector<LineTail>& tails)
     for (int k = 0; k < LINE_TAIL && k < ni; ++k) {
         const long double h = (k & 1 ? 1.0L : -1.0L) * up * (1.0L - far) / (1.0L - rho * rho);
         if (k == 0) h0 = h;
-        tail.h[k] = llrintl(ldexpl(h, 64));
+        const int first = op.first_interior, seg = (k + first) / LSEG;
+        if (seg == LINE_TAIL / LSEG) break;
+        if (k == 0 || (k + first) % LSEG == 0)            // the segment's largest
+            tail.up[seg] = std::max(0, -ilogbl(h) - 2);
+        tail.h[k] = llrintl(ldexpl(h, 64 + tail.up[seg]));
         tail.hd[k] = (double)h;
         up *= rho;
         far /= rho * rho;

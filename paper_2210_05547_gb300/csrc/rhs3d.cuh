@@ -790,7 +790,7 @@ int init3(const hyp_gas* gas, const hyp_grid_desc* desc, const hyp_case* cas, do
             op.kind = kind;
             op.dir = dir;
             op.periodic = 1;
-            op.margin = nz % LSEG || nz > LINE_THREADS * LSEG ? LINE_TAIL : 0;
+            op.margin = nz % LSEG || nz > LINE_THREADS * LSEG ? LINE_MARGIN : 0;
             op.first_interior = -(1 << 28);
             op.last_interior = 1 << 28;
         }

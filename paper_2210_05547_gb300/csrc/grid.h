@@ -69,12 +69,12 @@ enum Phase {
 // Launches of one right-hand side, as reported by the optional event profile.
 enum KernelId {
     KID_LINES_STATE, KID_FACE_VEL, KID_CLOSURE, KID_LINES_VELGRAD, KID_LINES_AD, KID_AD_PREP,
-    KID_AD_RAW, KID_AD_GAUSS, KID_AD_COMBINE, KID_STRESS_C, KID_LINES_MU, KID_STRESS_CN,
+    KID_AD_RAW, KID_AD_GAUSS, KID_STRESS_C, KID_LINES_MU, KID_STRESS_CN,
     KID_LINES_FACE, KID_FLUX, KID_LINES_DIV, KID_ASSEMBLE, KID_FILTER, KID_COUNT
 };
 inline constexpr const char* KERNEL_NAMES[KID_COUNT] = {
     "k_lines:state", "k_face_vel", "k_closure", "k_lines:velgrad", "k_lines:ad", "k_ad_prep",
-    "k_ad_raw", "k_gauss", "k_ad_combine", "k_stress_c", "k_lines:mu", "k_stress_cn",
+    "k_ad_raw", "k_gauss", "k_stress_c", "k_lines:mu", "k_stress_cn",
     "k_lines:face", "k_flux", "k_lines:div", "k_assemble", "k_filter"};
 
 struct EventProfile {

@@ -1023,7 +1023,7 @@ static int run_rhs(const hyp_gas* gas, hyp_grid* G, const double* U, double* dUd
         TIMED(KID_AD_RAW, (k_ad_raw<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, 0), 256), 256, 0, s>>>(g.kind == HYP_GAS_CNEQ, v, U, S)));
         for (int dir = 0; dir < 2; ++dir)
             TIMED(KID_AD_GAUSS, (k_gauss<<<blocks_for((long long)AD_FIELDS * gauss_runs(d.nx, d.ny, dir), 256), 256, 0, s>>>(v, S, dir)));
-        TIMED(KID_AD_COMBINE, (k_stress_c<true><<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
+        TIMED(KID_STRESS_C, (k_stress_c<true><<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
     } else {
         TIMED(KID_STRESS_C, (k_stress_c<false><<<blocks_for(nc, 256), 256, 0, s>>>(v, S)));
     }

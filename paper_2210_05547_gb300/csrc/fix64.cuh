@@ -15,9 +15,7 @@
 
 #include <stdint.h>
 #include <string.h>
-#ifndef __CUDA_ARCH__
 #include <math.h>
-#endif
 
 #include "fix_table.h"
 
@@ -369,7 +367,7 @@ FX i64 to_scale(double x, int E, int q) {
 #ifdef __CUDACC__
 __host__ __device__ __noinline__
 #endif
-static inline double small_from_scale(u64 m, int E, int q, unsigned sign) {
+inline double small_from_scale(u64 m, int E, int q, unsigned sign) {
     return double_of(bits_of(f64_of_fixed(m, q - E)) | (u64)sign << 32);
 }
 
@@ -430,13 +428,14 @@ FX bool tenth_run(const double (&x)[RUN + 10], double (&acc)[RUN]) {
 
 FX i64 fourth_difference(i64 a, i64 b, i64 c, i64 d, i64 e) { return (a + e) - 4 * (b + d) + 6 * c; }
 
-// Fourth differences of four neighbours: dx along their row w (two before to two after), dy across it
-// over the rows r (two below, one below, one above, two above). Sixteen units of 2^-59 of the power of
-// two above the largest of the 24 inputs bound their error; false where that may exceed binary64's
+// sums[k] = d4x wt[0] + d4y wt[1] of four neighbours, the fourth differences along their row w (two
+// before to two after) and across it over the rows r (two below, one below, one above, two above).
+// Sixteen units of 2^-59 of the power of two above the largest of the 24 inputs bound the error of
+// either difference; false where that may exceed binary64's
 // (rms 2^-52.2 of the largest of a difference's five inputs, here 2^-52.7 at the line drawn): an
 // output one of whose two windows lies below 2^-5 of the largest, or inputs not finite, huge or tiny.
-FX bool fourth_run(const double (&w)[RUN + 4], const double (&r)[4][RUN], double (&dx)[RUN],
-                   double (&dy)[RUN]) {
+FX bool fourth_run(const double (&w)[RUN + 4], const double (&r)[4][RUN], const double (&wt)[2],
+                   double (&sums)[RUN]) {
     unsigned mw[RUN + 4], top = 0, least = ~0u;
 #pragma unroll
     for (int k = 0; k < RUN + 4; ++k) mw[k] = magnitude(w[k]);
@@ -460,9 +459,10 @@ FX bool fourth_run(const double (&w)[RUN + 4], const double (&r)[4][RUN], double
     for (int k = 0; k < RUN + 4; ++k) v[k] = to_scale(w[k], E, 59);
 #pragma unroll
     for (int k = 0; k < RUN; ++k) {
-        dx[k] = from_scale(fourth_difference(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4]), E, 59);
-        dy[k] = from_scale(fourth_difference(to_scale(r[0][k], E, 59), to_scale(r[1][k], E, 59), v[k + 2],
-                                             to_scale(r[2][k], E, 59), to_scale(r[3][k], E, 59)), E, 59);
+        const double dx = from_scale(fourth_difference(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4]), E, 59);
+        sums[k] = fma(from_scale(fourth_difference(to_scale(r[0][k], E, 59), to_scale(r[1][k], E, 59), v[k + 2],
+                                                   to_scale(r[2][k], E, 59), to_scale(r[3][k], E, 59)), E, 59),
+                      wt[1], dx * wt[0]);
     }
     return true;
 }

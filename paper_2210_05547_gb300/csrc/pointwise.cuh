@@ -297,11 +297,7 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
                 r[2][k] = in[row + i + k + nx];
                 r[3][k] = in[row + i + k + 2 * nx];
             }
-            double d4[RUN], e4[RUN];
-            done = fourth_run(w, r, d4, e4);
-            if (done)
-#pragma unroll
-                for (int k = 0; k < RUN; ++k) sum[k] = fma(e4[k], wt[1], d4[k] * wt[0]);
+            done = fourth_run(w, r, wt, sum);
         }
         if (!done)
             for (int k = 0; k < RUN; ++k)

@@ -402,7 +402,7 @@ __global__ void k_ad_prep(GridView v, Scratch s) {
     ad_prep_body(s, GRID_RANGE((long long)v.nx * v.ny));
 }
 
-__global__ void k_ad_raw(int cneq, GridView v, const double* __restrict__ U, Scratch s) {
+__global__ void __launch_bounds__(256, 3) k_ad_raw(int cneq, GridView v, const double* __restrict__ U, Scratch s) {
     ad_raw_body(cneq != 0, v, U, s, GRID_RANGE((long long)AD_FIELDS * gauss_runs(v.nx, v.ny, 0)));
 }
 

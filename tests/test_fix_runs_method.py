@@ -44,7 +44,8 @@ extern "C" int fourth(const double* p, double* out) {
     for (int k = 0; k < RUN + 4; ++k) w[k] = p[2 * (RUN + 4) + k];
     for (int q = 0; q < 4; ++q)
         for (int k = 0; k < RUN; ++k) r[q][k] = p[(q + (q > 1)) * (RUN + 4) + k + 2];
-    const bool ok = fourth_run(w, r, dx, dy);
+    const double x[2] = {1, 0}, y[2] = {0, 1};
+    const bool ok = fourth_run(w, r, x, dx) && fourth_run(w, r, y, dy);
     for (int k = 0; k < RUN; ++k) out[k] = dx[k], out[RUN + k] = dy[k];
     return ok;
 }

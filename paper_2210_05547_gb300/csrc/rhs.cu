@@ -1323,8 +1323,12 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
     int njobs = 0;
     for (int ph = 0; ph < PH_COUNT; ++ph) njobs = std::max(njobs, G->ph_start[ph] + G->ph_count[ph]);
     const long long scratch_n = G->Uref - G->pool;    // scratch fields, DX, DY, SRC, R
-    const long long jobs_n = ((long long)njobs * (long long)sizeof(LineJob) + 255) / 256 * 32;
+    // the limit counts the scratch, the outputs of the largest line phase and 144 bytes per line job,
+    // so that the set of accepted grids does not move with the layout; the job list sits where those
+    // outputs are counted, which is always enough (26 values per face against 19 per job)
+    const long long jobs_n = ((long long)njobs * 144 + 255) / 256 * 32;
     const long long need = scratch_n + G->linetmp_n + jobs_n;
+    static_assert(sizeof(LineJob) <= 19 * sizeof(double), "the job list outgrows its place");
     if (njobs > HYP_NOALLOC_MAX_JOBS || need > HYP_NOALLOC_DOUBLES)
         return fail(HYP_ERR_ARG, "grid too large for hyp_rhs_noalloc: needs " +
                                      std::to_string(need) + " doubles of scratch, the static array holds " +
@@ -1332,7 +1336,7 @@ extern "C" int hyp_rhs_noalloc(const hyp_gas* gas, const hyp_grid* grid, const d
     double* base = nullptr;
     int rc = noalloc_base(&base);
     if (rc) return rc;
-    LineJob* djobs = (LineJob*)(base + scratch_n + G->linetmp_n);
+    LineJob* djobs = (LineJob*)(base + scratch_n);
     auto relocate = [&](const double* p) -> double* {
         if (p >= G->pool && p < G->pool + scratch_n) return base + (p - G->pool);
         return const_cast<double*>(p);

@@ -44,7 +44,9 @@ PEAK_SOURCE = "derived: 152 SMs x 4 warp instructions/clk x 32 x 2.07 GHz"
 CLOSURE_INSTR = (15496, 284.7)
 CLOSURE3_INSTR = (14698, 438.5)
 THERMO_INSTR = (19944, 417.1)
-RHS_INSTR = (50923, 676.7)
+RHS_INSTR = (52789, 714.7)              # of the RK3 step of the shock case at 1024 x 256
+# DRAM bytes (read + write) of one k_closure launch per point, from ncu at 1024 x 256
+CLOSURE_DRAM_BYTES_PER_POINT = 564.4
 
 
 def issue_roofline(instr, units_per_s):
@@ -687,7 +689,8 @@ def ours_arm(args, rank, world, local_rank):
     roof = {"kernel": name, "launches": kcount, "avg_launch_ms": avg_s * 1e3,
             "share_of_step": kms / max(dev_ms, 1e-30)}
     if name == "k_closure":
-        roof.update(issue_roofline(CLOSURE_INSTR, points / avg_s), traffic=None)
+        roof.update(issue_roofline(CLOSURE_INSTR, points / avg_s),
+                    traffic=CLOSURE_DRAM_BYTES_PER_POINT * points)
     else:
         roof.update(bound="alu", achieved=None, peak=ISSUE_PEAK_TINSTR,
                     unit="T thread instructions/s", frac=None, traffic=None,

@@ -18,8 +18,8 @@
  *   thermo_eval inputs and outputs). The library owns the opaque handles and everything inside
  *   them (gas tables, metrics, sponge, reference state, scratch), and frees them in *_free.
  * - Floating point: inputs and results are binary64. With precision HYP_FP64 every step is in
- *   binary64 or on 64-bit integers that carry at least its 53 bits; HYP_MIXED moves the parts
- *   listed at enum hyp_precision to binary32. No call falls back to the CPU: every arithmetic step of
+ *   binary64 or on 64-bit integers (enum hyp_precision says to what precision); HYP_MIXED moves the
+ *   parts listed there to binary32. No call falls back to the CPU: every arithmetic step of
  *   rhs / rk_stage / thermo_eval runs in CUDA kernels.
  * - A grid handle carries scratch memory: calls that use the same grid (rhs, rk_stage) must not
  *   overlap on the device; serialise them on one stream.
@@ -62,9 +62,13 @@ enum hyp_gas_kind {
                             hyp_lte_eval) */
 };
 
-/* HYP_FP64: every step in binary64 or on 64-bit integers that carry at least its 53 bits (the
- * species thermodynamics, kinetics, compact operators, filters and fourth differences, in a common
- * scale; states and lines outside their range take binary64). HYP_MIXED: the transport and
+/* HYP_FP64: every step in binary64 or on 64-bit integers. Species thermodynamics, kinetics and
+ * transport carry at least binary64's 53 bits. Compact operators share a scale over eight rows of a
+ * line: their error is a few units of 2^-60 of the largest value within sixteen rows, of farther
+ * values as far as their influence reaches (and 2^-61 of the line's largest where a line of more
+ * than 2301 rows, or a period that 8 does not divide, is cut). Filters and fourth differences share
+ * one over four outputs, and only where binary64 would be no closer for any of them. States, lines
+ * and outputs outside these ranges take binary64. HYP_MIXED: the transport and
  * diffusion coefficients (Blottner, Eucken, Wilke, Chapman-Enskog; Sec. 2.2.1, Eq. 19) and the
  * forward-rate exponentials (Eq. 13) in binary32, all else as HYP_FP64. */
 enum hyp_precision { HYP_FP64 = 0, HYP_MIXED = 1 };
@@ -341,8 +345,8 @@ int hyp_round_f32(int64_t n, const double* x, float* y, double* back, void* stre
 
 /* The binary64 exponential, quotient, reciprocal and logarithm of the closure's general form
  * (diagnostics; no counterpart in the paper), on 64-bit integers, each within 2 ulp; arguments outside
- * their fast ranges (|a| >= 512 for exp, |b| outside [2^-120, 2^120] for the quotients, a outside
- * [2, 2^1000) for log) go through CUDA's exp, division and log. fn 0: out[i] = exp(a[i]); fn 1:
+ * their fast ranges (|a| >= 512 for exp; for the quotients |b| outside (2^-120, 2^120) or |a| neither
+ * zero nor in [2^-499, 2^500); a outside [2, 2^45) for log) go through CUDA's exp, division and log. fn 0: out[i] = exp(a[i]); fn 1:
  * out[i] = a[i] / b[i]; fn 2: out[i] = 1 / b[i]; fn 3: out[i] = log(a[i]). a, b (the one a
  * function does not read may be null), out: DEVICE arrays of n doubles. */
 int hyp_fp64_fast(int fn, int64_t n, const double* a, const double* b, double* out, void* stream);
@@ -387,7 +391,8 @@ int hyp_lte_eval(const hyp_gas* gas, int64_t n, const double* rho, const double*
  * - Scratch: every per-call scratch field and the launch plan live in one
  *   file-scope device array of 12 MiB (1,572,864 doubles) that every GPU loading the library holds
  *   until exit. Grids needing more (a few thousand cells, e.g. up to 64 x 64) are rejected with
- *   HYP_ERR_ARG and the required size in hyp_last_error(). The grid's own scratch and predictor
+ *   HYP_ERR_ARG and the required size in hyp_last_error(); that size counts the scratch fields, the
+ *   outputs of the largest line phase (room that an earlier layout used) and 144 bytes per line job. The grid's own scratch and predictor
  *   cache are not touched, so hyp_rhs and hyp_rhs_noalloc may be mixed on one grid; its read-only
  *   data (metrics, reference state, sponge, operators) are used. Per-point status bits (Newton,
  *   energy range, rho <= 0) are OR-ed into the grid's status word, read with hyp_grid_status.

@@ -496,13 +496,8 @@ FX int gauss_fixed(const double (&x)[RUN + 8], double (&y)[RUN]) {
     return top == 0u ? 0 : coarse;
 }
 
-// 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a zero or of
-// the same range (positive under the roots): one rounding, within 0.51 ulp.
-FX bool fix_in_range(double b) {
-    const int eb = (int)((bits_of(b) >> 52) & 0x7ff);
-    return eb > 1023 - 500 && eb < 1023 + 500;
-}
-
+// 1 / b, a / b, sqrt(a) and 1 / sqrt(a) for b in [2^-500, 2^500] in magnitude and a of the same range
+// (positive under the roots): one rounding, within 0.51 ulp.
 FX double fix_rcp(double b) {
     const u64 u = bits_of(b);
     const double r = f64_of_xf(xf_rcp(xf_of(b)));

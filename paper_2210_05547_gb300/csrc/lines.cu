@@ -41,13 +41,15 @@
 // Lines with NaN, infinities or magnitudes above 2^899 run the same steps in binary64 (the whole
 // block), so that such values spread as far as a binary64 solve lets them.
 //
-// Measured (GB300): the 50 operators of the face phase at 1024 x 256 take 190 us (the binary64
-// sweeps 234, those in pairs of binary32 words 201), a phase of one or two operators 19-21 us
-// (38-46); the step of the 2048 x 256 shock case 6.69 -> 5.96 ms, of the 256 x 64 boundary layer 0.85 -> 0.57,
-// the 256 x 128 x 64 jet's right-hand side 12.2 -> 10.5. About 280 integer instructions a row
-// warp at 2.2 per clock and SM bound it; eight rows a thread (four blocks of 288 threads per SM)
-// against sixteen (three): 5.96 against 6.5 ms. Converting the results to binary64 on the binary64
-// pipe instead of with integers: 6.4.
+// Measured (GB300): the 50 operators of the face phase at 1024 x 256 take 197 us (189 with one scale
+// per line; the binary64 sweeps 234, those in pairs of binary32 words 201), a phase of one or two
+// operators 19-21 us (38-46). When the solver came in, with one scale per line: the step of the
+// 2048 x 256 shock case 6.69 -> 5.96 ms, of the 256 x 64 boundary layer 0.85 -> 0.57, the
+// 256 x 128 x 64 jet's right-hand side 12.2 -> 10.5; sixteen rows a thread (three blocks of 288 threads
+// per SM instead of four) 6.5 ms, converting the results and adding the corrections on the binary64
+// pipe 7.5. The scales per segment cost 1.5-2% of a step; ten neighbours read one by one instead of
+// the three exchanges cost 10%. About 310 integer instructions per 32 rows at 2.2 per clock and SM
+// bound it.
 #include "fix64.cuh"
 #include "internal.h"
 #include "line_table.h"

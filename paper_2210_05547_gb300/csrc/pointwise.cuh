@@ -260,7 +260,7 @@ __device__ __forceinline__ double d4y(const double* f, int j, int i, int nx, int
 // Raw artificial diffusivities: a factor times |d4x wx + d4y wy|. Fourteen binary64 operations per
 // point and field bound the plain form (110 us at 2048 x 256); here a thread takes four neighbours
 // along x of one field, the fourth differences (weights 1, -4, 6, exact) on integers (fourth_run,
-// fix64.cuh), and two products and a sum remain binary64: 73 us. (The same in three dimensions, forty
+// fix64.cuh), and two products and a sum remain binary64: 80 us. (The same in three dimensions, forty
 // inputs a run, was slower than the plain form there: jet right-hand side 9.77 against 9.61 ms.) Runs
 // at the ends of a row and those that fourth_run does not take have the plain form.
 // Runs of four per field along dir.
@@ -324,9 +324,9 @@ __device__ __forceinline__ void ad_raw_body(bool cneq, const GridView& v,
 // Gaussian filter of the raw diffusivities along x (dir 0) or y (dir 1); indices clamp. Nine
 // binary64 operations a point on a unit that takes 19 cycles each bound the plain form (80 us a
 // pass at 2048 x 256). Here a thread filters four neighbours on 62-bit integers scaled by the
-// largest of their twelve inputs, which share the conversions (gauss_fixed, fix64.cuh): 36 us
+// largest of their twelve inputs, which share the conversions (gauss_fixed, fix64.cuh): 40 us
 // (binary32 in the mixed path before: 37). Outputs that it does not give to binary64's precision
-// take the plain form.
+// take the plain form (without that check 36 us).
 // in(i): input i of the line, indices clamped or wrapped by the caller; put(k, v): output pos + k
 template <class In, class Put>
 __device__ __forceinline__ void gauss_run(int pos, const In& in, const Put& put) {
@@ -558,7 +558,7 @@ __host__ __device__ __forceinline__ long long filter_runs(int nx, int ny, int di
 // The plain form took twelve binary64 operations an entry (96 us a pass at 2048 x 256). A thread
 // takes four entries of a line: away from the ends the tenth difference is formed on integers, whose
 // weights are exact (tenth_run, fix64.cuh: closer than the plain form's eleven roundings); one FMA with
-// the entry itself (binary64) finishes: 43 us. Entries near the ends, and runs that tenth_run does not
+// the entry itself (binary64) finishes: 47 us. Entries near the ends, and runs that tenth_run does not
 // take, have the plain form.
 __device__ __forceinline__ void filter_body(int nx, int ny, const double* __restrict__ in,
                                             double* __restrict__ out, int dir, double sigma,

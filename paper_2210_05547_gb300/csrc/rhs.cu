@@ -838,13 +838,13 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     for (int sp = 0; sp < NSP; ++sp) {
         B.add(OX_ICF, S.Y[sp], NC, S.Yx[sp], NXF, nullptr);
         B.add(OX_ICF, S.G[sp], NC, S.Gx[sp], NXF, nullptr);
-            B.add(OX_ICF, S.h[sp], NC, S.hx[sp], NXF, nullptr);
-            B.add(OX_DCF, S.X[sp], NC, S.dXdx[sp], NXF, G->xi_f);
-            B.add(OY_ICF, S.Y[sp], NC, S.Yy[sp], NYF, nullptr);
+        B.add(OX_ICF, S.h[sp], NC, S.hx[sp], NXF, nullptr);
+        B.add(OX_DCF, S.X[sp], NC, S.dXdx[sp], NXF, G->xi_f);
+        B.add(OY_ICF, S.Y[sp], NC, S.Yy[sp], NYF, nullptr);
         B.add(OY_ICF, S.G[sp], NC, S.Gy[sp], NYF, nullptr);
-            B.add(OY_ICF, S.h[sp], NC, S.hy[sp], NYF, nullptr);
-            B.add(OY_DCF, S.X[sp], NC, S.dXdy[sp], NYF, G->eta_f);
-        }
+        B.add(OY_ICF, S.h[sp], NC, S.hy[sp], NYF, nullptr);
+        B.add(OY_DCF, S.X[sp], NC, S.dXdy[sp], NYF, G->eta_f);
+    }
     B.add(OX_ICF, S.H, NC, S.Hx, NXF, nullptr);
     B.add(OX_ICF, S.K, NC, S.Kx, NXF, nullptr);
     B.add(OX_ICF, S.tau_xx, NC, S.txx_x, NXF, nullptr);
@@ -858,10 +858,10 @@ extern "C" int hyp_state_init(const hyp_gas* gas, const hyp_grid_desc* desc, con
     if (G->view().sm) {
         // face temperature and pressure for the binary coefficients of Eq. (17)
         B.add(OX_ICF, S.T, NC, S.Tx, NXF, nullptr);
-            B.add(OX_ICF, S.p, NC, S.px, NXF, nullptr);
-            B.add(OY_ICF, S.T, NC, S.Ty, NYF, nullptr);
-            B.add(OY_ICF, S.p, NC, S.py, NYF, nullptr);
-        }
+        B.add(OX_ICF, S.p, NC, S.px, NXF, nullptr);
+        B.add(OY_ICF, S.T, NC, S.Ty, NYF, nullptr);
+        B.add(OY_ICF, S.p, NC, S.py, NYF, nullptr);
+    }
     B.begin(PH_FACEB);
     B.add(OY_IFC, S.tau_xy, NCN, S.txy_x, NXF, nullptr);
     B.add(OX_IFC, S.tau_xy, NCN, S.txy_y, NYF, nullptr);

@@ -1,7 +1,8 @@
-// Per-point thermochemistry closure (Sec. 2.2), FP64, shared by the host set-up code and the
-// kernels of this library. All quantities SI unless stated.
+// Per-point thermochemistry closure (Sec. 2.2) in binary64: what the host set-up code runs, what the
+// kernels run for the states and gases that the integer closure (closure_fix.cuh, included below)
+// does not take, and the thermally perfect and equilibrium closures. All quantities SI unless stated.
 //
-// On GB300 the FP64 pipe (two FMAs per clock per SM) bounds this code, so it avoids FP64 work
+// On GB300 the FP64 pipe (two FMAs per clock per SM) bounds this form, so it avoids FP64 work
 // that cannot change a result: electronic levels whose Boltzmann factor is below e^-45 of the
 // ground level are not evaluated (relative contribution under 1e-19), the equilibrium constants
 // come from molar partition functions instead of logarithms of Gibbs energies, reactions sharing
@@ -860,8 +861,9 @@ __host__ __device__ __forceinline__ void lte_at(const GasDev& g, double T, doubl
                                        const double* lnb, bool warm, LteState& q) {
     species_state(g, T, q.s);
     // CUDA's log in the equilibrium closure: its element-potential solve carries the rounding of
-    // ln q into the composition, and the table-driven log moved the stepped LTE parity check from
-    // 0.73 to 1.04 of its bound (a different rounding, not a larger error)
+    // ln q into the composition, and an earlier table-driven binary64 log (not cl_log's integer one,
+    // which has not been tried here) moved the stepped LTE parity check from 0.73 to 1.04 of its
+    // bound (a different rounding, not a larger error)
     const double lnT = log(T);
     double gam[NSP];
     lte_gammas(g, T, lnT, q.s, gam);
